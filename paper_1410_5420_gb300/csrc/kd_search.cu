@@ -2,9 +2,9 @@
 // region search (the "Nearest Neighbors" subsection and the region search
 // of the source-code subsection of the paper).
 //
-// A search index holds the tree's tuples in address order (node a's k
-// coordinates side by side, AoS) and the tuple index of every node, so that
-// a walk reads one contiguous record per visited node.  The tree is the
+// A search index holds the tree's tuples in address order (one plane per
+// coordinate, so that 32 lanes reading 32 consecutive addresses coalesce)
+// and the tuple index of every node.  The tree is the
 // in-order layout the builder writes: the subtree of a node covers a
 // contiguous address range [lo, hi], its node is the median lo + (hi-lo)/2,
 // its children cover [lo, mid-1] and [mid+1, hi], and the split dimension
@@ -12,11 +12,12 @@
 // with x_d <= the node's x_d, the "greater" side only x_d >= (super keys
 // order ties by the next coordinates), which is what both searches prune on.
 //
-//   k_index_gather  node_coords[a] = coords[node_tuple[a]]
-//   k_knn           one thread per query: depth-first walk, near side first,
-//                   the far side only while its splitting-plane distance
-//                   does not exceed the current m-th best; the m best kept
-//                   sorted by (distance, tuple index)
+//   k_index_gather  planes of the tuples' coordinates in address order
+//   k_boxes         bounding boxes over blocks of 32 consecutive addresses
+//   k_knn           one warp per query: walk of the box tree, nearest first,
+//                   the best candidates sorted across the warp
+//   k_knn_walk      one thread per query: depth-first walk of the tree, for
+//                   an index without boxes
 //   k_region        one thread per box: depth-first walk visiting a side
 //                   only if the box reaches it; counts, then (second launch
 //                   after a scan of the counts) the indices
@@ -49,8 +50,12 @@ struct kd_index_s {
     int64_t m = 0;
     int k = 0;
     int dtype = 0;
-    void* node_coords = nullptr;  // m x k, address order, input dtype
+    void* pts = nullptr;  // k planes of m words, address order, input dtype
     int32_t* node_tuple = nullptr;
+    void* boxes = nullptr;  // bounding boxes of every level (nullptr: they did not fit the budget)
+    int64_t box_off[5] = {};  // level l: first word in boxes ...
+    int32_t nbox[5] = {};     // ... and number of boxes
+    int top = 0;
 };
 
 namespace {
@@ -61,6 +66,7 @@ using kd::MAXK;
 
 constexpr int SEARCH_THREADS = 128;
 constexpr int STACK_MAX = 64;  // a tree of at most 2^30 nodes is at most 31 levels deep
+constexpr int REGION_STACK = 32;  // at most one waiting side per level
 
 template <typename T>
 __device__ __forceinline__ double abs_diff(T a, T b);
@@ -83,19 +89,385 @@ __device__ __forceinline__ bool is_nan(T) { return false; }
 template <>
 __device__ __forceinline__ bool is_nan<float>(float v) { return v != v; }
 
+// pts[d * m + a] = coordinate d of the tuple at address a.
 template <typename T>
 __global__ void __launch_bounds__(256) k_index_gather(const T* __restrict__ coords, const int32_t* __restrict__ tuple,
-                                                      int64_t m, int k, int64_t n, T* __restrict__ out,
+                                                      int64_t m, int k, int64_t n, T* __restrict__ pts,
                                                       int* __restrict__ err) {
-    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < m * k; e += (int64_t)gridDim.x * 256) {
-        const int64_t a = e / k;
-        const int d = (int)(e - a * k);
+    for (int64_t a = (int64_t)blockIdx.x * 256 + threadIdx.x; a < m; a += (int64_t)gridDim.x * 256) {
         const int32_t t = tuple[a];
         if (t < 0 || t >= n) {
             atomicOr(err, ERR_INTERNAL);
             continue;
         }
-        out[e] = coords[(int64_t)t * k + d];
+        for (int d = 0; d < k; ++d) pts[d * m + a] = coords[(int64_t)t * k + d];
+    }
+}
+
+// ---------------------------------------------------- nearest neighbours
+// Address order is spatially coherent (it is the tree's in-order), so every
+// 32 consecutive tuples are a compact block.  Over these blocks lies a tree
+// of bounding boxes with 32 children per node: level 0 holds the boxes of
+// the blocks, level l + 1 one box per 32 boxes of level l.  One warp answers
+// one query: at a node every lane tests one child's box, the children are
+// entered nearest first, and in a block every lane computes one distance.
+// The best candidates so far lie sorted across the warp, one per lane
+// (KD_KNN_MAX = 32 of them).
+//
+// What bounded the one-thread-per-query walk this replaces: at two FP64
+// lanes per cycle and SM the double distance of every visited tuple, the
+// neighbour list and the stack in local memory, and, for clustered points, a
+// few queries whose split-plane bounds let them walk most of a dense cluster
+// while the rest of the GPU had finished.  Here candidates are kept by a
+// float distance and only the at most 32 survivors get the double one; the
+// boxes bound by the distance to the tuples themselves.  Eight neighbours of
+// each of 2^22 int64 tuples: 33.9 -> 8.1 ms, now bound by instruction issue
+// (71%, 1570 warp instructions per query); five of 100003 float32 queries
+// among 10^6 clustered tuples: 3.5-28 ms (by the cluster geometry) -> 0.65.
+//
+// Float distances.  a = the float sum of the squared float |p - q| differs
+// from the exact distance t by less than 2^-20 t (roundings of at most
+// (K + 4) 2^-24 in all), unless it underflows (below KNN_TINY) or overflows to +inf.  So
+// with A the kn-th smallest a, every one of the kn nearest tuples has
+// a <= A (1 + 2^-18) = the bound, and a box whose float distance, less
+// 2^-18 of itself, exceeds the bound holds none of them.  All candidates up
+// to the bound are ranked by (double distance, tuple index).  If more than
+// the list's 32 lie below it (ties, or near ties, around kn), the query is
+// answered again with double distances for every candidate (`exact`).
+constexpr int BOX_W = 32;        // tuples per block, children per node
+constexpr int BOX_LEVELS = 5;    // level 4 has at most 32 boxes for 2^30 tuples
+constexpr int KNN_THREADS = 256;
+constexpr float KNN_MARGIN = 3.814697265625e-6f;  // 2^-18
+constexpr float KNN_TINY = 1e-35f;
+constexpr uint32_t KNN_NONE = 0xffffffffu;  // no candidate / child done
+constexpr uint32_t KNN_OPEN = 0xfffffffeu;  // bound while the list holds fewer than kn
+
+template <typename T>
+struct KnnTree {
+    const T* pts;  // k planes of `stride` words, address order
+    int64_t stride;
+    const int32_t* tuple;
+    int32_t m;
+    int k;
+    int top;  // the level whose boxes (at most 32) are tested first
+    // boxes of level l, 32 siblings side by side: word (g * 2k + d) * 32 + c
+    // is the lower bound in dimension d of child c of node g, d + k the upper
+    const T* box[BOX_LEVELS];
+    int32_t nbox[BOX_LEVELS];
+};
+
+// |a - b| as a float, within 2^-23 of it.  (64 bits: from its two halves,
+// three roundings; the conversion instruction for 64-bit integers runs on
+// the FP64 pipe, which it kept 92% busy.)
+__device__ __forceinline__ float diff_f(int32_t a, int32_t b) {
+    return __uint2float_rn(a > b ? (uint32_t)a - (uint32_t)b : (uint32_t)b - (uint32_t)a);
+}
+__device__ __forceinline__ float diff_f(int64_t a, int64_t b) {
+    const uint64_t u = a > b ? (uint64_t)a - (uint64_t)b : (uint64_t)b - (uint64_t)a;
+    return fmaf(__uint2float_rn((uint32_t)(u >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)u));
+}
+__device__ __forceinline__ float diff_f(float a, float b) { return __fsub_rn(a, b); }
+
+// Distance of q from the interval [lo, hi], as diff_f.
+template <typename T>
+__device__ __forceinline__ float gap_f(T q, T lo, T hi) {
+    return q < lo ? diff_f(lo, q) : (q > hi ? diff_f(q, hi) : 0.0f);
+}
+
+__device__ __forceinline__ uint32_t knn_bound(float a) {
+    return __float_as_uint(fmaxf(a * (1.0f + KNN_MARGIN), KNN_TINY));
+}
+
+// The query of one warp and its candidates (lane j: the j-th best).
+template <typename T, int K>  // K: the dimensions, or MAXK: at most that many
+struct KnnQuery {
+    T q[K];
+    int32_t self;    // address excluded, or -1
+    int kn;
+    uint32_t bound;  // float bits: nothing above it can be among the kn nearest
+    uint32_t key;    // candidate: float bits of its distance ...
+    int32_t addr;    // ... and address
+    uint32_t lost;   // smallest float distance that did not fit the list
+    uint64_t dkey;   // exact form: the double distance's bits and the tuple index
+    int32_t tup;
+};
+
+template <typename T, int K>
+__device__ __forceinline__ double exact_dist(const KnnTree<T>& X, const T (&q)[K], int32_t a) {
+    double acc = 0.0;
+#pragma unroll
+    for (int d = 0; d < K; ++d) {
+            if (K == MAXK && d >= X.k) break;
+        const double u = abs_diff<T>(X.pts[d * X.stride + a], q[d]);
+        acc = __dadd_rn(acc, __dmul_rn(u, u));
+    }
+    return acc;
+}
+
+// Ascending by key across the warp (bitonic).
+__device__ __forceinline__ void warp_sort(uint32_t& key, int32_t& val) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+        for (int st = size >> 1; st > 0; st >>= 1) {
+            const uint32_t ok = __shfl_xor_sync(0xffffffffu, key, st);
+            const int32_t ov = __shfl_xor_sync(0xffffffffu, val, st);
+            const bool up = ((lane & size) == 0) == ((lane & st) == 0);  // this lane keeps the smaller
+            if (up ? ok < key : ok > key) {
+                key = ok;
+                val = ov;
+            }
+        }
+    }
+}
+
+template <typename T, int K, bool EXACT>
+__device__ __forceinline__ void knn_block(const KnnTree<T>& X, KnnQuery<T, K>& Q, int32_t blk) {
+    const int lane = threadIdx.x & 31;
+    const int32_t a = blk * BOX_W + lane;
+    const bool ok = a < X.m && a != Q.self;
+    float s = 0.0f;
+    if (ok) {
+#pragma unroll
+        for (int d = 0; d < K; ++d) {
+            if (K == MAXK && d >= X.k) break;
+            const float u = diff_f(X.pts[d * X.stride + a], Q.q[d]);
+            s = fmaf(u, u, s);
+        }
+    }
+    const uint32_t key = __float_as_uint(s);
+    const bool pass = ok && s == s && key <= Q.bound;  // (an infinite coordinate may give no distance: NaN)
+    uint32_t mask = __ballot_sync(0xffffffffu, pass);
+    if (mask == 0) return;
+    if constexpr (EXACT) {
+        uint64_t dk = 0;
+        int32_t tp = 0;
+        if (pass) {
+            dk = (uint64_t)__double_as_longlong(exact_dist<T, K>(X, Q.q, a));
+            tp = X.tuple[a];
+        }
+        for (; mask; mask &= mask - 1) {
+            const int src = __ffs(mask) - 1;
+            const uint64_t d = __shfl_sync(0xffffffffu, dk, src);
+            const int32_t t = __shfl_sync(0xffffffffu, tp, src);
+            const bool before = Q.dkey < d || (Q.dkey == d && Q.tup < t);
+            const int pos = __popc(__ballot_sync(0xffffffffu, before));
+            const uint64_t ud = __shfl_up_sync(0xffffffffu, Q.dkey, 1);
+            const int32_t ut = __shfl_up_sync(0xffffffffu, Q.tup, 1);
+            if (lane > pos) {
+                Q.dkey = ud;
+                Q.tup = ut;
+            } else if (lane == pos) {
+                Q.dkey = d;
+                Q.tup = t;
+            }
+        }
+        const uint64_t A = __shfl_sync(0xffffffffu, Q.dkey, Q.kn - 1);
+        if (A != ~0ull) Q.bound = knn_bound(__double2float_ru(__longlong_as_double((long long)A)));
+    } else {
+        if (__popc(mask) > 8) {
+            // many: sort them, then merge with the list (both ascending)
+            uint32_t nk = pass ? key : KNN_NONE;
+            int32_t na = a;
+            warp_sort(nk, na);
+            nk = __shfl_xor_sync(0xffffffffu, nk, 31);
+            na = __shfl_xor_sync(0xffffffffu, na, 31);
+            const bool take = nk < Q.key;
+            const uint32_t out = take ? Q.key : nk;
+            if (take) {
+                Q.key = nk;
+                Q.addr = na;
+            }
+            Q.lost = min(Q.lost, __reduce_min_sync(0xffffffffu, out));
+#pragma unroll
+            for (int st = 16; st > 0; st >>= 1) {
+                const uint32_t ok2 = __shfl_xor_sync(0xffffffffu, Q.key, st);
+                const int32_t oa = __shfl_xor_sync(0xffffffffu, Q.addr, st);
+                if ((lane & st) == 0 ? ok2 < Q.key : ok2 > Q.key) {
+                    Q.key = ok2;
+                    Q.addr = oa;
+                }
+            }
+        } else {
+            for (; mask; mask &= mask - 1) {
+                const int src = __ffs(mask) - 1;
+                const uint32_t d = __shfl_sync(0xffffffffu, key, src);
+                const int pos = __popc(__ballot_sync(0xffffffffu, Q.key <= d));
+                const uint32_t uk = __shfl_up_sync(0xffffffffu, Q.key, 1);
+                const int32_t ua = __shfl_up_sync(0xffffffffu, Q.addr, 1);
+                Q.lost = min(Q.lost, pos == 32 ? d : __shfl_sync(0xffffffffu, Q.key, 31));
+                if (lane > pos) {
+                    Q.key = uk;
+                    Q.addr = ua;
+                } else if (lane == pos) {
+                    Q.key = d;
+                    Q.addr = blk * BOX_W + src;
+                }
+            }
+        }
+        const uint32_t A = __shfl_sync(0xffffffffu, Q.key, Q.kn - 1);
+        if (A != KNN_NONE) Q.bound = knn_bound(__uint_as_float(A));
+    }
+}
+
+// The children (boxes of level L) of node `node`, nearest first.
+template <typename T, int K, bool EXACT, int L>
+__device__ __forceinline__ void knn_node(const KnnTree<T>& X, KnnQuery<T, K>& Q, int32_t node) {
+    if constexpr (L > 0) {
+        if (L > X.top) {
+            knn_node<T, K, EXACT, L - 1>(X, Q, 0);
+            return;
+        }
+    }
+    const int lane = threadIdx.x & 31;
+    uint32_t key = KNN_NONE;
+    if (node * BOX_W + lane < X.nbox[L]) {
+        const T* b = X.box[L] + (int64_t)node * (2 * (K == MAXK ? X.k : K) * BOX_W) + lane;
+        float s = 0.0f;
+#pragma unroll
+        for (int d = 0; d < K; ++d) {
+            if (K == MAXK && d >= X.k) break;
+            const float u = gap_f<T>(Q.q[d], b[d * BOX_W], b[((K == MAXK ? X.k : K) + d) * BOX_W]);
+            s = fmaf(u, u, s);
+        }
+        key = __float_as_uint(s * (1.0f - KNN_MARGIN));
+    }
+    for (int i = 0; i < BOX_W; ++i) {
+        const uint32_t best = __reduce_min_sync(0xffffffffu, key);
+        if (best > Q.bound) break;
+        const int c = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+        if (lane == c) key = KNN_NONE;
+        if constexpr (L > 0) knn_node<T, K, EXACT, L - 1>(X, Q, node * BOX_W + c);
+        else knn_block<T, K, EXACT>(X, Q, node * BOX_W + c);
+    }
+}
+
+// The candidates of this lane's group of `width` lanes (address c of query
+// qc, or c = -1) by (double distance, tuple index): the first kn to row qi.
+template <typename T, int K>
+__device__ __forceinline__ void knn_emit(const KnnTree<T>& X, const T* __restrict__ queries, int64_t qi, int32_t c,
+                                         int width, int kn, int32_t* __restrict__ idx_out,
+                                         double* __restrict__ d_out) {
+    const int lane = threadIdx.x & 31, first = lane & ~(width - 1);
+    uint64_t dk = ~0ull;
+    int32_t tp = INT32_MAX;
+    if (c >= 0) {
+        T q[K];
+#pragma unroll
+        for (int d = 0; d < K; ++d) {
+            if (K == MAXK && d >= X.k) break;
+            q[d] = queries ? queries[qi * (K == MAXK ? X.k : K) + d] : X.pts[d * X.stride + qi];
+        }
+        dk = (uint64_t)__double_as_longlong(exact_dist<T, K>(X, q, c));
+        tp = X.tuple[c];
+    }
+    int rank = 0;
+    for (int j = 0; j < width; ++j) {
+        const uint64_t d = __shfl_sync(0xffffffffu, dk, first + j);
+        const int32_t t = __shfl_sync(0xffffffffu, tp, first + j);
+        rank += (d < dk || (d == dk && t < tp)) ? 1 : 0;
+    }
+    const uint32_t group = width == 32 ? 0xffffffffu : ((1u << width) - 1u) << first;
+    const int cnt = __popc(__ballot_sync(0xffffffffu, c >= 0) & group);
+    if (c >= 0 ? rank < kn : (cnt > 0 && lane - first >= cnt && lane - first < kn)) {
+        const int j = c >= 0 ? rank : lane - first;  // (rows past the last candidate: no tuple)
+        idx_out[qi * kn + j] = c >= 0 ? tp : -1;
+        if (d_out) d_out[qi * kn + j] = __longlong_as_double(c >= 0 ? (long long)dk : 0x7ff0000000000000ll);
+    }
+}
+
+// queries == nullptr: every address is a query (row = its address) and its
+// own tuple is not a candidate.  A warp answers 32 / width queries in turn
+// (width: a power of two, at least kn) and then computes the double
+// distances of all their candidates at once, one per lane: with kn = 8 and
+// one query at a time, 24 of the 32 lanes of every FP64 instruction idled
+// while that pipe was 89% busy.
+template <typename T, int K>
+__global__ void __launch_bounds__(KNN_THREADS) k_knn(const __grid_constant__ KnnTree<T> X,
+                                                     const T* __restrict__ queries, int64_t nq, int kn, int width,
+                                                     int32_t* __restrict__ idx_out, double* __restrict__ d_out,
+                                                     int* __restrict__ err) {
+    const int lane = threadIdx.x & 31;
+    const int per = 32 / width;
+    for (int64_t q0 = ((int64_t)blockIdx.x * (KNN_THREADS / 32) + (threadIdx.x >> 5)) * per; q0 < nq;
+         q0 += (int64_t)gridDim.x * (KNN_THREADS / 32) * per) {
+        int32_t cand = -1;  // lane r * width + j: candidate j of query q0 + r
+        for (int r = 0; r < per && q0 + r < nq; ++r) {
+            const int64_t qi = q0 + r;
+            KnnQuery<T, K> Q;
+            bool nan = false;
+#pragma unroll
+            for (int d = 0; d < K; ++d) {
+                if (K == MAXK && d >= X.k) break;
+                Q.q[d] = queries ? queries[qi * (K == MAXK ? X.k : K) + d] : X.pts[d * X.stride + qi];
+                nan |= is_nan(Q.q[d]);
+            }
+            if (nan) {
+                if (lane == 0) atomicOr(err, ERR_NAN);
+                continue;
+            }
+            Q.self = queries ? -1 : (int32_t)qi;
+            Q.kn = kn;
+            Q.bound = KNN_OPEN;
+            Q.key = Q.lost = KNN_NONE;
+            Q.addr = -1;
+            Q.dkey = ~0ull;
+            Q.tup = INT32_MAX;
+            if (X.m > 0) knn_node<T, K, false, BOX_LEVELS - 1>(X, Q, 0);
+            const int32_t c = Q.key != KNN_NONE && Q.key <= Q.bound ? Q.addr : -1;  // the first lanes
+            const int cnt = __popc(__ballot_sync(0xffffffffu, c >= 0));
+            if (Q.lost <= Q.bound || cnt == 0) {
+                // more candidates up to the bound than the list holds, or none at all
+                Q.bound = KNN_OPEN;
+                if (cnt > 0) knn_node<T, K, true, BOX_LEVELS - 1>(X, Q, 0);
+                if (lane < kn) {
+                    const bool none = Q.dkey == ~0ull;
+                    idx_out[qi * kn + lane] = none ? -1 : Q.tup;
+                    if (d_out)
+                        d_out[qi * kn + lane] = __longlong_as_double(none ? 0x7ff0000000000000ll : (long long)Q.dkey);
+                }
+            } else if (cnt > width) {
+                knn_emit<T, K>(X, queries, qi, c, 32, kn, idx_out, d_out);
+            } else {
+                const int32_t v = __shfl_sync(0xffffffffu, c, lane & (width - 1));
+                if (lane / width == r) cand = v;
+            }
+        }
+        if (__any_sync(0xffffffffu, cand >= 0))
+            knn_emit<T, K>(X, queries, q0 + lane / width, cand, width, kn, idx_out, d_out);
+    }
+}
+
+// Boxes of level 0 (src: the point planes, n tuples) or of level l + 1
+// (src: the boxes of level l, n of them): one warp per box.
+template <typename T>
+__global__ void __launch_bounds__(256) k_boxes(const T* __restrict__ src, int64_t stride, int from_points, int64_t n,
+                                               int k, int64_t nbox, T* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); b < nbox; b += (int64_t)gridDim.x * 8) {
+        const int64_t e = b * BOX_W + lane < n ? b * BOX_W + lane : n - 1;  // (a lane past the end repeats the last)
+        for (int d = 0; d < k; ++d) {
+            T lo, hi;
+            if (from_points) {
+                lo = hi = src[d * stride + e];
+            } else {
+                const T* p = src + (e / BOX_W) * (2 * k * BOX_W) + e % BOX_W;
+                lo = p[d * BOX_W];
+                hi = p[(k + d) * BOX_W];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const T l2 = __shfl_xor_sync(0xffffffffu, lo, o), h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+                lo = l2 < lo ? l2 : lo;
+                hi = h2 > hi ? h2 : hi;
+            }
+            if (lane == 0) {
+                T* q = out + (b / BOX_W) * (2 * k * BOX_W) + b % BOX_W;
+                q[d * BOX_W] = lo;
+                q[(k + d) * BOX_W] = hi;
+            }
+        }
     }
 }
 
@@ -117,22 +489,21 @@ __device__ __forceinline__ void knn_insert(double* bd, int32_t* bi, int kn, doub
     bi[j] = t;
 }
 
-// queries == nullptr: every node is a query (row = its address) and its own
-// tuple is not a candidate.
+// An index without boxes: one thread per query walks the tree depth first,
+// near side first.  queries as for k_knn.
 template <typename T>
-__global__ void __launch_bounds__(SEARCH_THREADS) k_knn(const T* __restrict__ nodes, const int32_t* __restrict__ tuple,
-                                                        int32_t m, int k, const T* __restrict__ queries, int64_t nq,
+__global__ void __launch_bounds__(SEARCH_THREADS) k_knn_walk(const T* __restrict__ pts, int64_t stride,
+                                                             const int32_t* __restrict__ tuple, int32_t m, int k, const T* __restrict__ queries, int64_t nq,
                                                         int kn, int32_t* __restrict__ idx_out,
                                                         double* __restrict__ d_out, int* __restrict__ err) {
     const int64_t qi = (int64_t)blockIdx.x * SEARCH_THREADS + threadIdx.x;
     if (qi >= nq) return;
     const int32_t self = queries ? -1 : tuple[qi];
-    if (!queries) queries = nodes;
     T q[MAXK];
     bool nan = false;
 #pragma unroll
     for (int d = 0; d < MAXK; ++d) {
-        q[d] = d < k ? queries[qi * k + d] : (T)0;
+        q[d] = d < k ? (queries ? queries[qi * k + d] : pts[d * stride + qi]) : (T)0;
         nan |= d < k && is_nan(q[d]);
     }
     if (nan) {
@@ -152,22 +523,20 @@ __global__ void __launch_bounds__(SEARCH_THREADS) k_knn(const T* __restrict__ no
         const KnnEntry e = st[--sp];
         if (e.bound > bd[kn - 1]) continue;  // nothing in this subtree can enter the list
         const int32_t mid = e.lo + ((e.hi - e.lo) >> 1);
-        const T* p = nodes + (int64_t)mid * k;
+        const T* p = pts + mid;
         double acc = 0.0;
         for (int d = 0; d < k; ++d) {
-            const double u = abs_diff<T>(p[d], q[d]);
+            const double u = abs_diff<T>(p[d * stride], q[d]);
             acc = __dadd_rn(acc, __dmul_rn(u, u));
         }
         const int32_t tm = tuple[mid];
         if (tm != self) knn_insert(bd, bi, kn, acc, tm);
         const int dim = e.depth % k;
-        T qd = q[0], pd = p[0];
+        T qd = q[0];
+        const T pd = p[dim * stride];
 #pragma unroll
         for (int d = 1; d < MAXK; ++d)
-            if (d == dim) {
-                qd = q[d];
-                pd = p[dim];
-            }
+            if (d == dim) qd = q[d];
         const double u = abs_diff<T>(pd, qd);
         const double plane = __dmul_rn(u, u);
         const bool less = qd < pd;  // the query lies on the "less" side
@@ -194,89 +563,88 @@ __global__ void __launch_bounds__(SEARCH_THREADS) k_knn(const T* __restrict__ no
 }
 
 // Region search over box qi: count (out == nullptr) or write the indices
-// of the tuples inside it at out[offs[qi] ...].
-template <typename T>
-__global__ void __launch_bounds__(SEARCH_THREADS) k_region(const T* __restrict__ nodes,
+// of the tuples inside it at out[offs[qi] ...].  The walk takes a node, its
+// less side, then its greater side; the side entered at once stays in
+// registers, the other waits on the stack as one word (lo, hi, dimension);
+// one kernel per dimension count keeps the box and the node in registers.
+// 2^20 boxes of about 3 of 2^22 int64 tuples each: 0.95 -> 0.62 ms a walk.
+template <typename T, int K>
+__global__ void __launch_bounds__(SEARCH_THREADS) k_region(const T* __restrict__ pts, int64_t stride,
                                                            const int32_t* __restrict__ tuple, int32_t m, int k,
                                                            const T* __restrict__ lo, const T* __restrict__ hi,
-                                                           int64_t nq, int64_t* __restrict__ counts,
+                                                           int64_t nq, uint32_t* __restrict__ counts,
                                                            const int64_t* __restrict__ offs, int32_t* __restrict__ out,
                                                            int* __restrict__ err) {
-    const int64_t qi = (int64_t)blockIdx.x * SEARCH_THREADS + threadIdx.x;
-    if (qi >= nq) return;
-    T a[MAXK], b[MAXK];
-    bool nan = false;
+    for (int64_t qi = (int64_t)blockIdx.x * SEARCH_THREADS + threadIdx.x; qi < nq;
+         qi += (int64_t)gridDim.x * SEARCH_THREADS) {
+        const int kk = K == MAXK ? k : K;
+        T a[K], b[K];
+        bool nan = false;
 #pragma unroll
-    for (int d = 0; d < MAXK; ++d) {
-        a[d] = d < k ? lo[qi * k + d] : (T)0;
-        b[d] = d < k ? hi[qi * k + d] : (T)0;
-        nan |= d < k && (is_nan(a[d]) || is_nan(b[d]));
-    }
-    if (nan) {
-        atomicOr(err, ERR_NAN);
-        if (!out) counts[qi] = 0;
-        return;
-    }
-    int64_t o = out ? offs[qi] : 0;
-    const int64_t o_end = out ? offs[qi + 1] : 0;
-    int64_t c = 0;
-    int32_t st_lo[STACK_MAX], st_hi[STACK_MAX], st_dp[STACK_MAX];
-    int sp = 0;
-    if (m > 0) {
-        st_lo[0] = 0;
-        st_hi[0] = m - 1;
-        st_dp[0] = 0;
-        sp = 1;
-    }
-    while (sp > 0) {
-        --sp;
-        const int32_t l = st_lo[sp], h = st_hi[sp], depth = st_dp[sp];
-        const int32_t mid = l + ((h - l) >> 1);
-        const T* p = nodes + (int64_t)mid * k;
-        bool in = true;
-        for (int d = 0; d < k; ++d) {
-            T ad = a[0], bdv = b[0];
+        for (int d = 0; d < K; ++d) {
+            if (d >= kk) break;
+            a[d] = lo[qi * kk + d];
+            b[d] = hi[qi * kk + d];
+            nan |= is_nan(a[d]) || is_nan(b[d]);
+        }
+        if (nan) {
+            atomicOr(err, ERR_NAN);
+            if (!out) counts[qi] = 0;
+            continue;
+        }
+        int64_t o = out ? offs[qi] : 0;
+        const int64_t o_end = out ? offs[qi + 1] : 0;
+        uint32_t c = 0;
+        uint64_t st[REGION_STACK];  // lo | hi << 30 | dimension << 60
+        int sp = 0;
+        int32_t l = 0, h = m - 1, dim = 0;
+        bool more = m > 0;
+        while (more) {
+            const int32_t mid = l + ((h - l) >> 1);
+            T p[K];
 #pragma unroll
-            for (int x = 1; x < MAXK; ++x)
-                if (x == d) {
-                    ad = a[x];
-                    bdv = b[x];
+            for (int d = 0; d < K; ++d)
+                if (d < kk) p[d] = pts[d * stride + mid];
+            bool in = true, go_less = l < mid, go_greater = mid < h;
+#pragma unroll
+            for (int d = 0; d < K; ++d) {
+                if (d >= kk) break;
+                const bool ge = a[d] <= p[d], le = p[d] <= b[d];
+                in = in && ge && le;
+                if (d == dim) {
+                    go_less = go_less && ge;        // the less side holds x_dim <= p_dim
+                    go_greater = go_greater && le;  // the greater side holds x_dim >= p_dim
                 }
-            in = in && ad <= p[d] && p[d] <= bdv;
-        }
-        if (in) {
-            if (out) {
-                if (o < o_end) out[o++] = tuple[mid]; else atomicOr(err, ERR_INTERNAL);
             }
-            ++c;
-        }
-        const int dim = depth % k;
-        T ad = a[0], bdv = b[0];
-#pragma unroll
-        for (int x = 1; x < MAXK; ++x)
-            if (x == dim) {
-                ad = a[x];
-                bdv = b[x];
+            if (in) {
+                if (out) {
+                    if (o < o_end) out[o++] = tuple[mid]; else atomicOr(err, ERR_INTERNAL);
+                }
+                ++c;
             }
-        const T pd = p[dim];
-        if (sp + 2 > STACK_MAX) {
-            atomicOr(err, ERR_INTERNAL);
-            break;
+            dim = dim + 1 == kk ? 0 : dim + 1;
+            if (go_less) {
+                if (go_greater) {
+                    if (sp == REGION_STACK) {
+                        atomicOr(err, ERR_INTERNAL);
+                        break;
+                    }
+                    st[sp++] = (uint64_t)(uint32_t)(mid + 1) | ((uint64_t)(uint32_t)h << 30) | ((uint64_t)dim << 60);
+                }
+                h = mid - 1;
+            } else if (go_greater) {
+                l = mid + 1;
+            } else if (sp > 0) {
+                const uint64_t e = st[--sp];
+                l = (int32_t)(e & 0x3fffffffu);
+                h = (int32_t)((e >> 30) & 0x3fffffffu);
+                dim = (int)(e >> 60);
+            } else {
+                more = false;
+            }
         }
-        if (mid + 1 <= h && pd <= bdv) {  // the greater side holds x_dim >= pd
-            st_lo[sp] = mid + 1;
-            st_hi[sp] = h;
-            st_dp[sp] = depth + 1;
-            ++sp;
-        }
-        if (l <= mid - 1 && ad <= pd) {  // the less side holds x_dim <= pd
-            st_lo[sp] = l;
-            st_hi[sp] = mid - 1;
-            st_dp[sp] = depth + 1;
-            ++sp;
-        }
+        if (!out) counts[qi] = c;
     }
-    if (!out) counts[qi] = c;
 }
 
 // Reverse nearest neighbours: inv[tuple] = address, then per target
@@ -315,48 +683,96 @@ __global__ void __launch_bounds__(256) k_rev_fill(const int32_t* __restrict__ nn
     }
 }
 
-// offs[i] = sum of counts[0..i), offs[n] = total; one block.
-__global__ void __launch_bounds__(1024) k_offsets(const int64_t* __restrict__ counts, int64_t n,
-                                                 int64_t* __restrict__ offs) {
+// offs[i] = sum of counts[0..i), offs[n] = total, in three launches: the
+// sum of every chunk of OFF_CHUNK counts, their exclusive scan by one block,
+// and every chunk's own scan from its base.  (One block scanning all counts
+// 1024 at a time took 1.08 ms for 2^20 of them: a serial chain of barriers
+// on one SM.)
+constexpr int OFF_VPT = 8;
+constexpr int OFF_CHUNK = 256 * OFF_VPT;
+
+// Inclusive scan of one value per lane.
+__device__ __forceinline__ int64_t warp_incl(int64_t x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+template <typename C>
+__global__ void __launch_bounds__(256) k_offsets_sums(const C* __restrict__ counts, int64_t n,
+                                                      int64_t* __restrict__ sums) {
+    __shared__ int64_t s_w[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t v = 0;
+#pragma unroll
+    for (int j = 0; j < OFF_VPT; ++j) {
+        const int64_t i = (int64_t)blockIdx.x * OFF_CHUNK + j * 256 + threadIdx.x;
+        v += i < n ? (int64_t)counts[i] : 0;
+    }
+    v = warp_incl(v);
+    if (lane == 31) s_w[warp] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int64_t t = 0;
+        for (int w = 0; w < 8; ++w) t += s_w[w];
+        sums[blockIdx.x] = t;
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_offsets_bases(int64_t nchunks, int64_t* __restrict__ sums,
+                                                        int64_t* __restrict__ total) {
     __shared__ int64_t s_w[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int64_t carry = 0;
-    for (int64_t base = 0; base < n; base += 1024) {
+    for (int64_t base = 0; base < nchunks; base += 1024) {
         const int64_t i = base + tid;
-        const int64_t v = i < n ? counts[i] : 0;
-        int64_t x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
+        const int64_t v = i < nchunks ? sums[i] : 0;
+        const int64_t x = warp_incl(v);
         if (lane == 31) s_w[warp] = x;
         __syncthreads();
-        if (warp == 0) {
-            int64_t w = s_w[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int64_t y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            s_w[lane] = w;
-        }
+        if (warp == 0) s_w[lane] = warp_incl(s_w[lane]);
         __syncthreads();
-        const int64_t excl = carry + (warp ? s_w[warp - 1] : 0) + x - v;
-        if (i < n) offs[i] = excl;
+        if (i < nchunks) sums[i] = carry + (warp ? s_w[warp - 1] : 0) + x - v;
         carry += s_w[31];
         __syncthreads();
     }
-    if (tid == 0) offs[n] = carry;
+    if (tid == 0) *total = carry;
 }
 
-bool device_ptr(const void* p) {
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+template <typename C>
+__global__ void __launch_bounds__(256) k_offsets_write(const C* __restrict__ counts, int64_t n,
+                                                       const int64_t* __restrict__ sums, int64_t* __restrict__ offs) {
+    __shared__ int64_t s_w[OFF_VPT][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * OFF_CHUNK;
+    int64_t v[OFF_VPT], x[OFF_VPT];
+#pragma unroll
+    for (int j = 0; j < OFF_VPT; ++j) {
+        const int64_t i = base + j * 256 + threadIdx.x;
+        v[j] = i < n ? (int64_t)counts[i] : 0;
     }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+#pragma unroll
+    for (int j = 0; j < OFF_VPT; ++j) {
+        x[j] = warp_incl(v[j]);
+        if (lane == 31) s_w[j][warp] = x[j];
+    }
+    __syncthreads();
+    int64_t run = sums[blockIdx.x];
+#pragma unroll
+    for (int j = 0; j < OFF_VPT; ++j) {
+        int64_t before = run;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) before += s_w[j][w];
+            run += s_w[j][w];
+        }
+        const int64_t i = base + j * 256 + threadIdx.x;
+        if (i < n) offs[i] = before + x[j] - v[j];
+    }
 }
 
 size_t dtype_size(int dtype) { return dtype == KD_I64 ? 8 : 4; }
@@ -409,6 +825,115 @@ kd_status read_err(kd_ctx* ctx, int* d_err, cudaStream_t s) {
 
 int grid_of(int64_t n, int per) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 1 << 20)); }
 
+// Levels of boxes over m tuples: words per level (whole groups of 32
+// siblings) and in all; returns the total.
+int64_t box_layout(kd_index_s* ix) {
+    int64_t words = 0, n = ix->m;
+    for (int l = 0; l < BOX_LEVELS; ++l) {
+        n = (n + BOX_W - 1) / BOX_W;
+        ix->nbox[l] = (int32_t)n;
+        ix->box_off[l] = words;
+        words += (n + BOX_W - 1) / BOX_W * (2 * ix->k * BOX_W);
+        ix->top = l;
+        if (n <= BOX_W) break;
+    }
+    return words;
+}
+
+// The planes and boxes of a new index from coords and the tree.
+template <typename T>
+void index_fill(kd_ctx* ctx, kd_index_s* ix, const void* coords, int64_t n, int* err, cudaStream_t s) {
+    k_index_gather<T><<<grid_of(ix->m, 256), 256, 0, s>>>((const T*)coords, ix->node_tuple, ix->m, ix->k, n,
+                                                          (T*)ix->pts, err);
+    kd::ctx_add_launches(ctx, 1);
+    if (!ix->boxes) return;
+    for (int l = 0; l <= ix->top; ++l) {
+        const T* src = l ? (const T*)ix->boxes + ix->box_off[l - 1] : (const T*)ix->pts;
+        k_boxes<T><<<grid_of(ix->nbox[l], 8), 256, 0, s>>>(src, ix->m, l == 0, l ? ix->nbox[l - 1] : ix->m, ix->k,
+                                                           ix->nbox[l], (T*)ix->boxes + ix->box_off[l]);
+        kd::ctx_add_launches(ctx, 1);
+    }
+}
+
+template <typename T, int K>
+void knn_as(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err,
+            cudaStream_t s) {
+    KnnTree<T> X{};
+    X.pts = (const T*)ix->pts;
+    X.stride = ix->m;
+    X.tuple = ix->node_tuple;
+    X.m = (int32_t)ix->m;
+    X.k = ix->k;
+    X.top = ix->top;
+    for (int l = 0; l <= ix->top; ++l) {
+        X.box[l] = (const T*)ix->boxes + ix->box_off[l];
+        X.nbox[l] = ix->nbox[l];
+    }
+    // several queries per warp only where there are warps enough without it (152 SMs x 32 warps)
+    int width = 32;
+    while (width / 2 >= kn && width > 4 && nq * width / 64 >= 152 * 32) width /= 2;
+    const int per = KNN_THREADS / width;  // queries of a block at a time
+    k_knn<T, K><<<grid_of(nq, per), KNN_THREADS, 0, s>>>(X, (const T*)queries, nq, kn, width, di, dd, err);
+}
+
+template <typename T, int K>
+void region_as(kd_index_s* ix, const void* lo, const void* hi, int64_t nq, uint32_t* counts, const int64_t* offs,
+               int32_t* out, int* err, cudaStream_t s) {
+    k_region<T, K><<<grid_of(nq, SEARCH_THREADS), SEARCH_THREADS, 0, s>>>(
+        (const T*)ix->pts, ix->m, ix->node_tuple, (int32_t)ix->m, ix->k, (const T*)lo, (const T*)hi, nq, counts, offs, out,
+        err);
+}
+
+// Calls NAME<T, K>(...): K the index's dimension count, MAXK for those
+// without kernels of their own.
+#define KD_SEARCH_K(NAME, T, ...)                                 \
+    switch (ix->k) {                                              \
+        case 2: NAME<T, 2>(__VA_ARGS__); break;                   \
+        case 3: NAME<T, 3>(__VA_ARGS__); break;                   \
+        case 4: NAME<T, 4>(__VA_ARGS__); break;                   \
+        default: NAME<T, MAXK>(__VA_ARGS__); break;               \
+    }
+
+template <typename T>
+void knn_of(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err,
+            cudaStream_t s) {
+    if (ix->m > 0 && !ix->boxes)
+        k_knn_walk<T><<<grid_of(nq, SEARCH_THREADS), SEARCH_THREADS, 0, s>>>(
+            (const T*)ix->pts, ix->m, ix->node_tuple, (int32_t)ix->m, ix->k, (const T*)queries, nq, kn, di, dd, err);
+    else
+        KD_SEARCH_K(knn_as, T, ix, queries, nq, kn, di, dd, err, s)
+}
+
+// The kn nearest tuples of nq queries (nullptr: of every address).
+void launch_knn(kd_ctx* ctx, kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd,
+                int* err, cudaStream_t s) {
+    if (ix->dtype == KD_I32) knn_of<int32_t>(ix, queries, nq, kn, di, dd, err, s);
+    else if (ix->dtype == KD_I64) knn_of<int64_t>(ix, queries, nq, kn, di, dd, err, s);
+    else knn_of<float>(ix, queries, nq, kn, di, dd, err, s);
+    kd::ctx_add_launches(ctx, 1);
+}
+
+void launch_region(kd_ctx* ctx, kd_index_s* ix, const void* lo, const void* hi, int64_t nq, uint32_t* counts,
+                   const int64_t* offs, int32_t* out, int* err, cudaStream_t s) {
+    if (nq == 0) return;
+    if (ix->dtype == KD_I32) KD_SEARCH_K(region_as, int32_t, ix, lo, hi, nq, counts, offs, out, err, s)
+    else if (ix->dtype == KD_I64) KD_SEARCH_K(region_as, int64_t, ix, lo, hi, nq, counts, offs, out, err, s)
+    else KD_SEARCH_K(region_as, float, ix, lo, hi, nq, counts, offs, out, err, s)
+    kd::ctx_add_launches(ctx, 1);
+}
+
+int64_t offsets_chunks(int64_t n) { return std::max<int64_t>(1, (n + OFF_CHUNK - 1) / OFF_CHUNK); }
+
+// offs[0..n] from counts[0..n); sums: offsets_chunks(n) words.
+template <typename C>
+void launch_offsets(kd_ctx* ctx, const C* counts, int64_t n, int64_t* sums, int64_t* offs, cudaStream_t s) {
+    const int64_t chunks = offsets_chunks(n);
+    k_offsets_sums<C><<<(unsigned)chunks, 256, 0, s>>>(counts, n, sums);
+    k_offsets_bases<<<1, 1024, 0, s>>>(chunks, sums, offs + n);
+    k_offsets_write<C><<<(unsigned)chunks, 256, 0, s>>>(counts, n, sums, offs);
+    kd::ctx_add_launches(ctx, 3);
+}
+
 }  // namespace
 
 extern "C" {
@@ -440,7 +965,7 @@ kd_status kd_index_create(kd_ctx* ctx, const kd_cloud* cloud, const kd_tree* tre
     const void* tuple = nullptr;
     kd_status st = to_device(ctx, S, cloud->coords, (size_t)cloud->n * cloud->k * ts, cloud->on_device, &coords, s);
     if (st == KD_OK) st = to_device(ctx, S, tree->node_tuple, (size_t)ix->m * 4, tree->on_device, &tuple, s);
-    if (st == KD_OK) st = kd::ctx_alloc(ctx, &ix->node_coords, (size_t)ix->m * ix->k * ts);
+    if (st == KD_OK) st = kd::ctx_alloc(ctx, &ix->pts, (size_t)ix->m * ix->k * ts);
     if (st == KD_OK) st = kd::ctx_alloc(ctx, (void**)&ix->node_tuple, (size_t)ix->m * 4);
     int* d_err = nullptr;
     if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
@@ -448,19 +973,13 @@ kd_status kd_index_create(kd_ctx* ctx, const kd_cloud* cloud, const kd_tree* tre
         kd_index_destroy(ctx, ix.release());
         return st;
     }
+    // the boxes (a sixteenth of the planes) are left out where they do not fit the budget
+    if (kd::ctx_alloc(ctx, &ix->boxes, (size_t)box_layout(ix.get()) * ts) != KD_OK) sfail(ctx, KD_OK, "");
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
     cudaMemcpyAsync(ix->node_tuple, tuple, (size_t)ix->m * 4, cudaMemcpyDeviceToDevice, s);
-    const int g = grid_of(ix->m * ix->k, 256);
-    if (ix->dtype == KD_I32)
-        k_index_gather<int32_t><<<g, 256, 0, s>>>((const int32_t*)coords, (const int32_t*)tuple, ix->m, ix->k,
-                                                  cloud->n, (int32_t*)ix->node_coords, d_err);
-    else if (ix->dtype == KD_I64)
-        k_index_gather<int64_t><<<g, 256, 0, s>>>((const int64_t*)coords, (const int32_t*)tuple, ix->m, ix->k,
-                                                  cloud->n, (int64_t*)ix->node_coords, d_err);
-    else
-        k_index_gather<float><<<g, 256, 0, s>>>((const float*)coords, (const int32_t*)tuple, ix->m, ix->k,
-                                                cloud->n, (float*)ix->node_coords, d_err);
-    kd::ctx_add_launches(ctx, 1);
+    if (ix->dtype == KD_I32) index_fill<int32_t>(ctx, ix.get(), coords, cloud->n, d_err, s);
+    else if (ix->dtype == KD_I64) index_fill<int64_t>(ctx, ix.get(), coords, cloud->n, d_err, s);
+    else index_fill<float>(ctx, ix.get(), coords, cloud->n, d_err, s);
     st = read_err(ctx, d_err, s);
     if (st != KD_OK) {
         kd_index_destroy(ctx, ix.release());
@@ -474,7 +993,8 @@ kd_status kd_index_destroy(kd_ctx* ctx, kd_index ix) {
     if (!ctx || !ix) return KD_EINVAL;
     std::lock_guard<std::recursive_mutex> lk(kd::ctx_mutex(ctx));
     cudaSetDevice(kd::ctx_device(ctx));
-    if (ix->node_coords) kd::ctx_free(ctx, ix->node_coords);
+    if (ix->pts) kd::ctx_free(ctx, ix->pts);
+    if (ix->boxes) kd::ctx_free(ctx, ix->boxes);
     if (ix->node_tuple) kd::ctx_free(ctx, ix->node_tuple);
     delete ix;
     return KD_OK;
@@ -503,41 +1023,12 @@ kd_status kd_knn(kd_ctx* ctx, kd_index ix, const void* queries, int64_t nq, int 
     if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
     if (st != KD_OK) return st;
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
-    const int g = grid_of(nq, SEARCH_THREADS);
-    const int32_t m = (int32_t)ix->m;
-    if (ix->dtype == KD_I32)
-        k_knn<int32_t><<<g, SEARCH_THREADS, 0, s>>>((const int32_t*)ix->node_coords, ix->node_tuple, m, ix->k,
-                                                    (const int32_t*)q, nq, kn, di, dd, d_err);
-    else if (ix->dtype == KD_I64)
-        k_knn<int64_t><<<g, SEARCH_THREADS, 0, s>>>((const int64_t*)ix->node_coords, ix->node_tuple, m, ix->k,
-                                                    (const int64_t*)q, nq, kn, di, dd, d_err);
-    else
-        k_knn<float><<<g, SEARCH_THREADS, 0, s>>>((const float*)ix->node_coords, ix->node_tuple, m, ix->k,
-                                                  (const float*)q, nq, kn, di, dd, d_err);
-    kd::ctx_add_launches(ctx, 1);
+    launch_knn(ctx, ix, q, nq, kn, di, dd, d_err, s);
     if (!on_device) {
         cudaMemcpyAsync(idx_out, di, (size_t)nq * kn * 4, cudaMemcpyDeviceToHost, s);
         if (dist_out) cudaMemcpyAsync(dist_out, dd, (size_t)nq * kn * 8, cudaMemcpyDeviceToHost, s);
     }
     return read_err(ctx, d_err, s);
-}
-
-// m nearest neighbours of every node (address order), its own tuple excluded.
-static kd_status knn_all_device(kd_ctx* ctx, kd_index ix, int kn, int32_t* di, double* dd, int* d_err,
-                                cudaStream_t s) {
-    const int64_t m = ix->m;
-    const int g = grid_of(m, SEARCH_THREADS);
-    if (ix->dtype == KD_I32)
-        k_knn<int32_t><<<g, SEARCH_THREADS, 0, s>>>((const int32_t*)ix->node_coords, ix->node_tuple, (int32_t)m,
-                                                    ix->k, nullptr, m, kn, di, dd, d_err);
-    else if (ix->dtype == KD_I64)
-        k_knn<int64_t><<<g, SEARCH_THREADS, 0, s>>>((const int64_t*)ix->node_coords, ix->node_tuple, (int32_t)m,
-                                                    ix->k, nullptr, m, kn, di, dd, d_err);
-    else
-        k_knn<float><<<g, SEARCH_THREADS, 0, s>>>((const float*)ix->node_coords, ix->node_tuple, (int32_t)m, ix->k,
-                                                  nullptr, m, kn, di, dd, d_err);
-    kd::ctx_add_launches(ctx, 1);
-    return KD_OK;
 }
 
 kd_status kd_knn_all(kd_ctx* ctx, kd_index ix, int kn, int on_device, int32_t* idx_out, double* dist_out) {
@@ -560,7 +1051,7 @@ kd_status kd_knn_all(kd_ctx* ctx, kd_index ix, int kn, int on_device, int32_t* i
     if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
     if (st != KD_OK) return st;
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
-    knn_all_device(ctx, ix, kn, di, dd, d_err, s);
+    launch_knn(ctx, ix, nullptr, ix->m, kn, di, dd, d_err, s);
     if (!on_device) {
         cudaMemcpyAsync(idx_out, di, (size_t)ix->m * kn * 4, cudaMemcpyDeviceToHost, s);
         if (dist_out) cudaMemcpyAsync(dist_out, dd, (size_t)ix->m * kn * 8, cudaMemcpyDeviceToHost, s);
@@ -611,13 +1102,13 @@ kd_status kd_reverse_knn(kd_ctx* ctx, kd_index ix, int kn, int on_device, int64_
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
     cudaMemsetAsync(inv, 0xff, (size_t)n * 4, s);
     cudaMemsetAsync(cnt, 0, (size_t)m * 8, s);
-    knn_all_device(ctx, ix, kn, nn, nullptr, d_err, s);
+    launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, s);
     k_inv_map<<<grid_of(m, 256), 256, 0, s>>>(ix->node_tuple, m, n, inv, d_err);
     k_rev_count<<<grid_of(total, 256), 256, 0, s>>>(nn, total, inv, n, cnt, d_err);
-    k_offsets<<<1, 1024, 0, s>>>(cnt, m, offs);
+    launch_offsets(ctx, cnt, m, cursor, offs, s);  // (the cursors' words hold the chunk sums meanwhile)
     cudaMemcpyAsync(cursor, offs, (size_t)(m + 1) * 8, cudaMemcpyDeviceToDevice, s);
     k_rev_fill<<<grid_of(total, 256), 256, 0, s>>>(nn, total, kn, ix->node_tuple, inv, n, cursor, rev, d_err);
-    kd::ctx_add_launches(ctx, 4);
+    kd::ctx_add_launches(ctx, 3);
     int64_t tot = 0;
     cudaMemcpyAsync(&tot, offs + m, 8, cudaMemcpyDeviceToHost, s);
     if (!on_device) {
@@ -639,34 +1130,18 @@ kd_status kd_region(kd_ctx* ctx, kd_index ix, const void* lo, const void* hi, in
     const void *dlo = nullptr, *dhi = nullptr;
     kd_status st = to_device(ctx, S, lo, (size_t)nq * ix->k * ts, on_device, &dlo, s);
     if (st == KD_OK) st = to_device(ctx, S, hi, (size_t)nq * ix->k * ts, on_device, &dhi, s);
-    int64_t *counts = nullptr, *doffs = offsets;
+    uint32_t* counts = nullptr;
+    int64_t *sums = nullptr, *doffs = offsets;
     int* d_err = nullptr;
-    if (st == KD_OK) st = S.get((void**)&counts, (size_t)std::max<int64_t>(nq, 1) * 8);
+    const int64_t chunks = offsets_chunks(nq);  // the chunk sums of the scan, then the counts, in one allocation
+    if (st == KD_OK) st = S.get((void**)&sums, (size_t)chunks * 8 + (size_t)nq * 4);
+    counts = reinterpret_cast<uint32_t*>(sums + chunks);
     if (st == KD_OK && !on_device) st = S.get((void**)&doffs, (size_t)(nq + 1) * 8);
     if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
     if (st != KD_OK) return st;
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
-    const int g = grid_of(nq, SEARCH_THREADS);
-    const int32_t m = (int32_t)ix->m;
-    auto launch = [&](const int64_t* offs, int32_t* out) {
-        if (nq == 0) return;
-        if (ix->dtype == KD_I32)
-            k_region<int32_t><<<g, SEARCH_THREADS, 0, s>>>((const int32_t*)ix->node_coords, ix->node_tuple, m, ix->k,
-                                                           (const int32_t*)dlo, (const int32_t*)dhi, nq, counts, offs,
-                                                           out, d_err);
-        else if (ix->dtype == KD_I64)
-            k_region<int64_t><<<g, SEARCH_THREADS, 0, s>>>((const int64_t*)ix->node_coords, ix->node_tuple, m, ix->k,
-                                                           (const int64_t*)dlo, (const int64_t*)dhi, nq, counts, offs,
-                                                           out, d_err);
-        else
-            k_region<float><<<g, SEARCH_THREADS, 0, s>>>((const float*)ix->node_coords, ix->node_tuple, m, ix->k,
-                                                         (const float*)dlo, (const float*)dhi, nq, counts, offs, out,
-                                                         d_err);
-        kd::ctx_add_launches(ctx, 1);
-    };
-    launch(nullptr, nullptr);
-    k_offsets<<<1, 1024, 0, s>>>(counts, nq, doffs);
-    kd::ctx_add_launches(ctx, 1);
+    launch_region(ctx, ix, dlo, dhi, nq, counts, nullptr, nullptr, d_err, s);
+    launch_offsets(ctx, counts, nq, sums, doffs, s);
     int64_t total = 0;
     cudaMemcpyAsync(&total, doffs + nq, 8, cudaMemcpyDeviceToHost, s);
     st = read_err(ctx, d_err, s);  // synchronises
@@ -681,7 +1156,7 @@ kd_status kd_region(kd_ctx* ctx, kd_index ix, const void* lo, const void* hi, in
             st = S.get((void**)&dout, (size_t)total * 4);
             if (st != KD_OK) return st;
         }
-        launch(doffs, dout);
+        launch_region(ctx, ix, dlo, dhi, nq, counts, doffs, dout, d_err, s);
         if (!on_device) cudaMemcpyAsync(idx_out, dout, (size_t)total * 4, cudaMemcpyDeviceToHost, s);
     }
     return read_err(ctx, d_err, s);
