@@ -31,8 +31,10 @@ cudaError_t launch_transform(int dtype, const void* coords, int64_t n, int k, vo
 size_t sort_status_words(int64_t max_count);
 cudaError_t launch_sort_pass(int key64, const int64_t* count_ptr, int64_t max_count, const void* key_src,
                              void* key_dst, const PayloadArgs& pay, const uint32_t* digit_base, int shift,
-                             uint32_t* status, int* err, cudaStream_t s, uint32_t spin_limit = SPIN_LIMIT,
-                             int withhold = 0);
+                             uint32_t* status, uint32_t pass, int* err, cudaStream_t s,
+                             uint32_t spin_limit = SPIN_LIMIT, int withhold = 0);
+bool sort_pass_small(int64_t max_count);
+size_t sort_small_words(int64_t max_count);
 cudaError_t launch_digit_bases(const uint32_t* hist, int nrows, uint32_t* bases, cudaStream_t s);
 cudaError_t launch_pack_clouds(const PackDesc* d, int count, void* dst, cudaStream_t s);
 cudaError_t launch_gather(int key64, const int64_t* count_ptr, int64_t max_count, const void* plane,
@@ -74,6 +76,12 @@ cudaError_t launch_level_pass(int k, int tile, const AllBufs& bufs, int q, const
                               const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, uint32_t* status,
                               int* err, cudaStream_t s);
 size_t level_status_words(int k, int ntiles);
+int level_small_tile();
+bool level_steps_small(int64_t m);
+size_t level_small_bytes(int k, int64_t max_ntiles, int nsteps);
+cudaError_t launch_level_small(int k, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
+                               const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, void* area,
+                               int64_t max_ntiles, int step, int* err, cudaStream_t s);
 size_t finish_smem(int k, int smax);
 cudaError_t init_presort_kernels();
 cudaError_t init_build_kernels();
@@ -609,6 +617,10 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     const size_t status_words = sort_status_words(N);
     const size_t dedup_words = dedup_scratch_words(N);
     CKS(S.get(&status, (status_words + dedup_words) * 4));
+    uint32_t pass_no = 0;  // sort passes so far
+    const bool small_passes = sort_pass_small(N);
+    const int pass_extra = small_passes ? 0 : 2;  // launches of a pass beside its move
+    if (small_passes) CK(cudaMemsetAsync(status, 0, sort_small_words(N) * 4, s));
     unsigned char* kbuf[2];
     uint32_t* ibuf[2];
     const int maxpay = k + 1;
@@ -669,9 +681,9 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             const bool inject = ctx->inject_timeout && i == 0;
             {
                 LaunchTimer lt(ctx, F_SORT, (double)N, nullptr, pass_bytes(P, kdst != nullptr, pay.n));
-                ctx->launches += 2;  // count and scan kernels of the pass
+                ctx->launches += pass_extra;  // count and scan kernels of the pass
                 CK(launch_sort_pass(plane64(P.plane), d_n, N, ksrc, kdst, pay,
-                                    bases_all + (size_t)row_of(P.plane, P.digit) * RADIX, 8 * P.digit, status, d_err, s,
+                                    bases_all + (size_t)row_of(P.plane, P.digit) * RADIX, 8 * P.digit, status, ++pass_no, d_err, s,
                                     ctx->spin_limit, inject ? 1 : 0));
             }
             if (inject) {  // the injected wait: report it before anything else runs
@@ -764,9 +776,9 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             ksrc = kbuf[kc];
         }
         LaunchTimer lt(ctx, F_SORT, 0.0, H->d_m, pass_bytes(P, !last, 1));
-        ctx->launches += 2;  // count and scan kernels of the pass
+        ctx->launches += pass_extra;  // count and scan kernels of the pass
         CK(launch_sort_pass(0, H->d_m, N, ksrc, last ? nullptr : (void*)kbuf[kc ^ 1], pay,
-                            bases_kept + (size_t)row_of(-1, P.digit) * RADIX, 8 * P.digit, status, d_err, s,
+                            bases_kept + (size_t)row_of(-1, P.digit) * RADIX, 8 * P.digit, status, ++pass_no, d_err, s,
                             ctx->spin_limit));
         kc ^= 1;
         ic ^= 1;
@@ -844,10 +856,10 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
                     ksrc = kbuf[kc];
                 }
                 LaunchTimer lt(ctx, F_SORT, 0.0, H->d_m, pass_bytes(P, kdst != nullptr, pay.n));
-                ctx->launches += 2;  // count and scan kernels of the pass
+                ctx->launches += pass_extra;  // count and scan kernels of the pass
                 CK(launch_sort_pass(plane64(P.plane), H->d_m, N, ksrc, kdst, pay,
                                     bases_kept + (size_t)row_of(P.plane, P.digit) * RADIX, 8 * P.digit, status,
-                                    d_err, s, ctx->spin_limit));
+                                    ++pass_no, d_err, s, ctx->spin_limit));
                 kc ^= 1;
                 if (carry_id) cur_id = new_id;
                 for (size_t j = 0; j < ranks.size(); ++j) rsrc[j] = last ? H->rec.p[d][ranks[j]] : pbuf[pb][j];
@@ -899,8 +911,8 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
                 uint32_t* gdest = ibuf[0];
                 {
                     LaunchTimer lt(ctx, F_RECORDS, 0.0, H->d_m, 4.0 + 8.0 * nv + 4.0);
-                    ctx->launches += 2;  // count and scan kernels of the pass
-                    CK(launch_sort_pass(0, H->d_m, N, H->rec.p[1][d], gdest, pay, pbases, shift, status, d_err, s,
+                    ctx->launches += pass_extra;  // count and scan kernels of the pass
+                    CK(launch_sort_pass(0, H->d_m, N, H->rec.p[1][d], gdest, pay, pbases, shift, status, ++pass_no, d_err, s,
                                         ctx->spin_limit));
                 }
                 PayloadArgs sc{};
@@ -1042,6 +1054,9 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
     }
     ctx->last_smax = smax;
     ctx->last_ltile = tile;
+    // few tuples: every level step is one launch
+    const bool small_steps = level_steps_small(M);
+    if (small_steps) tile = level_small_tile();
     if (k >= 2 && smax * 3 < tile + 3) return fail(ctx, KD_EINVAL, "switch threshold too small");
 
     // outputs: user device arrays, or staging for host arrays
@@ -1266,12 +1281,17 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
     CK(cudaMemcpyAsync(d_uprefix, unit_prefix.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
     // per step: tile counts, their segmented scan and head flags (no zeroing needed)
     size_t st_words = 0;
-    for (size_t st = 0; st < step_jobs.size(); ++st)
+    int64_t max_ntiles = 0;
+    for (size_t st = 0; st < step_jobs.size(); ++st) {
         st_words = std::max(st_words, level_status_words(std::max(k, 2), (int)step_ntiles[st]));
+        max_ntiles = std::max(max_ntiles, step_ntiles[st]);
+    }
+    if (small_steps) st_words = level_small_bytes(std::max(k, 2), max_ntiles, (int)step_jobs.size()) / 4;
     if (!flat.empty()) {
         CKS(S.get(&d_jobs, sizeof(LevelJob) * flat.size()));
         CK(cudaMemcpyAsync(d_jobs, flat.data(), sizeof(LevelJob) * flat.size(), cudaMemcpyHostToDevice, s));
         CKS(S.get(&d_status, st_words * 4));
+        if (small_steps) CK(cudaMemsetAsync(d_status, 0, st_words * 4, s));
     }
     // launches ----------------------------------------------------------------
     {
@@ -1282,6 +1302,11 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
         const int F = step_jobs[st][0].lev_out - step_jobs[st][0].lev_in;
         // array q moves k planes (array 0) or k - 1 (its own rank is not carried)
         LaunchTimer lt(ctx, F_LEVEL, step_elems[st], nullptr, 8.0 * (k - (step_q[st] != 0)) + 4.0 * F);
+        if (small_steps) {
+            CK(launch_level_small(k, bufs, step_q[st], d_jobs + job_off[st], (int)step_jobs[st].size(),
+                                  (int)step_ntiles[st], d_cd, medr, H->perm0, d_status, max_ntiles, (int)st, d_err, s));
+            continue;
+        }
         ctx->launches += 3;  // tile records, count pass and scan
         CK(launch_level_pass(k, tile, bufs, step_q[st], d_jobs + job_off[st], (int)step_jobs[st].size(),
                              (int)step_ntiles[st], d_cd, medr, H->perm0, d_status, d_err, s));

@@ -711,6 +711,278 @@ __global__ void __launch_bounds__(LEVEL_BLOCK, K <= 3 ? 3 : 2)
     }
 }
 
+// ------------------------------------------- level step, few tiles
+// The whole level step in one launch, one tile of 1024 positions per block:
+// the tile's elements go straight to registers while warp 0 finds the
+// tile's segments and medians; the counts of earlier tiles come from a
+// decoupled look-back.  A step of few tiles is bound by the latency of its
+// launches, not by the bytes it moves: the four launches above take 26 us
+// on 300007 tuples of k = 4, this one 11 (profiler, serialised).  (As one
+// persistent kernel with staged copies the fused step was slower than the
+// four launches on large steps, whose move is bound by instruction issue:
+// 450 us against 407 at 2^26 tuples.)
+//
+// Look-back.  A tile publishes, per bucket of its last segment, one 64-bit
+// word: the count of its own elements (AGG), or, once known, of all the
+// segment's elements up to and including its own (INC; at once where the
+// segment starts in the tile).  The state shares the word with the value, so
+// a word is read and believed without a fence, and carries the step's
+// number, so the words are cleared once per build.  Blocks take their tile
+// from a counter, so the tiles a block waits for belong to blocks that
+// already run.
+constexpr int SMALL_IPT = 4;
+constexpr int SMALL_TILE = LEVEL_THREADS * SMALL_IPT;
+constexpr int LB_ROWS = 8;  // rows of status words a look-back round trip reads
+constexpr uint32_t LB_AGG = 1u, LB_INC = 2u;
+
+__device__ __forceinline__ uint64_t ld_status(const uint64_t* p) {
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_status(uint64_t* p, uint32_t epoch, uint32_t state, uint32_t value) {
+    const uint64_t v = ((uint64_t)(epoch << 2 | state) << 32) | value;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Sums of nbl (a power of two, at most 32) buckets over the tiles t - 1,
+// t - 2, ..., t_head (where the segment starts); status points to the first
+// of them.  Called by a whole warp; with fewer than 32 buckets the lanes hold
+// several tiles of a row.  Lane i < nbl returns bucket i's sum.
+__device__ __forceinline__ uint32_t level_lookback(const uint64_t* __restrict__ status, int nbp, int nbl, int t,
+                                                   int t_head, uint32_t epoch, int* err) {
+    const int lane = threadIdx.x & 31;
+    const int tpw = 32 / nbl, off = lane / nbl;
+    const uint64_t* col = status + (lane & (nbl - 1));
+    // the lanes holding this lane's bucket, nearest tile first
+    const uint32_t mine = (nbl == 32 ? 1u : 0xffffffffu / ((1u << nbl) - 1u)) << (lane & (nbl - 1));
+    const uint64_t past = (uint64_t)(epoch << 2 | LB_INC) << 32;  // tiles before t_head: nothing
+    uint32_t part = 0, spins = 0;
+    bool done = false;
+    int hi = t - 1;
+    for (;;) {
+        uint64_t w[LB_ROWS];
+#pragma unroll
+        for (int r = 0; r < LB_ROWS; ++r) {
+            const int u = hi - (r * tpw + off);
+            w[r] = u >= t_head ? ld_status(col + (int64_t)u * nbp) : past;
+        }
+        bool stuck = false;
+        int rows = 0;
+#pragma unroll
+        for (int r = 0; r < LB_ROWS; ++r) {
+            if (stuck) continue;
+            const uint32_t f = (uint32_t)(w[r] >> 32);
+            const bool ready = (f >> 2) == epoch;
+            const uint32_t inc = __ballot_sync(0xffffffffu, ready && (f & 3u) == LB_INC) & mine;
+            const uint32_t late = __ballot_sync(0xffffffffu, !ready) & mine;
+            const uint32_t upto = inc ? (2u << (__ffs(inc) - 1)) - 1u : 0xffffffffu;
+            if (__any_sync(0xffffffffu, !done && (late & upto))) {
+                stuck = true;
+            } else {
+                if (!done) {
+                    if ((upto >> lane) & 1u) part += (uint32_t)w[r];
+                    done = inc != 0;
+                }
+                rows = r + 1;
+            }
+        }
+        if (__all_sync(0xffffffffu, done)) break;
+        hi -= rows * tpw;
+        if (stuck) {
+            if (++spins > SPIN_LIMIT) {
+                if (lane == 0) atomicOr(err, ERR_TIMEOUT);
+                break;
+            }
+            __nanosleep(100);
+        }
+    }
+    for (int o = nbl; o < 32; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    return part;
+}
+
+// The last of the jobs whose tile_begin is at most t (whole warp).
+__device__ __forceinline__ int warp_find_job(const LevelJob* __restrict__ jobs, int njobs, int t) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, n = njobs;  // the job is in [lo, lo + n)
+    while (n > 1) {
+        const int step = (n + 31) / 32;
+        const int i = lane * step;
+        const uint32_t le = __ballot_sync(0xffffffffu, i < n && jobs[lo + i].tile_begin <= t);
+        const int c = 31 - __clz(le);  // (lane 0 always: the first job of the range begins at or before t)
+        lo += c * step;
+        n = min(step, n - c * step);
+    }
+    return lo;
+}
+
+template <int K>
+__global__ void __launch_bounds__(LEVEL_THREADS)
+    k_level_small(const __grid_constant__ AllBufs bufs, int q, const LevelJob* __restrict__ jobs, int njobs,
+                  const CloudDev* __restrict__ clouds, uint32_t* __restrict__ medr, const uint32_t* __restrict__ perm0,
+                  uint64_t* __restrict__ status, uint32_t epoch, uint32_t* __restrict__ ctr, int* __restrict__ err) {
+    constexpr int IPT = SMALL_IPT, TILE = SMALL_TILE;
+    constexpr int NBMAX = 1 << (K - 1);
+    constexpr int NDMAX = LEVEL_NSMAX * NBMAX;
+    __shared__ uint32_t s_rec[trec_words(K)];
+    __shared__ uint32_t s_wc[LEVEL_WARPS][NDMAX];
+    __shared__ int32_t s_dmid[NDMAX];
+    __shared__ uint32_t s_ticket;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < LEVEL_WARPS * NDMAX; i += LEVEL_THREADS) (&s_wc[0][0])[i] = 0;
+    // the counters, jobs, clouds and the tile's segments do not depend on the
+    // previous step: they are ready when its last block ends
+    if (tid == 0) s_ticket = atomicAdd(ctr, 1u);
+    __syncthreads();
+    const int t = (int)s_ticket;
+    const LevelJob J = jobs[warp_find_job(jobs, njobs, t)];
+    const CloudDev& C = clouds[J.cloud];
+    const int32_t m = C.m, pos0 = (int32_t)((int64_t)(t - J.tile_begin) * TILE);
+    const int32_t npos = min(m - pos0, TILE);
+    const int64_t goff = C.off;
+    const int F = J.lev_out - J.lev_in, NB = 1 << F;
+    const int own = q != 0 ? (q - J.lev_in % K + K) % K : -1;  // slot of the array's own plane: not carried
+    if (warp == 0) {
+        // the first segment at or after pos0 (pos0 itself may be a node of a
+        // shallower level), then its neighbours, one per lane
+        Seg sg = segment_of(pos0, m, J.lev_in);
+        if (sg.idx < 0 && npos > 1) sg = segment_of(pos0 + 1, m, J.lev_in);
+        int32_t lo = 0, hi = -1;
+        const int64_t si = (int64_t)sg.idx + lane;
+        bool in = sg.idx >= 0 && si < ((int64_t)1 << J.lev_in);
+        if (in) {
+            segment_bounds(m, J.lev_in, (int32_t)si, lo, hi);
+            in = lo <= pos0 + npos - 1;
+        }
+        int ns = __popc(__ballot_sync(0xffffffffu, in));
+        if (ns > LEVEL_NSMAX) {
+            if (lane == 0) atomicOr(err, ERR_INTERNAL);
+            ns = LEVEL_NSMAX;
+        }
+        if (lane < LEVEL_NSMAX) {
+            s_rec[1 + lane] = (uint32_t)(lane < ns ? lo : 0);
+            s_rec[5 + lane] = (uint32_t)(lane < ns ? hi : -1);
+            s_rec[9 + lane] = (uint32_t)(lane < ns ? si : 0);
+        }
+        if (lane == 0) s_rec[0] = (uint32_t)ns;
+    }
+    pdl_wait();  // the previous step's planes and medians
+    pdl_trigger();
+    uint32_t v[K][IPT];
+#pragma unroll
+    for (int f = 0; f < K; ++f) {
+        const uint32_t* src = bufs.p[q][J.src_buf][(J.lev_in + f) % K] + goff + pos0;
+#pragma unroll
+        for (int j = 0; j < IPT; ++j) {
+            const int o = warp * 32 * IPT + j * 32 + lane;
+            v[f][j] = f != own && o < npos ? src[o] : 0u;
+        }
+    }
+    if (warp == 0) {
+        __syncwarp();
+        const int per = NB - 1, sidx = (int)s_rec[9];
+        for (int e = lane; e < (int)s_rec[0] * per; e += 32) {
+            const int j = e / per, h = e - j * per + 1, f = 31 - __clz(h);
+            const int64_t gseg = ((int64_t)(sidx + j) << f) + (h - (1 << f));
+            s_rec[TR_HEAD + j * NBMAX + h] = medr[C.medr_off + ((int64_t)1 << (J.lev_in + f)) - 1 + gseg];
+        }
+    }
+    __syncthreads();
+    const int ns = (int)s_rec[0];
+    int32_t tlo[LEVEL_NSMAX], thi[LEVEL_NSMAX];
+    tile_bounds(s_rec, tlo, thi);
+    const uint32_t marker = (uint32_t)(ns * NB);
+    uint32_t dig[IPT], rank[IPT];
+#pragma unroll
+    for (int j = 0; j < IPT; ++j) {
+        const int o = warp * 32 * IPT + j * 32 + lane;
+        dig[j] = marker;
+        const int sj = o < npos ? tile_slot(tlo, thi, ns, pos0 + o) : -1;
+        if (sj >= 0) {
+            uint32_t r[K];
+#pragma unroll
+            for (int f = 0; f < K; ++f) r[f] = v[f][j];
+            const uint32_t d = route_rec<K>(r, F, sj, s_rec);
+            if (d != INV) dig[j] = d;
+        }
+    }
+    warp_rank<IPT>(dig, marker, s_wc[warp], rank);
+    __syncthreads();
+    // per digit: prefix over warps, base and middle of its final segment; the
+    // counts of the tile's last segment are published
+    const bool cont = ns > 0 && tlo[0] < pos0;  // the first segment continues earlier tiles
+    uint64_t* const row = status + (int64_t)t * NBMAX;
+    uint32_t total = 0;  // of digit tid
+    for (int d = tid; d < ns * NB; d += LEVEL_THREADS) {
+        const int sj = d >> F, b = d - (sj << F);
+        int32_t a = (int32_t)s_rec[1 + sj], z = (int32_t)s_rec[5 + sj];
+        const bool starts = a >= pos0;
+        for (int f = F - 1; f >= 0; --f) {
+            const int32_t mid = a + ((z - a) >> 1);
+            if ((b >> f) & 1) a = mid + 1; else z = mid - 1;
+        }
+        uint32_t c = 0;
+#pragma unroll
+        for (int w = 0; w < LEVEL_WARPS; ++w) {
+            const uint32_t x = s_wc[w][d];
+            s_wc[w][d] = (uint32_t)a + c;
+            c += x;
+        }
+        if (d == tid) total = c;
+        if (sj == ns - 1) st_status(row + b, epoch, starts ? LB_INC : LB_AGG, c);
+        s_dmid[d] = (J.write_med & LEVEL_MED) ? a + ((z - a) >> 1) : -2;
+    }
+    if (cont && warp * 32 < NB) {
+        __syncwarp();
+        // tiles of this job back to the one holding the segment's first position
+        const int t_head = t - (pos0 - tlo[0] + TILE - 1) / TILE;
+        const uint32_t before = level_lookback(status + warp * 32, NBMAX, NB < 32 ? NB : 32, t, t_head, epoch, err);
+        if (tid < NB) {
+            if (ns == 1) st_status(row + tid, epoch, LB_INC, before + total);
+#pragma unroll
+            for (int w = 0; w < LEVEL_WARPS; ++w) s_wc[w][tid] += before;
+        }
+    }
+    __syncthreads();
+    int32_t dest[IPT];
+#pragma unroll
+    for (int j = 0; j < IPT; ++j) {
+        dest[j] = -1;
+        const uint32_t d = dig[j];
+        if (d >= marker) continue;
+        const int32_t dd = (int32_t)(s_wc[warp][d] + rank[j]);
+        const int sj = (int)(d >> F);
+        // the destination must lie in the element's segment; any other value
+        // means inconsistent inputs and is never written
+        if (dd < (int32_t)s_rec[1 + sj] || dd > (int32_t)s_rec[5 + sj]) {
+            atomicOr(err, ERR_INTERNAL);
+            continue;
+        }
+        dest[j] = dd;
+        if (dd == s_dmid[d]) {
+            const int32_t si = ((int32_t)s_rec[9 + sj] << F) + (int32_t)(d - ((uint32_t)sj << F));
+            // rank 0 of the median (its position in array 0) gives its tuple
+            // and, through array 0's initial record, its rank in super key q
+            const uint32_t r0 = plane_value<K, IPT>(v, j, (K - J.lev_in % K) % K);
+            if (r0 >= goff && r0 < goff + m) {
+                medr[C.medr_off + ((int64_t)1 << J.lev_out) - 1 + si] = q == 0 ? r0 : bufs.p[0][0][q][r0];
+                C.node[dd] = (int32_t)((int64_t)perm0[r0] - C.in_off);
+            } else {
+                atomicOr(err, ERR_INTERNAL);
+            }
+        }
+    }
+    const bool final_move = (J.write_med & LEVEL_FINAL) != 0;  // only rank 0 is read after it
+#pragma unroll
+    for (int f = 0; f < K; ++f) {
+        if (f == own || (final_move && (J.lev_in + f) % K != 0)) continue;
+        uint32_t* dp = bufs.p[q][J.dst_buf][(J.lev_in + f) % K] + goff;
+#pragma unroll
+        for (int j = 0; j < IPT; ++j)
+            if (dest[j] >= 0) dp[dest[j]] = v[f][j];
+    }
+}
+
 // ------------------------------------------------------------- finisher
 
 __device__ __forceinline__ uint32_t seg_pack(int32_t a, int32_t b) { return (uint32_t)a | ((uint32_t)b << 16); }
@@ -1305,6 +1577,40 @@ cudaError_t launch_level_pass(int k, int tile, const AllBufs& bufs, int q, const
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+
+// Status area of a build's one-launch level steps: the look-back words of
+// max_ntiles tiles, then a tile counter per step.  Cleared once, before the
+// first of them.
+int level_small_tile() { return SMALL_TILE; }
+// Most tuples of a build whose level steps are one launch each.  Whole builds,
+// four launches per step against one (k = 3 float32): 16384 tuples 564 -> 531
+// us, 2^18 704 -> 637, 2^20 1000 -> 923, 2^21 1264 -> 1238, 2^22 1829 ->
+// 1911; k = 6 int64: 2^20 2360 -> 2188.
+bool level_steps_small(int64_t m) { return m <= (int64_t)1 << 21; }
+static size_t small_counters_at(int k, int64_t max_ntiles) { return (size_t)max_ntiles * ((size_t)8 << (k - 1)); }
+size_t level_small_bytes(int k, int64_t max_ntiles, int nsteps) {
+    return small_counters_at(k, max_ntiles) + (size_t)nsteps * 4;
+}
+
+// launch_level_pass in one launch, for the jobs' tiles of SMALL_TILE
+// positions; `step` numbers the build's calls.
+cudaError_t launch_level_small(int k, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
+                               const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, void* area,
+                               int64_t max_ntiles, int step, int* err, cudaStream_t s) {
+    if (ntiles == 0) return cudaSuccess;
+    uint64_t* status = static_cast<uint64_t*>(area);
+    uint32_t* ctr =
+        reinterpret_cast<uint32_t*>(static_cast<unsigned char*>(area) + small_counters_at(k, max_ntiles)) + step;
+#define KD_SMALL(K)                                                                                                \
+    case K:                                                                                                        \
+        return launch_dependent(k_level_small<K>, dim3(ntiles), dim3(LEVEL_THREADS), 0, s, bufs, q, jobs, njobs,   \
+                                clouds, medr, perm0, status, (uint32_t)step + 1u, ctr, err);
+    switch (k) {
+        KD_SMALL(2) KD_SMALL(3) KD_SMALL(4) KD_SMALL(5) KD_SMALL(6) KD_SMALL(7) KD_SMALL(8)
+        default: return cudaErrorInvalidValue;
+    }
+#undef KD_SMALL
 }
 
 template <int K, int IPT>

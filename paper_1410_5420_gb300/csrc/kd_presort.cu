@@ -595,6 +595,176 @@ __global__ void __launch_bounds__(RS_BLOCK, (rs_min_blocks<KW, TILE, SP>()))
     }
 }
 
+// ----------------------------------------------- sort pass, few tiles
+// A whole digit pass in one launch, one tile of 2048 elements per block: the
+// tile's keys and payloads come in by bulk copies, are ranked as in
+// k_rs_move, the tile's digit counts are published, and the counts of
+// earlier tiles come from a decoupled look-back, one thread per digit.  A
+// pass of few tiles is bound by the latency of its launches: count, scan
+// and move take 19 us on 300007 elements with three payload planes, this one
+// launch 13; on 16384 elements 14 and 9 (profiler, serialised).
+//
+// A status word holds the pass number (9 bits), a state (1: the tile's own
+// count, 2: the count up to and including it) and a count of 21 bits, so
+// the words are cleared once per presort and believed without a fence.
+// Blocks take their tile from a counter, so the tiles a block waits for
+// belong to blocks that already run.
+constexpr int RS_SMALL_TILE = 2048;
+constexpr int RS_SMALL_ROWS = 16;  // status rows a look-back round trip reads
+// Most elements of such a pass.  Whole builds, three launches per pass against
+// one (k = 3): 16384 float32 534 -> 483 us, 2^18 643 -> 583, 2^20 922 -> 876,
+// 2 * 10^6 1221 -> 1248; int64 562 -> 516, 707 -> 631, 1046 -> 972, 1468 ->
+// 1435.  (The status words hold counts below 2^21.)
+constexpr int64_t RS_SMALL_MAX = (int64_t)3 << 19;
+constexpr uint32_t RS_SMALL_PASSES = 511;
+
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+template <typename KW>
+constexpr size_t rs_small_smem(int npay) {
+    return (size_t)RS_SMALL_TILE * (sizeof(KW) + 4 * (size_t)npay + 2);
+}
+
+template <typename KW>
+__global__ void __launch_bounds__(RS_THREADS)
+    k_rs_small(const int64_t* __restrict__ count_ptr, const KW* __restrict__ key_src, KW* __restrict__ key_dst,
+               const __grid_constant__ PayloadArgs pay, const uint32_t* __restrict__ digit_base, int shift,
+               uint32_t* __restrict__ status, uint32_t pass, uint32_t* __restrict__ ctr, int* __restrict__ err,
+               uint32_t spin_limit, int withhold) {
+    constexpr int TILE = RS_SMALL_TILE, IPT = TILE / RS_THREADS;
+    extern __shared__ __align__(128) unsigned char rss[];
+    KW* s_key = reinterpret_cast<KW*>(rss);                                     // [TILE], then payloads [pay.n][TILE]
+    uint32_t* s_pay = reinterpret_cast<uint32_t*>(s_key + TILE);
+    uint16_t* s_perm = reinterpret_cast<uint16_t*>(s_pay + (size_t)pay.n * TILE);  // element at each sorted place
+    __shared__ __align__(8) uint64_t full;
+    __shared__ uint32_t s_wc[RS_WARPS][RADIX];
+    __shared__ uint32_t s_match[RS_WARPS][RADIX];
+    __shared__ uint32_t s_goff[RADIX], s_tstart[RADIX];
+    __shared__ uint32_t s_wsum[RS_WARPS];
+    __shared__ uint32_t s_ticket;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        s_ticket = atomicAdd(ctr, 1u);  // (cleared long before the previous pass)
+        mbar_init(&full, 1);
+        fence_mbar_init();
+    }
+    for (int i = tid; i < RS_WARPS * RADIX; i += RS_THREADS) {
+        (&s_wc[0][0])[i] = 0;
+        (&s_match[0][0])[i] = 0;
+    }
+    __syncthreads();
+    const int64_t t = s_ticket;
+    pdl_wait();  // the previous pass's keys and payloads
+    pdl_trigger();
+    const int64_t count = *count_ptr;
+    const int64_t base = t * TILE;
+    if (base >= count) return;
+    const int n = (int)(count - base < TILE ? count - base : (int64_t)TILE);
+    if (tid == 0) {
+        const uint32_t kb = ((uint32_t)n * sizeof(KW) + 15u) & ~15u, pb = ((uint32_t)n * 4u + 15u) & ~15u;
+        int nst = 0;
+        for (int p = 0; p < pay.n; ++p) nst += pay.src[p] != nullptr;
+        mbar_arrive_expect_tx(&full, kb + (uint32_t)nst * pb);
+        bulk_g2s(s_key, key_src + base, kb, &full);
+        for (int p = 0; p < pay.n; ++p)
+            if (pay.src[p]) bulk_g2s(s_pay + (size_t)p * TILE, pay.src[p] + base, pb, &full);
+    }
+    const uint32_t dbase = digit_base[tid];
+    const bool ok = mbar_wait(&full, 0);
+    if (__syncthreads_or(!ok)) {
+        if (tid == 0) atomicOr(err, ERR_TIMEOUT);
+        return;
+    }
+    const int wbase = warp * 32 * IPT;
+    uint32_t dig[IPT], slot[IPT];
+#pragma unroll
+    for (int j = 0; j < IPT; ++j) {
+        const int o = wbase + j * 32 + lane;
+        dig[j] = o < n ? digit_of(s_key[o], shift) : (uint32_t)RADIX;
+    }
+    warp_rank_adaptive<IPT>(dig, RADIX, s_wc[warp], s_match[warp], slot);
+    __syncthreads();
+    // digit tid: prefix over warps, the tile's count (published), its first place
+    uint32_t c = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) {
+        const uint32_t x = s_wc[w][tid];
+        s_wc[w][tid] = c;
+        c += x;
+    }
+    uint32_t* const row = status + t * RADIX + tid;
+    if (!(withhold && t == 0)) st_relaxed(row, pass << 23 | (t == 0 ? 2u : 1u) << 21 | c);
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_wsum[warp] = x;
+    __syncthreads();
+    uint32_t tstart = x - c;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) tstart += w < warp ? s_wsum[w] : 0u;
+    s_tstart[tid] = tstart;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < IPT; ++j)
+        if (dig[j] < RADIX) s_perm[slot[j] + s_tstart[dig[j]] + s_wc[warp][dig[j]]] = (uint16_t)(wbase + j * 32 + lane);
+    // look-back of digit tid
+    uint32_t before = 0, spins = 0;
+    bool done = t == 0, late = false;
+    int64_t hi = t - 1;
+    while (!done) {
+        uint32_t w[RS_SMALL_ROWS];
+#pragma unroll
+        for (int r = 0; r < RS_SMALL_ROWS; ++r)
+            w[r] = hi - r >= 0 ? ld_relaxed(status + (hi - r) * RADIX + tid) : pass << 23 | 2u << 21;
+        int r = 0;
+#pragma unroll
+        for (int i = 0; i < RS_SMALL_ROWS; ++i) {
+            if (done || r != i || (w[i] >> 23) != pass) continue;
+            before += w[i] & 0x1fffffu;
+            done = (w[i] >> 21 & 3u) == 2u;
+            r = i + 1;
+        }
+        hi -= r;
+        if (!done && r == 0 && ++spins > spin_limit) {
+            late = true;
+            break;
+        }
+    }
+    if (t > 0 && !late) st_relaxed(row, pass << 23 | 2u << 21 | (before + c));
+    s_goff[tid] = dbase + before - tstart;  // destination of sorted place i with digit d: s_goff[d] + i
+    if (__syncthreads_or(late)) {
+        if (tid == 0) atomicOr(err, ERR_TIMEOUT);
+        return;
+    }
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const int i = r * RS_THREADS + tid;
+        if (i >= n) break;
+        const int o = s_perm[i];
+        const KW kk = s_key[o];
+        const uint32_t dd = s_goff[digit_of(kk, shift)] + (uint32_t)i;
+        // a destination outside [0, count) can only come from inconsistent
+        // counts; it is reported and never written
+        if ((int64_t)dd >= count) {
+            atomicOr(err, ERR_INTERNAL);
+            continue;
+        }
+        if (key_dst) key_dst[dd] = kk;
+        for (int p = 0; p < pay.n; ++p)
+            pay.dst[p][dd] = pay.src[p] ? s_pay[(size_t)p * TILE + o] : (uint32_t)(base + o);
+    }
+}
+
 // Gather of key words by tuple id: out[pos] = plane[ids[pos]], positions in
 // [0, *count_ptr).  Each thread issues GI independent gathers, so a random
 // read of the key plane keeps many requests in flight.
@@ -1412,6 +1582,18 @@ size_t sort_status_words(int64_t max_count) {
     return (size_t)(2 * tiles * RADIX + chunks + 2 * chunks * RADIX + 4);
 }
 
+// Whether passes over at most max_count elements are one launch each.
+bool sort_pass_small(int64_t max_count) {
+    return max_count <= RS_SMALL_MAX;
+}
+
+// Words at the start of the status area that such passes need cleared before
+// the first of them: a row of status words per tile, then a tile counter per
+// pass.
+size_t sort_small_words(int64_t max_count) {
+    return (size_t)((max_count + RS_SMALL_TILE - 1) / RS_SMALL_TILE) * RADIX + RS_SMALL_PASSES + 1;
+}
+
 // Resident blocks per SM of the move kernels (by variant) and the SM count.
 static int g_rs_occ[5];
 static int g_rs_sms = 0;
@@ -1440,15 +1622,29 @@ static cudaError_t rs_pass(const int64_t* count_ptr, int64_t max_count, const vo
 // One stable LSD pass over *count_ptr (<= max_count) elements on digit
 // (key >> shift) & 255: keys from key_src (written to key_dst when not
 // NULL), payload planes moved along (a NULL source means the position).
+// pass numbers the calls that share a status area, from 1.
 // Key, payload and plane buffers must be 16-byte aligned and readable up to
 // the count rounded up to a multiple of 4 elements.  spin_limit bounds the
 // scan's look-back polls; withhold is the failure-detection tests' switch
 // (k_rs_scan).
 cudaError_t launch_sort_pass(int key64, const int64_t* count_ptr, int64_t max_count, const void* key_src,
                              void* key_dst, const PayloadArgs& pay, const uint32_t* digit_base, int shift,
-                             uint32_t* status, int* err, cudaStream_t s, uint32_t spin_limit, int withhold) {
+                             uint32_t* status, uint32_t pass, int* err, cudaStream_t s, uint32_t spin_limit,
+                             int withhold) {
     if (max_count == 0) return cudaSuccess;
     if (g_rs_sms == 0) return cudaErrorInvalidValue;
+    if (sort_pass_small(max_count)) {
+        if (pass == 0 || pass > RS_SMALL_PASSES) return cudaErrorInvalidValue;
+        const unsigned tiles = (unsigned)((max_count + RS_SMALL_TILE - 1) / RS_SMALL_TILE);
+        uint32_t* ctr = status + (size_t)tiles * RADIX + pass;
+        if (key64)
+            return launch_dependent(k_rs_small<uint64_t>, dim3(tiles), dim3(RS_THREADS), rs_small_smem<uint64_t>(pay.n),
+                                    s, count_ptr, (const uint64_t*)key_src, (uint64_t*)key_dst, pay, digit_base, shift,
+                                    status, pass, ctr, err, spin_limit, withhold);
+        return launch_dependent(k_rs_small<uint32_t>, dim3(tiles), dim3(RS_THREADS), rs_small_smem<uint32_t>(pay.n), s,
+                                count_ptr, (const uint32_t*)key_src, (uint32_t*)key_dst, pay, digit_base, shift, status,
+                                pass, ctr, err, spin_limit, withhold);
+    }
     const SortStatusArea A = sort_status_layout(max_count, status);
     const bool many = pay.n > 1;
     if (!key64 && pay.n >= 3)
@@ -1499,6 +1695,8 @@ cudaError_t init_presort_kernels() {
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_rs_sms, cudaDevAttrMultiProcessorCount, dev);
+    set((const void*)k_rs_small<uint32_t>, rs_small_smem<uint32_t>(MAXPAY));
+    set((const void*)k_rs_small<uint64_t>, rs_small_smem<uint64_t>(MAXPAY));
     if (e == cudaSuccess) e = init_rs_move<uint32_t, 2048, 1>(&g_rs_occ[0]);
     if (e == cudaSuccess) e = init_rs_move<uint32_t, 2048, 2>(&g_rs_occ[1]);
     if (e == cudaSuccess) e = init_rs_move<uint64_t, 2048, 1>(&g_rs_occ[2]);
