@@ -5,27 +5,19 @@
 // has already handed all device memory to its own allocator (a call would
 // then fail with KD_ENOMEM), or a latency-bound loop where a growing pool or
 // a cudaFree would stall the device for every stream.  kd_presort_noalloc
-// serves them for clouds of up to KD_NOALLOC_MAX_N tuples: its only
-// workspace is one file-scope device array (1 MiB of key planes plus a
-// status word), set up once per device, and its outputs go to buffers the
-// caller owns.
+// serves them for clouds of up to KD_NOALLOC_MAX_N tuples: its outputs go to
+// buffers the caller owns, and what it needs beside them fits the shared
+// memory of one thread block per super key (k_small_sort in kd_small.cu, one
+// launch).
 //
 // It computes what kd_presort + kd_handle_arrays compute (Section 2.1: the
 // k index arrays sorted by the cyclic super keys x_d : x_{d+1} : ... and
-// duplicate tuples removed, the smallest index of a run surviving) with two
-// kernels sized for small clouds:
-//   k_noalloc_keys  coordinates -> order-preserving unsigned key planes in
-//                   the static array; a NaN sets the status word;
-//   k_noalloc_sort  one block per super key d: the indices and their key
-//                   x_d in shared memory, a bitonic sort whose comparisons
-//                   fall back to x_{d+1}, ... (static array, L2-resident)
-//                   and then to the index on ties, then an adjacent-compare
-//                   and block-scan compaction dropping duplicate tuples.
+// duplicate tuples removed, the smallest index of a run surviving).
 //
-// The one static array per device is shared by every call on that device:
-// two calls whose kernels can overlap (different streams, or different
-// threads without ordering between them) race on it.  Order such calls on
-// one stream.
+// The blocks read the coordinates until the last of them ends.  A call whose
+// outputs overlap its coordinates therefore first copies these to a
+// file-scope device array (1 MiB per device, set up once): two such calls on
+// one device whose work can overlap race on it.
 #include <mutex>
 #include <string>
 
@@ -38,131 +30,19 @@ int ctx_device(const kd_ctx* ctx);
 cudaStream_t ctx_stream(const kd_ctx* ctx);
 void ctx_set_error(kd_ctx* ctx, const std::string& msg);
 void ctx_add_launches(kd_ctx* ctx, int n);
+cudaError_t launch_small_arrays(int dtype, const void* coords, int n, int k, int32_t* rows, int32_t* m_out,
+                                cudaStream_t s);
 }  // namespace kd
 
 namespace {
 
 constexpr int NA_MAX_N = KD_NOALLOC_MAX_N;
-constexpr int NA_THREADS = 1024;
-constexpr int NA_KEYS_THREADS = 256;
-constexpr uint32_t NA_PAD = 0xffffffffu;  // index of a padding slot; sorts last
 
-// Workspace: KD_MAX_K key planes of NA_MAX_N words, then the status word
-// (nonzero once a NaN coordinate was seen).  The key planes are written in
-// full for the cloud before they are read; only the status word must start
-// at zero, and each call clears it on its stream before the first kernel.
-constexpr size_t NA_STATUS_WORD = (size_t)KD_MAX_K * NA_MAX_N;
-static __device__ __align__(256) uint64_t na_scratch[NA_STATUS_WORD + 32];
-
-template <typename T>
-__global__ void __launch_bounds__(NA_KEYS_THREADS) k_noalloc_keys(const T* __restrict__ coords, int n, int k,
-                                                                  uint64_t* __restrict__ ws) {
-    const int total = n * k;
-    int nan = 0;
-    for (int e = blockIdx.x * NA_KEYS_THREADS + threadIdx.x; e < total; e += gridDim.x * NA_KEYS_THREADS) {
-        const int i = e / k, d = e - i * k;
-        ws[(size_t)d * NA_MAX_N + i] = (uint64_t)kd::key_of(coords[e], &nan);
-    }
-    if (nan) atomicOr(reinterpret_cast<unsigned int*>(ws + NA_STATUS_WORD), 1u);
-}
-
-// Is (ka, ia) after (kb, ib) in super-key-d order?  ka, kb are the x_d keys.
-__device__ __forceinline__ bool na_after(uint64_t ka, uint32_t ia, uint64_t kb, uint32_t ib, int d, int k,
-                                         const uint64_t* __restrict__ ws) {
-    if (ka != kb) return ka > kb;
-    if (ia == NA_PAD || ib == NA_PAD) return ia > ib;
-    for (int r = 1; r < k; ++r) {
-        const int dd = d + r < k ? d + r : d + r - k;
-        const uint64_t xa = ws[(size_t)dd * NA_MAX_N + ia], xb = ws[(size_t)dd * NA_MAX_N + ib];
-        if (xa != xb) return xa > xb;
-    }
-    return ia > ib;
-}
-
-// Block d sorts the indices by super key d and writes the deduplicated order
-// to row d of out (row stride n).  Dynamic shared memory: npow2 keys (u64)
-// then npow2 indices (u32).
-__global__ void __launch_bounds__(NA_THREADS, 1) k_noalloc_sort(int n, int npow2, int k,
-                                                                 const uint64_t* __restrict__ ws,
-                                                                 int32_t* __restrict__ out, int32_t* m_out) {
-    extern __shared__ __align__(16) unsigned char na_smem[];
-    __shared__ int warp_tot[NA_THREADS / 32];
-    uint64_t* sk = reinterpret_cast<uint64_t*>(na_smem);
-    uint32_t* si = reinterpret_cast<uint32_t*>(sk + npow2);
-    const int d = blockIdx.x, tid = threadIdx.x;
-    if (*reinterpret_cast<const volatile unsigned int*>(ws + NA_STATUS_WORD)) {
-        if (d == 0 && tid == 0) *m_out = KD_ENAN;
-        return;
-    }
-    const uint64_t* xd = ws + (size_t)d * NA_MAX_N;
-    for (int p = tid; p < npow2; p += NA_THREADS) {
-        sk[p] = p < n ? xd[p] : ~0ull;
-        si[p] = p < n ? (uint32_t)p : NA_PAD;
-    }
-    __syncthreads();
-    // bitonic sort of npow2 slots; the order is total (ties end at the index)
-    for (int size = 2; size <= npow2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = tid; t < (npow2 >> 1); t += NA_THREADS) {
-                const int i = ((t & ~(stride - 1)) << 1) | (t & (stride - 1));
-                const int j = i + stride;
-                const bool up = (i & size) == 0;
-                const uint64_t ki = sk[i], kj = sk[j];
-                const uint32_t ii = si[i], ij = si[j];
-                if (na_after(ki, ii, kj, ij, d, k, ws) == up) {
-                    sk[i] = kj;
-                    sk[j] = ki;
-                    si[i] = ij;
-                    si[j] = ii;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    // Duplicate removal: a slot whose tuple equals its predecessor's goes.
-    // Each thread owns a contiguous chunk; a block scan of the kept counts
-    // gives the chunk's output offset.
-    const int chunk = (n + NA_THREADS - 1) / NA_THREADS;
-    const int b = tid * chunk < n ? tid * chunk : n;
-    const int e = b + chunk < n ? b + chunk : n;
-    auto kept = [&](int p) -> bool {
-        if (p == 0) return true;
-        if (sk[p] != sk[p - 1]) return true;
-        const uint32_t a = si[p], c = si[p - 1];
-        for (int r = 1; r < k; ++r) {
-            const int dd = d + r < k ? d + r : d + r - k;
-            if (ws[(size_t)dd * NA_MAX_N + a] != ws[(size_t)dd * NA_MAX_N + c]) return true;
-        }
-        return false;
-    };
-    int cnt = 0;
-    for (int p = b; p < e; ++p) cnt += kept(p);
-    const int lane = tid & 31, warp = tid >> 5;
-    int incl = cnt;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int w = warp_tot[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += v;
-        }
-        warp_tot[lane] = w;  // inclusive over warps
-    }
-    __syncthreads();
-    int pos = (warp ? warp_tot[warp - 1] : 0) + incl - cnt;
-    int32_t* row = out + (size_t)d * n;
-    for (int p = b; p < e; ++p)
-        if (kept(p)) row[pos++] = (int32_t)si[p];
-    if (d == 0 && tid == NA_THREADS - 1) *m_out = warp_tot[31];
-}
+// The coordinates of a call whose outputs overlap them.
+static __device__ __align__(256) uint64_t na_scratch[(size_t)KD_MAX_K * NA_MAX_N];
 
 // Per-device set-up, once per device with that device current: the address
-// of the static workspace and the shared-memory limit of the sort kernel.
+// of the static array.
 std::mutex na_mu;
 uint64_t* na_ws[64] = {};
 
@@ -172,9 +52,6 @@ cudaError_t noalloc_setup(int device, uint64_t** ws) {
     if (!na_ws[device]) {
         void* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, na_scratch);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_noalloc_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 NA_MAX_N * (int)(sizeof(uint64_t) + sizeof(uint32_t)));
         if (e != cudaSuccess) return e;
         na_ws[device] = static_cast<uint64_t*>(p);
     }
@@ -193,13 +70,9 @@ bool on_device_memory(const void* p, int device) {
     return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == device;
 }
 
-// Launch with the error returned by the launch call itself, so that an
-// error pending from the caller's earlier work is neither reported as this
-// call's nor cleared.
-template <typename... P>
-cudaError_t na_launch(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t s, P... args) {
-    void* argv[] = {static_cast<void*>(&args)...};
-    return cudaLaunchKernel(reinterpret_cast<const void*>(kern), dim3(grid), dim3(block), argv, smem, s);
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x < y + nb && y < x + na;
 }
 
 kd_status na_fail(kd_ctx* ctx, kd_status code, const std::string& msg) {
@@ -238,31 +111,15 @@ extern "C" kd_status kd_presort_noalloc(kd_ctx* ctx, const kd_cloud* cloud, int3
         e = cudaMemsetAsync(m_out, 0, sizeof(int32_t), s);
         return e == cudaSuccess ? KD_OK : na_fail(ctx, KD_EDEVICE, cudaGetErrorString(e));
     }
-    e = cudaMemsetAsync(ws + NA_STATUS_WORD, 0, sizeof(uint64_t), s);
-    if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, cudaGetErrorString(e));
-    const int ni = (int)n;
-    int grid = (int)((n * k + NA_KEYS_THREADS - 1) / NA_KEYS_THREADS);
-    if (grid > 1024) grid = 1024;
-    switch (cloud->dtype) {
-        case KD_I32:
-            e = na_launch(k_noalloc_keys<int32_t>, grid, NA_KEYS_THREADS, 0, s,
-                          static_cast<const int32_t*>(cloud->coords), ni, k, ws);
-            break;
-        case KD_I64:
-            e = na_launch(k_noalloc_keys<int64_t>, grid, NA_KEYS_THREADS, 0, s,
-                          static_cast<const int64_t*>(cloud->coords), ni, k, ws);
-            break;
-        default:
-            e = na_launch(k_noalloc_keys<float>, grid, NA_KEYS_THREADS, 0, s, static_cast<const float*>(cloud->coords),
-                          ni, k, ws);
-            break;
+    const void* coords = cloud->coords;
+    const size_t bytes = (size_t)n * k * (cloud->dtype == KD_I64 ? 8 : 4);
+    if (overlap(coords, bytes, arrays_out, (size_t)n * k * 4) || overlap(coords, bytes, m_out, 4)) {
+        e = cudaMemcpyAsync(ws, coords, bytes, cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, cudaGetErrorString(e));
+        coords = ws;
     }
+    e = kd::launch_small_arrays(cloud->dtype, coords, (int)n, k, arrays_out, m_out, s);
     if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, std::string("launch: ") + cudaGetErrorString(e));
-    int npow2 = 2;
-    while (npow2 < ni) npow2 <<= 1;
-    const size_t smem = (size_t)npow2 * (sizeof(uint64_t) + sizeof(uint32_t));
-    e = na_launch(k_noalloc_sort, k, NA_THREADS, smem, s, ni, npow2, k, (const uint64_t*)ws, arrays_out, m_out);
-    if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, std::string("launch: ") + cudaGetErrorString(e));
-    kd::ctx_add_launches(ctx, 2);
+    kd::ctx_add_launches(ctx, 1);
     return KD_OK;
 }
