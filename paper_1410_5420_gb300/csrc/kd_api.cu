@@ -126,6 +126,20 @@ struct TimedLaunch {
 
 struct Request;
 
+// Allocations of at most SMALL_BLOCK bytes are rounded up to a power of two
+// and kept when freed: a build of a few thousand tuples makes about 15
+// allocations, and the pool's calls took a third of its time.
+constexpr size_t SMALL_BLOCK = (size_t)1 << 20;
+constexpr int SMALL_CLASSES = 13;  // 256 bytes ... SMALL_BLOCK
+constexpr size_t SMALL_KEPT = (size_t)32 << 20;
+constexpr size_t PINNED_BYTES = (size_t)256 << 10;
+
+int small_class(size_t bytes) {
+    int c = 0;
+    while (((size_t)256 << c) < bytes) ++c;
+    return c;
+}
+
 }  // namespace
 
 struct kd_presorted {
@@ -136,7 +150,7 @@ struct kd_presorted {
     AllPlanes rec{};
     void* rec_block = nullptr;
     void* sel_keys = nullptr;  // median-selection build: k key planes in array-0 order
-    int64_t* d_m = nullptr;
+    int64_t* d_m = nullptr;  // the presort's info block, m first (InfoBlock)
     size_t bytes = 0;
 };
 
@@ -170,6 +184,10 @@ struct kd_ctx {
     std::string last_error;
     std::recursive_mutex mu;
     std::unordered_map<void*, size_t> sizes;
+    // freed blocks of at most SMALL_BLOCK bytes, by power of two, for the next
+    // allocations on this stream (at most SMALL_KEPT bytes in all)
+    std::vector<void*> small_free[SMALL_CLASSES];
+    size_t small_kept = 0;
     std::atomic<int64_t> launches{0};
     // kernel timing (debug bit 2)
     std::vector<TimedLaunch> timed;
@@ -182,9 +200,12 @@ struct kd_ctx {
     // copies of host outputs overlapping the finisher (created on first use)
     cudaStream_t copy_stream = nullptr;
     std::vector<cudaEvent_t> chunk_events;
-    // pinned host scratch for small uploads
-    void* pinned = nullptr;
-    size_t pinned_bytes = 0;
+    // page-locked host scratch for tables sent to the device and values read
+    // back (stage)
+    unsigned char* pinned = nullptr;
+    size_t pinned_used = 0;
+    bool staged = false;  // copies from it may still be in flight
+    std::vector<unsigned char> large;  // tables and read backs that exceed it
     // serving (kd_submit / kd_wait): worker threads, each with a sub-context
     kd_config cfg{};
     std::vector<std::thread> workers;
@@ -231,6 +252,15 @@ kd_status fail(kd_ctx* ctx, kd_status code, const std::string& msg) {
         if (_s != KD_OK) return _s;                                                                \
     } while (0)
 
+// The kept small blocks back to the pool.
+void small_release(kd_ctx* ctx) {
+    for (auto& v : ctx->small_free) {
+        for (void* p : v) cudaFreeAsync(p, ctx->stream);
+        v.clear();
+    }
+    ctx->small_kept = 0;
+}
+
 kd_status dev_alloc(kd_ctx* ctx, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return KD_OK;
@@ -238,11 +268,24 @@ kd_status dev_alloc(kd_ctx* ctx, void** p, size_t bytes) {
     if (ctx->budget && ctx->in_use + bytes > ctx->budget)
         return fail(ctx, KD_ENOMEM, "device memory budget exceeded (" + std::to_string(ctx->in_use + bytes) +
                                         " > " + std::to_string(ctx->budget) + " bytes)");
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        *p = nullptr;
-        return fail(ctx, KD_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
+    const bool small = bytes <= SMALL_BLOCK;
+    const int c = small ? small_class(bytes) : 0;
+    if (small && !ctx->small_free[c].empty()) {
+        *p = ctx->small_free[c].back();
+        ctx->small_free[c].pop_back();
+        ctx->small_kept -= (size_t)256 << c;
+    } else {
+        cudaError_t e = cudaMallocFromPoolAsync(p, small ? (size_t)256 << c : bytes, ctx->pool, ctx->stream);
+        if (e == cudaErrorMemoryAllocation && ctx->small_kept) {  // once more without the kept blocks
+            cudaGetLastError();
+            small_release(ctx);
+            e = cudaMallocFromPoolAsync(p, small ? (size_t)256 << c : bytes, ctx->pool, ctx->stream);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+            return fail(ctx, KD_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
+        }
     }
     ctx->in_use += bytes;
     ctx->sizes[*p] = bytes;
@@ -253,8 +296,17 @@ void dev_free(kd_ctx* ctx, void* p) {
     if (!p) return;
     auto it = ctx->sizes.find(p);
     if (it != ctx->sizes.end()) {
-        ctx->in_use -= it->second;
+        const size_t bytes = it->second;
+        ctx->in_use -= bytes;
         ctx->sizes.erase(it);
+        if (bytes <= SMALL_BLOCK) {
+            const int c = small_class(bytes);
+            if (ctx->small_kept + ((size_t)256 << c) <= SMALL_KEPT) {
+                ctx->small_free[c].push_back(p);  // its users so far precede the next user on the stream
+                ctx->small_kept += (size_t)256 << c;
+                return;
+            }
+        }
     }
     cudaFreeAsync(p, ctx->stream);
 }
@@ -363,15 +415,91 @@ bool pinned_host(const void* p) {
     return a.type == cudaMemoryTypeHost;
 }
 
-kd_status check_device_err(kd_ctx* ctx, int* d_err) {
-    int err = 0;
-    CK(cudaMemcpyAsync(&err, d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+// Host scratch for one copy, valid until the stream has completed it and the
+// next call starts (stage_begin): page-locked, so that copies to and from it
+// run without a staging copy of the driver's; large ones take pageable
+// memory (then the copy call itself has read it, or waits for it).
+unsigned char* stage(kd_ctx* ctx, size_t bytes) {
+    bytes = (bytes + 63) & ~(size_t)63;
+    if (!ctx->pinned && cudaMallocHost((void**)&ctx->pinned, PINNED_BYTES) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->pinned = nullptr;
+    }
+    if (!ctx->pinned || ctx->pinned_used + bytes > PINNED_BYTES) {
+        ctx->large.resize(std::max(ctx->large.size(), bytes));
+        return ctx->large.data();
+    }
+    unsigned char* p = ctx->pinned + ctx->pinned_used;
+    ctx->pinned_used += bytes;
+    return p;
+}
+
+// Start of a call: the scratch is free again (a call that failed may have
+// left copies from it in flight).
+void stage_begin(kd_ctx* ctx) {
+    if (ctx->staged) cudaStreamSynchronize(ctx->stream);
+    ctx->staged = false;
+    ctx->pinned_used = 0;
+}
+
+// bytes at dev, read back after everything on the stream.
+kd_status fetch(kd_ctx* ctx, const void* dev, size_t bytes, const unsigned char** host) {
+    unsigned char* h = stage(ctx, bytes);
+    CK(cudaMemcpyAsync(h, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    ctx->staged = false;
+    *host = h;
+    return KD_OK;
+}
+
+kd_status err_status(kd_ctx* ctx, int err) {
     if (err & ERR_NAN) return fail(ctx, KD_ENAN, "a float coordinate is NaN");
     if (err & ERR_TIMEOUT) return fail(ctx, KD_ETIMEOUT, "a device look-back wait exceeded its bound");
     if (err & ERR_INTERNAL) return fail(ctx, KD_EDEVICE, "internal consistency check failed on the device");
     return KD_OK;
 }
+
+kd_status check_device_err(kd_ctx* ctx, int* d_err) {
+    const unsigned char* h = nullptr;
+    CKS(fetch(ctx, d_err, sizeof(int), &h));
+    int err = 0;
+    memcpy(&err, h, sizeof(int));
+    return err_status(ctx, err);
+}
+
+// Host tables that go to the device in one allocation and one copy.
+struct Tables {
+    std::vector<std::pair<const void*, size_t>> parts;
+    std::vector<size_t> at;
+    size_t bytes = 0;
+    // Adds a table (src NULL: zeros); returns its number.
+    int add(const void* src, size_t n) {
+        at.push_back(bytes);
+        parts.push_back({src, n});
+        bytes += (n + 15) & ~(size_t)15;
+        return (int)parts.size() - 1;
+    }
+    // Sends the tables to dev (bytes of them).
+    kd_status send(kd_ctx* ctx, void* dev) {
+        unsigned char* h = stage(ctx, bytes);
+        for (size_t i = 0; i < parts.size(); ++i) {
+            if (parts[i].first) memcpy(h + at[i], parts[i].first, parts[i].second);
+            else memset(h + at[i], 0, parts[i].second);
+        }
+        ctx->staged = true;
+        CK(cudaMemcpyAsync(dev, h, bytes, cudaMemcpyHostToDevice, ctx->stream));
+        return KD_OK;
+    }
+};
+
+// What the host reads back of a presort: the head of its handle's info
+// block, followed by the kept tuples of every cloud (32-bit each).
+struct InfoBlock {
+    int64_t m;             // kept tuples
+    int64_t n;             // tuples
+    int32_t err, pad[3];   // error bits
+    uint32_t run_meta[4];  // of launch_run_stats
+};
 
 size_t dtype_size(int dtype) { return dtype == KD_I64 ? 8 : 4; }
 
@@ -447,9 +575,10 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
 
     // persistent (handle-owned) allocations
     void* p = nullptr;
-    CKS(dev_alloc(ctx, &p, sizeof(int64_t)));
+    stage_begin(ctx);
+    CKS(dev_alloc(ctx, &p, sizeof(InfoBlock) + (((size_t)count * 4 + 15) & ~(size_t)15)));
     H->d_m = (int64_t*)p;
-    CK(cudaMemsetAsync(H->d_m, 0, sizeof(int64_t), s));
+    InfoBlock* const d_info = (InfoBlock*)p;
     H->M = 0;
     H->m_c.assign(count, 0);
     H->m_off.assign(count + 1, 0);
@@ -487,6 +616,19 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     } guard{ctx, H.get()};
 
     Scratch S(ctx);
+    {
+        InfoBlock info{};
+        info.n = N;
+        std::vector<int32_t> nc32(count);
+        for (int i = 0; i < count; ++i) nc32[i] = (int32_t)H->n_c[i];
+        Tables t;
+        t.add(&info, sizeof(info));
+        t.add(nc32.data(), (size_t)count * 4);
+        CKS(t.send(ctx, d_info));
+    }
+    int* const d_err = &d_info->err;
+    int64_t* const d_n = &d_info->n;
+    int32_t* const mcloud = (int32_t*)(d_info + 1);
     // One cloud small enough for a block per super key: two launches and one
     // read back instead of about 25 and three.  Whole builds (float32, k = 3),
     // digit passes over the whole GPU against this: 256 tuples 410 -> 153 us,
@@ -500,11 +642,8 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             x = cb;
         }
         uint32_t* work = nullptr;
-        int* d_err = nullptr;
         if (all_arrays) CKS(S.get(&work, small_presort_words((int)N, k) * 4));
         else CKS(dev_alloc(ctx, &H->sel_keys, (size_t)k * pad4(N) * w + 16));
-        CKS(S.get(&d_err, 4));
-        CK(cudaMemsetAsync(d_err, 0, 4, s));
         {
             LaunchTimer lt(ctx, F_SORT, (double)N, nullptr, (double)k * (tsz + 4));
             ctx->launches += 1;  // the sort, then the records (or the key planes)
@@ -512,8 +651,12 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
                                     s));
         }
         ctx->inject_timeout = false;  // (no look-back to withhold a flag from)
-        CK(cudaMemcpyAsync(&H->M, H->d_m, 8, cudaMemcpyDeviceToHost, s));
-        CKS(check_device_err(ctx, d_err));
+        const unsigned char* h = nullptr;
+        InfoBlock info;
+        CKS(fetch(ctx, d_info, sizeof(info), &h));
+        memcpy(&info, h, sizeof(info));
+        CKS(err_status(ctx, info.err));
+        H->M = info.m;
         H->m_c[0] = H->m_off[1] = H->M;
         guard.armed = false;
         *out = H.release();
@@ -557,9 +700,7 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     }
     unsigned char* keys = nullptr;
     uint32_t *cloud_plane = nullptr, *hist = nullptr;
-    int64_t *cstart = nullptr, *d_n = nullptr;
-    int32_t* mcloud = nullptr;
-    int* d_err = nullptr;
+    int64_t* cstart = nullptr;
     // every plane and sort buffer: stride padded to 16 bytes plus 16 bytes of
     // slack, for the 16-byte-aligned bulk copies of the sort passes
     const int64_t NS = pad4(N);
@@ -572,19 +713,11 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         CKS(S.get(&cloud_plane, (size_t)NS * 4 + 16));
         CKS(S.get(&cstart, (size_t)(count + 1) * 8));
     }
-    CKS(S.get(&hist, (size_t)nrows * RADIX * 4));
+    CKS(S.get(&hist, (size_t)nrows * RADIX * 4 + 4));
     uint32_t *bases_all = nullptr, *bases_kept = nullptr;  // digit bases over all / kept tuples
     CKS(S.get(&bases_all, (size_t)nrows * RADIX * 4));
     CKS(S.get(&bases_kept, (size_t)nrows * RADIX * 4));
-    CKS(S.get(&d_n, 8));
-    CKS(S.get(&mcloud, (size_t)count * 4));
-    CKS(S.get(&d_err, 4));
     CK(cudaMemsetAsync(hist, 0, (size_t)nrows * RADIX * 4, s));
-    CK(cudaMemsetAsync(d_err, 0, 4, s));
-    std::vector<int32_t> nc32(count);
-    for (int i = 0; i < count; ++i) nc32[i] = (int32_t)H->n_c[i];
-    CK(cudaMemcpyAsync(d_n, &N, 8, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(mcloud, nc32.data(), (size_t)count * 4, cudaMemcpyHostToDevice, s));
     if (count > 1)
         CK(cudaMemcpyAsync(cstart, H->in_off.data(), (size_t)(count + 1) * 8, cudaMemcpyHostToDevice, s));
     if (up_chunks > 1) {
@@ -617,14 +750,21 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         LaunchTimer lt(ctx, F_OTHER, 0.0);
         CK(launch_digit_bases(hist, nrows, bases_all, s));
     }
-    std::vector<uint32_t> h_hist((size_t)nrows * RADIX);
-    CK(cudaMemcpyAsync(h_hist.data(), hist, h_hist.size() * 4, cudaMemcpyDeviceToHost, s));
-    CKS(check_device_err(ctx, d_err));  // synchronises
-    auto trivial = [&](int row) {
-        int nz = 0;
-        for (int b = 0; b < RADIX; ++b) nz += h_hist[(size_t)row * RADIX + b] != 0;
-        return nz <= 1;
-    };
+    // which digits are constant (the histograms end with the error bits)
+    std::vector<uint8_t> constant(nrows);
+    {
+        const unsigned char* h = nullptr;
+        CK(cudaMemcpyAsync(hist + (size_t)nrows * RADIX, d_err, 4, cudaMemcpyDeviceToDevice, s));
+        CKS(fetch(ctx, hist, (size_t)nrows * RADIX * 4 + 4, &h));  // synchronises
+        const uint32_t* h_hist = reinterpret_cast<const uint32_t*>(h);
+        CKS(err_status(ctx, (int)h_hist[(size_t)nrows * RADIX]));
+        for (int r = 0; r < nrows; ++r) {
+            int nz = 0;
+            for (int b = 0; b < RADIX; ++b) nz += h_hist[(size_t)r * RADIX + b] != 0;
+            constant[r] = nz <= 1;
+        }
+    }
+    auto trivial = [&](int row) { return constant[row] != 0; };
     auto row_of = [&](int plane, int digit) { return plane >= 0 ? plane * D + digit : k * D + digit; };
 
     // pass lists ------------------------------------------------------
@@ -745,16 +885,19 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     uint32_t* run_meta = nullptr;
     uint2 *run_range = nullptr, *cross_runs = nullptr;
     if (by_runs) {
-        CKS(S.get(&run_meta, 4 * sizeof(uint32_t)));
+        run_meta = d_info->run_meta;
         CKS(S.get(&run_range, run_tile_count(N) * sizeof(uint2)));
         CKS(S.get(&cross_runs, run_tile_count(N) * sizeof(uint2)));
         {
             LaunchTimer lt(ctx, F_TIES, (double)N, nullptr, (double)w);
             CK(launch_run_stats(key64, d_n, N, kbuf[kc], k - 1, run_range, cross_runs, run_meta, s));
         }
-        uint32_t meta[4] = {0, 0, 0, 0};
-        CK(cudaMemcpyAsync(meta, run_meta, sizeof(meta), cudaMemcpyDeviceToHost, s));
-        CKS(check_device_err(ctx, d_err));  // synchronises
+        const unsigned char* h = nullptr;
+        InfoBlock info;
+        CKS(fetch(ctx, d_info, sizeof(info), &h));  // synchronises
+        memcpy(&info, h, sizeof(info));
+        CKS(err_status(ctx, info.err));
+        const uint32_t* meta = info.run_meta;
         // ordering the runs by compares costs sum(L^2) over the long ones;
         // above RUN_COST_PER_TUPLE per tuple the whole-key sort is cheaper
         const uint64_t cost = (uint64_t)meta[0] | ((uint64_t)meta[1] << 32);
@@ -971,11 +1114,13 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         }
     }
     // learn m ----------------------------------------------------------------
-    int64_t M = 0;
-    CK(cudaMemcpyAsync(&M, H->d_m, 8, cudaMemcpyDeviceToHost, s));
-    std::vector<int32_t> mc(count);
-    CK(cudaMemcpyAsync(mc.data(), mcloud, (size_t)count * 4, cudaMemcpyDeviceToHost, s));
-    CKS(check_device_err(ctx, d_err));
+    const unsigned char* h_info = nullptr;
+    CKS(fetch(ctx, d_info, sizeof(InfoBlock) + (size_t)count * 4, &h_info));
+    InfoBlock info;
+    memcpy(&info, h_info, sizeof(info));
+    CKS(err_status(ctx, info.err));
+    const int32_t* mc = reinterpret_cast<const int32_t*>(h_info + sizeof(InfoBlock));
+    const int64_t M = info.m;
     H->M = M;
     int64_t acc = 0;
     for (int i = 0; i < count; ++i) {
@@ -1077,9 +1222,7 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
     }
     if (M == 0) return KD_OK;
     Scratch S(ctx);
-    int* d_err = nullptr;
-    CKS(S.get(&d_err, 4));
-    CK(cudaMemsetAsync(d_err, 0, 4, s));
+    stage_begin(ctx);
     // subtree size finished on chip (a power of two in [1024, 4096]) and
     // level-step tile (1024 or 2048 positions; a tile may touch at most 4
     // segments, so segments above the finisher need at least tile / 3):
@@ -1307,16 +1450,20 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
         job_off.push_back(flat.size());
         flat.insert(flat.end(), v.begin(), v.end());
     }
-    CloudDev* d_cd = nullptr;
-    int64_t *d_prefix = nullptr, *d_uprefix = nullptr;
-    LevelJob* d_jobs = nullptr;
+    Tables tb;
+    const int t_err = tb.add(nullptr, 4), t_cd = tb.add(cd.data(), sizeof(CloudDev) * count),
+              t_prefix = tb.add(top_prefix.data(), sizeof(int64_t) * (count + 1)),
+              t_uprefix = tb.add(unit_prefix.data(), sizeof(int64_t) * (count + 1)),
+              t_jobs = tb.add(flat.data(), sizeof(LevelJob) * flat.size());
+    unsigned char* d_tb = nullptr;
+    CKS(S.get(&d_tb, tb.bytes));
+    CKS(tb.send(ctx, d_tb));
+    int* const d_err = (int*)(d_tb + tb.at[t_err]);
+    CloudDev* const d_cd = (CloudDev*)(d_tb + tb.at[t_cd]);
+    int64_t* const d_prefix = (int64_t*)(d_tb + tb.at[t_prefix]);
+    int64_t* const d_uprefix = (int64_t*)(d_tb + tb.at[t_uprefix]);
+    LevelJob* const d_jobs = (LevelJob*)(d_tb + tb.at[t_jobs]);
     uint32_t* d_status = nullptr;
-    CKS(S.get(&d_cd, sizeof(CloudDev) * count));
-    CKS(S.get(&d_prefix, sizeof(int64_t) * (count + 1)));
-    CKS(S.get(&d_uprefix, sizeof(int64_t) * (count + 1)));
-    CK(cudaMemcpyAsync(d_cd, cd.data(), sizeof(CloudDev) * count, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(d_prefix, top_prefix.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(d_uprefix, unit_prefix.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice, s));
     // per step: tile counts, their segmented scan and head flags (no zeroing needed)
     size_t st_words = 0;
     int64_t max_ntiles = 0;
@@ -1326,8 +1473,6 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
     }
     if (small_steps) st_words = level_small_bytes(std::max(k, 2), max_ntiles, (int)step_jobs.size()) / 4;
     if (!flat.empty()) {
-        CKS(S.get(&d_jobs, sizeof(LevelJob) * flat.size()));
-        CK(cudaMemcpyAsync(d_jobs, flat.data(), sizeof(LevelJob) * flat.size(), cudaMemcpyHostToDevice, s));
         CKS(S.get(&d_status, st_words * 4));
         if (small_steps) CK(cudaMemsetAsync(d_status, 0, st_words * 4, s));
     }
@@ -1984,6 +2129,8 @@ kd_status kd_destroy(kd_ctx* ctx) {
             cudaEventDestroy(t.b);
         }
         for (auto e : ctx->event_pool) cudaEventDestroy(e);
+        small_release(ctx);
+        if (ctx->pinned) cudaFreeHost(ctx->pinned);
         if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
         if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
         if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
