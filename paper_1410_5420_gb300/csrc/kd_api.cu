@@ -62,14 +62,13 @@ int level_tile(int k);
 cudaError_t launch_shape(int32_t m, int k, int32_t* left, int32_t* right, uint8_t* dim, cudaStream_t s);
 cudaError_t launch_tune_cloud(int dtype, void* coords, int64_t count, uint64_t seed, cudaStream_t s);
 size_t sel_seg_bytes(int key64);
-int sel_finish_tile(int key64, int k);
+int sel_order_tile(int k);
 cudaError_t init_select_kernels();
 cudaError_t launch_sel_level(int key64, void* const* id, void* const* key, int cur, int k, int32_t m, int L,
                              int tile, void* segs, uint32_t* ghist, int32_t* gany, uint32_t* unresolved, int32_t* node,
                              int64_t in_off, int* err, cudaStream_t s, int round_begin, int round_end, int phase);
-cudaError_t launch_sel_finish(int key64, void* const* id, void* const* key, int cur, int k, int32_t m, int lam, int T,
-                              int32_t* node, int32_t* left, int32_t* right, uint8_t* dim, int64_t in_off, int* err,
-                              cudaStream_t s);
+cudaError_t launch_sel_order(int key64, void* const* id, void* const* key, int cur, int k, int32_t m, int lam,
+                             uint32_t** plane, uint32_t** perm, int* err, cudaStream_t s);
 bool level_tile_supported(int k, int tile);
 int level_status_stride(int k);
 cudaError_t launch_level_pass(int k, int tile, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
@@ -1601,8 +1600,8 @@ kd_status select_build(kd_ctx* ctx, kd_presorted* H, kd_tree* out) {
         keys[d] = (unsigned char*)H->sel_keys + (size_t)d * NS * w;
         keys[MAXK + d] = k1 + (size_t)d * NS * w;
     }
-    const int T = sel_finish_tile(key64, k);
-    const int stile = T >= 1024 ? 2048 : 1024;  // a level tile touches at most 4 segments of >= T tuples
+    const int T = sel_order_tile(k);
+    const int stile = 2048;  // a level tile touches at most 4 segments of >= 1024 tuples
     int lam = 0;
     while (max_seg(M, lam) > T) ++lam;
     void* segs = nullptr;
@@ -1662,21 +1661,28 @@ kd_status select_build(kd_ctx* ctx, kd_presorted* H, kd_tree* out) {
     cd.right = right;
     cd.dim = dim;
     const int64_t top = lam > 0 ? ((int64_t)1 << lam) - 1 : 0;
+    const int64_t prefix[2] = {0, top}, uprefix[2] = {0, (int64_t)1 << lam};
+    Tables tb;
+    const int t_cd = tb.add(&cd, sizeof(cd)), t_prefix = tb.add(prefix, sizeof(prefix)),
+              t_uprefix = tb.add(uprefix, sizeof(uprefix));
+    unsigned char* d_tb = nullptr;
+    CKS(S.get(&d_tb, tb.bytes));
+    CKS(tb.send(ctx, d_tb));
+    const CloudDev* d_cd = (const CloudDev*)(d_tb + tb.at[t_cd]);
     if (top > 0) {
-        CloudDev* d_cd = nullptr;
-        int64_t* d_prefix = nullptr;
-        CKS(S.get(&d_cd, sizeof(CloudDev)));
-        CKS(S.get(&d_prefix, 2 * sizeof(int64_t)));
-        const int64_t prefix[2] = {0, top};
-        CK(cudaMemcpyAsync(d_cd, &cd, sizeof(CloudDev), cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(d_prefix, prefix, sizeof(prefix), cudaMemcpyHostToDevice, s));
         LaunchTimer lt(ctx, F_TOP, (double)top, nullptr, 13.0);
-        CK(launch_top_nodes(d_cd, d_prefix, 1, top, k, H->perm0, nullptr, 0, s));
-        CK(cudaStreamSynchronize(s));  // the host copies of cd and prefix go out of scope
+        CK(launch_top_nodes(d_cd, (const int64_t*)(d_tb + tb.at[t_prefix]), 1, top, k, H->perm0, nullptr, 0, s));
     }
+    // every segment's orders, then the presorting build's finisher on them
     {
+        AllBufs bufs{};
+        uint32_t *plane[MAXK] = {}, *perm = nullptr;
         LaunchTimer lt(ctx, F_SELECT_FINISH, (double)M, nullptr, 0.0);
-        CK(launch_sel_finish(key64, ids, keys, cur, k, (int32_t)M, lam, T, node, left, right, dim, 0, d_err, s));
+        ctx->launches += 1;
+        CK(launch_sel_order(key64, ids, keys, cur, k, (int32_t)M, lam, plane, &perm, d_err, s));
+        for (int p = 0; p < k; ++p) bufs.p[p][0][0] = plane[p];
+        CK(launch_finish(bufs, k, (const int64_t*)(d_tb + tb.at[t_uprefix]), 1, 0, 1 << lam, d_cd, perm, T, d_err,
+                         nullptr, s));
     }
     CKS(check_device_err(ctx, d_err));
     if (!out->on_device) {

@@ -23,20 +23,21 @@
 //       greater -> the upper half, the median becomes the node.  Since the
 //       next level selects afresh, the halves need not keep an order: slots
 //       are claimed with atomics.
-//   k_sel_finish  a segment of at most SEL_T tuples is finished by one CTA in
-//       shared memory (4-bit selection rounds while sub-segments exceed 32
-//       tuples), then one warp per sub-segment of at most 32 tuples (each
-//       lane's rank in every super key from pairwise compares).
+//   k_sel_order  a segment of at most 2048 tuples (1024 for k > 4) is sorted
+//       by every super key in the shared memory of one block, which gives the
+//       presorting build's input for that segment alone; its on-chip
+//       finisher (k_finish) then builds the subtree.
 #include <cstdint>
 
-#include "kd_internal.cuh"
+#include "kd_block_sort.cuh"
 
 namespace kd {
 
 constexpr int SEL_THREADS = 256;
 constexpr int SEL_TILE = 2048;   // largest tile of the level kernels (positions)
 constexpr int SEL_IPT = SEL_TILE / SEL_THREADS;
-constexpr int SEL_FIN_SUBMAX = 64;  // sub-segments of a finisher unit while they exceed 32 tuples
+constexpr uint32_t KNONE = 0xffffffffu;
+constexpr int SEL_RUN = 32;  // longest run of equal sort words ordered by compares
 
 // Planes of the index array: tuple index and key words of each coordinate,
 // two buffers.
@@ -396,341 +397,156 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_move(const __grid_constant_
     }
 }
 
-// ------------------------------------------------------------- finisher
-// One CTA per segment of at most SEL_T tuples at level lam.  Shared memory
-// (dynamic): two buffers of (index, k key planes) for up to T elements,
-// then the segment word of every position (lo | hi << 12 | level << 24 |
-// done), the sub-segment index of every position, and the selection state of
-// the sub-segments.
-constexpr uint32_t SF_DONE = 0x80000000u;
+// ------------------------------------------------------ segment orders
+// One block per segment of level lam (at most 32 NW E tuples): the places
+// of its tuples in array 0 of the segment (super key 0 order) by every super
+// key, as the finisher of the presorting build reads them: plane[p][lo + i] =
+// lo + (place in array 0 of the i-th tuple by super key p), perm[lo + i] =
+// the i-th tuple by super key 0.
+//
+// Each order is a radix sort by the 16 leading differing bits of x_p (two
+// passes, where the finisher this replaces selected every median of every
+// level by 4-bit rounds over all keys), then runs of equal words by
+// super-key compares; where a run exceeds SEL_RUN, a radix sort by the whole
+// super key.  2^22 int64 tuples, k = 3: 0.23 ms, and 0.20 ms for the finisher,
+// against 3.77 ms.
+template <typename KW, int NW, int E>
+size_t sel_order_smem(int k) {
+    return (size_t)32 * NW * E * (k * sizeof(KW) + 4 + 2 + 2);
+}
 
-template <typename KW>
-struct SelSub {
-    int32_t lo, hi, pos;
-    uint32_t target;
-    uint32_t cnt[2];
-    int32_t start;  // first nibble of the super key the sub-segment's elements do not all share
-    uint32_t pad;
-    KW sand, sor;   // AND and OR of its leading key words
-    uint32_t hist[16];
-    int32_t any[16];
-    KW prefix[MAXK];
+struct SelOrder {
+    uint32_t* plane[MAXK];
+    uint32_t* perm;
 };
 
-template <typename KW>
-size_t sel_finish_smem(int k, int T) {
-    return (size_t)2 * T * (4 + (size_t)k * sizeof(KW)) + (size_t)T * 4 + (size_t)T + 16 +
-           sizeof(SelSub<KW>) * SEL_FIN_SUBMAX + 64;
-}
-
-template <typename KW>
-__device__ __forceinline__ void sf_emit(int32_t* node, int32_t* left, int32_t* right, uint8_t* dim, int32_t ulo,
-                                        int32_t a, int32_t b, int32_t c, uint32_t id, int64_t in_off, int d) {
-    const int32_t addr = ulo + c;
-    node[addr] = (int32_t)((int64_t)id - in_off);
-    if (left) left[addr] = a <= c - 1 ? ulo + child_mid(a, c - 1) : -1;
-    if (right) right[addr] = c + 1 <= b ? ulo + child_mid(c + 1, b) : -1;
-    if (dim) dim[addr] = (uint8_t)d;
-}
-
-template <typename KW>
-__global__ void __launch_bounds__(SEL_THREADS) k_sel_finish(const __grid_constant__ SelBufs<KW> bufs, int cur, int k,
-                                                            int32_t m, int lam, int T, int32_t* __restrict__ node,
-                                                            int32_t* __restrict__ left, int32_t* __restrict__ right,
-                                                            uint8_t* __restrict__ dim, int64_t in_off,
-                                                            int* __restrict__ err) {
-    extern __shared__ __align__(16) unsigned char sf_raw[];
-    __shared__ int s_first;  // smallest first nibble to select over the sub-segments of a level
+template <typename KW, int NW, int E>
+__global__ void __launch_bounds__(32 * NW) k_sel_order(const __grid_constant__ SelBufs<KW> bufs, int cur, int k,
+                                                       int32_t m, int lam, const __grid_constant__ SelOrder out,
+                                                       int* __restrict__ err) {
+    constexpr int NT = 32 * NW, CAP = NT * E, BITS = 16;
+    extern __shared__ __align__(16) unsigned char so_raw[];
+    KW* keys = reinterpret_cast<KW*>(so_raw);                         // [k][CAP]
+    uint32_t* s_key = reinterpret_cast<uint32_t*>(keys + (size_t)k * CAP);
+    uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_key + CAP);
+    uint16_t* s_inv = s_idx + CAP;                                    // place of every tuple in array 0
+    __shared__ __align__(16) uint16_t wc[NW][RADIX];
+    __shared__ uint32_t s_ws[32], s_w[4];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int32_t ulo, uhi;
-    segment_bounds(m, lam, blockIdx.x, ulo, uhi);
-    const int S = uhi - ulo + 1;
-    if (S <= 0) return;
-    if (S > T) {
+    const int base = warp * 32 * E + lane;
+    int32_t lo, hi;
+    segment_bounds(m, lam, blockIdx.x, lo, hi);
+    const int n = hi - lo + 1;
+    if (n <= 0) return;
+    if (n > CAP) {
         if (tid == 0) atomicOr(err, ERR_INTERNAL);
         return;
     }
-    // shared memory layout (see sel_finish_smem)
-    unsigned char* q = sf_raw;
-    KW* const keys0 = reinterpret_cast<KW*>(q);
-    q += (size_t)T * k * sizeof(KW);
-    uint32_t* const ids0 = reinterpret_cast<uint32_t*>(q);
-    q += (size_t)T * 4;
-    KW* const keys1 = reinterpret_cast<KW*>(q);
-    q += (size_t)T * k * sizeof(KW);
-    uint32_t* const ids1 = reinterpret_cast<uint32_t*>(q);
-    q += (size_t)T * 4;
-    // buffer bb of the element planes (selected, not indexed, to stay in registers)
-    auto KB = [&](int bb) { return bb ? keys1 : keys0; };
-    auto IB = [&](int bb) { return bb ? ids1 : ids0; };
-    uint32_t* segw = reinterpret_cast<uint32_t*>(q);
-    q += (size_t)T * 4;
-    uint8_t* subid = q;
-    q += ((size_t)T + 15) & ~(size_t)15;
-    SelSub<KW>* sub = reinterpret_cast<SelSub<KW>*>(q);
-    for (int i = tid; i < S; i += SEL_THREADS) {
-        ids0[i] = bufs.id[cur][ulo + i];
-        for (int d = 0; d < k; ++d) keys0[d * T + i] = bufs.key[cur][d][ulo + i];
-        segw[i] = (uint32_t)(S - 1) << 12;  // lo 0, hi S-1
-        subid[i] = 0;
-    }
+    for (int d = 0; d < k; ++d)
+        for (int i = tid; i < n; i += NT) keys[d * CAP + i] = bufs.key[cur][d][lo + i];
     __syncthreads();
-    int b = 0;  // buffer holding the elements
-    int l = 0;
-    bool bad = false;
-    constexpr int B = sizeof(KW);
-    const int nnib = 2 * k * B;
-    // ---- block levels: sub-segments of more than 32 tuples ----------------
-    for (; (S >> l) > 32; ++l) {
-        const int p = (lam + l) % k;
-        const int nsub = 1 << l;  // at most S / 32 <= SEL_FIN_SUBMAX
-        for (int s = tid; s < nsub; s += SEL_THREADS) {
-            int32_t lo = 0, hi = S - 1;
-            for (int f = l - 1; f >= 0; --f) {
-                const int32_t c = lo + ((hi - lo) >> 1);
-                if ((s >> f) & 1) lo = c + 1; else hi = c - 1;
+    uint32_t key[E], id[E];
+    auto load = [&](const KW* x, bool identity) {  // the current order; the bits in which its keys differ
+        KW a = ~(KW)0, r = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int o = base + e * 32;
+            id[e] = identity ? (uint32_t)o : (o < n ? s_idx[o] : 0u);
+            if (o < n) {
+                a &= x[id[e]];
+                r |= x[id[e]];
+                if (identity) s_idx[o] = (uint16_t)o;
             }
-            SelSub<KW>& U = sub[s];
-            U.lo = lo;
-            U.hi = hi;
-            U.pos = hi < lo ? -2 : -1;
-            U.target = hi < lo ? 0u : (uint32_t)((hi - lo) >> 1);
-            U.cnt[0] = U.cnt[1] = 0;
-            U.start = 0;
-            U.sand = ~(KW)0;
-            U.sor = 0;
-            for (int x = 0; x < 16; ++x) U.hist[x] = 0;
-            for (int j = 0; j < MAXK; ++j) U.prefix[j] = 0;
         }
-        if (tid == 0) s_first = 2 * B - 1;
-        __syncthreads();
-        // the leading nibbles every element of a sub-segment shares become
-        // its prefix; its selection starts at the first nibble where they differ
-        for (int i0 = 0; i0 < S; i0 += SEL_THREADS) {
-            const int i = i0 + tid;
-            const bool v = i < S && !(segw[i] & SF_DONE);
-            const uint32_t su = v ? subid[i] : 0xffffffffu;
-            const KW w = v ? KB(b)[p * T + i] : (KW)0;
-            const uint32_t peers = __match_any_sync(0xffffffffu, su);
-            KW a, o;
-            sel_warp_and_or(peers, w, a, o);
-            if (v && lane == __ffs(peers) - 1) sel_atomic_and_or(&sub[su].sand, &sub[su].sor, a, o);
+        return block_diff(a, r, s_w);
+    };
+    for (int p = 0; p < k; ++p) {
+        const KW* const xp = keys + p * CAP;
+        const KW differ = load(xp, true);
+        const int shift = word_shift<BITS>(differ);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int o = base + e * 32;
+            key[e] = o < n ? sort_word<BITS>(xp[o], shift) : 0u;
+            if (differ == 0 && o < n) s_key[o] = 0;  // (no pass writes the words)
         }
         __syncthreads();
-        for (int s = tid; s < nsub; s += SEL_THREADS) {
-            SelSub<KW>& U = sub[s];
-            if (U.pos != -1) continue;
-            const KW diff = U.sand ^ U.sor;
-            const int lead = diff == 0 ? 8 * B : (B == 8 ? __clzll((long long)diff) : __clz((int)(uint32_t)diff));
-            const int cn = lead / 4 < 2 * B ? lead / 4 : 2 * B - 1;
-            U.prefix[0] = cn == 0 ? (KW)0 : (U.sand & (~(KW)0 << (4 * (2 * B - cn))));
-            U.start = cn;
-            atomicMin(&s_first, cn);
+        if (differ != 0) {
+            for (int b = 0; b < BITS; b += 8) block_pass<NW, E>(key, id, b, n, s_key, s_idx, wc, s_ws);
         }
-        __syncthreads();
-        // selection: 4-bit rounds, most significant nibble first
-        for (int r4 = s_first; r4 < nnib; ++r4) {
-            const int r = r4 >> 1;
-            const int j = r / B;
-            const int sh = 8 * (B - 1 - r % B) + ((r4 & 1) ? 0 : 4);
-            int dj = p + j;
-            if (dj >= k) dj -= k;
-            for (int i0 = 0; i0 < S; i0 += SEL_THREADS) {  // whole warps, for the aggregation below
-                const int i = i0 + tid;
-                bool cand = i < S && !(segw[i] & SF_DONE);
-                const int su = cand ? subid[i] : 0;
-                cand = cand && sub[su].pos == -1 && r4 >= sub[su].start;
-                uint32_t nib = 0;
-                if (cand) {
-                    const SelSub<KW>& U = sub[su];
-                    for (int jj = 0; jj < j && cand; ++jj) {
-                        int d = p + jj;
-                        if (d >= k) d -= k;
-                        cand = KB(b)[d * T + i] == U.prefix[jj];
-                    }
-                    const KW wj = KB(b)[dj * T + i];
-                    if (cand && sh + 4 < 8 * B) cand = (wj >> (sh + 4)) == (U.prefix[j] >> (sh + 4));
-                    nib = (uint32_t)(wj >> sh) & 15u;
+        bool tie = false, lng = false;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int o = base + e * 32;
+            if (o + 1 >= n || s_key[o + 1] != s_key[o]) continue;
+            tie = true;
+            lng |= o + SEL_RUN < n && s_key[o + SEL_RUN] == s_key[o];
+        }
+        if (__syncthreads_or(lng)) {
+            for (int r = k - 1; r >= 0; --r) {  // least significant coordinate first
+                const KW* const x = keys + (p + r < k ? p + r : p + r - k) * CAP;
+                const KW df = load(x, r == k - 1);
+                __syncthreads();
+#pragma unroll
+                for (int w = 0; w < (int)sizeof(KW) * 8; w += 32) {
+                    if ((uint32_t)(df >> w) == 0) continue;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) key[e] = base + e * 32 < n ? (uint32_t)(x[id[e]] >> w) : 0u;
+                    for (int b = 0; b < 32; b += 8)
+                        if (((uint32_t)(df >> w) >> b) & 255u)
+                            block_pass<NW, E>(key, id, b, n, s_key, s_idx, wc, s_ws);
                 }
-                const uint32_t key = cand ? ((uint32_t)su << 4 | nib) : 0xffffffffu;
-                const uint32_t peers = __match_any_sync(0xffffffffu, key);
-                if (cand && lane == __ffs(peers) - 1) {
-                    atomicAdd(&sub[su].hist[nib], (uint32_t)__popc(peers));
-                    sub[su].any[nib] = i;
-                }
+                __syncthreads();
             }
-            __syncthreads();
-            bool open = false;
-            for (int s = tid; s < nsub; s += SEL_THREADS) {
-                SelSub<KW>& U = sub[s];
-                if (U.pos != -1) continue;
-                if (r4 < U.start) {  // this nibble is shared: already in the prefix
-                    open = true;
-                    continue;
-                }
-                uint32_t c = 0, hb = 0;
-                int bb = -1;
-                for (int x = 0; x < 16; ++x) {
-                    const uint32_t h = U.hist[x];
-                    if (bb < 0) {
-                        if (U.target < c + h) {
-                            bb = x;
-                            hb = h;
-                        } else {
-                            c += h;
+        } else if (__syncthreads_or(tie)) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int o = base + e * 32;
+                id[e] = 0;
+                key[e] = KNONE;  // the tuple's new place, if it is in a run
+                if (o >= n) continue;
+                const uint32_t x = s_key[o];
+                int s = o, f = o;
+                while (s > 0 && s_key[s - 1] == x) --s;
+                while (f + 1 < n && s_key[f + 1] == x) ++f;
+                if (s == f) continue;
+                const int i = s_idx[o];
+                id[e] = (uint32_t)i;
+                int c = s;
+                for (int y = s; y <= f; ++y) {
+                    if (y == o) continue;
+                    const int j = s_idx[y];
+                    for (int r = 0; r < k; ++r) {  // (no two super keys are equal)
+                        const KW* const z = keys + (p + r < k ? p + r : p + r - k) * CAP;
+                        if (z[j] != z[i]) {
+                            c += z[j] < z[i] ? 1 : 0;
+                            break;
                         }
                     }
-                    U.hist[x] = 0;
                 }
-                if (bb < 0) {
-                    bad = true;
-                    U.pos = -2;
-                    continue;
-                }
-                U.target -= c;
-                U.prefix[j] |= (KW)bb << sh;
-                if (hb == 1) {
-                    U.pos = U.any[bb];
-                } else if (r4 + 1 >= nnib) {
-                    bad = true;  // equal super keys after deduplication
-                    U.pos = -2;
-                } else {
-                    open = true;
-                }
+                key[e] = (uint32_t)c;
             }
-            if (!__syncthreads_or(open)) break;
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (key[e] != KNONE) s_idx[key[e]] = (uint16_t)id[e];
+            __syncthreads();
         }
-        // partition around the medians (the median becomes the node)
-        for (int i = tid; i < S; i += SEL_THREADS) {
-            if (segw[i] & SF_DONE) continue;
-            SelSub<KW>& U = sub[subid[i]];
-            if (U.pos < U.lo || U.pos > U.hi) {
-                bad = true;
-                continue;
-            }
-            const int32_t mid = U.lo + ((U.hi - U.lo) >> 1);
-            int c = 0;
-            for (int jj = 0; jj < k && c == 0; ++jj) {
-                int d = p + jj;
-                if (d >= k) d -= k;
-                const KW x = KB(b)[d * T + i], y = KB(b)[d * T + U.pos];
-                if (x != y) c = x < y ? -1 : 1;
-            }
-            if (c == 0) {
-                if (i != U.pos) bad = true;
-                sf_emit<KW>(node, left, right, dim, ulo, U.lo, U.hi, mid, IB(b)[i], in_off, p);
-                continue;
-            }
-            const int f = c > 0 ? 1 : 0;
-            const int32_t dst = (f ? mid + 1 : U.lo) + (int32_t)atomicAdd(&U.cnt[f], 1u);
-            if (f ? (dst <= mid || dst > U.hi) : (dst >= mid)) {
-                bad = true;
-                continue;
-            }
-            IB(b ^ 1)[dst] = IB(b)[i];
-            for (int d = 0; d < k; ++d) KB(b ^ 1)[d * T + dst] = KB(b)[d * T + i];
-        }
-        __syncthreads();
-        // the segment of every position at the next level
-        for (int i = tid; i < S; i += SEL_THREADS) {
-            if (segw[i] & SF_DONE) continue;
-            const int s = subid[i];
-            const int32_t lo = sub[s].lo, hi = sub[s].hi, mid = lo + ((hi - lo) >> 1);
-            if (i == mid) {
-                segw[i] |= SF_DONE;
-            } else if (i < mid) {
-                subid[i] = (uint8_t)(2 * s);
-                segw[i] = (uint32_t)lo | ((uint32_t)(mid - 1) << 12);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int o = base + e * 32;
+            if (o >= n) continue;
+            const int i = s_idx[o];
+            if (p == 0) {
+                s_inv[i] = (uint16_t)o;
+                out.perm[lo + o] = bufs.id[cur][lo + i];
+                out.plane[0][lo + o] = (uint32_t)(lo + o);
             } else {
-                subid[i] = (uint8_t)(2 * s + 1);
-                segw[i] = (uint32_t)(mid + 1) | ((uint32_t)hi << 12);
+                out.plane[p][lo + o] = (uint32_t)(lo + s_inv[i]);
             }
         }
-        b ^= 1;
-        __syncthreads();
+        __syncthreads();  // s_inv is written; s_idx and s_key are free
     }
-    // ---- warp levels: one warp per sub-segment of at most 32 tuples --------
-    // Each lane holds one tuple.  LESS_q (the lanes whose super key q is
-    // smaller) comes from pairwise compares; a lane's rank in its current
-    // sub-segment at a level with primary p is popc(LESS_p & SUB).
-    const int nsub = 1 << l;
-    const uint32_t lt = lanemask_lt();
-    for (int s = warp; s < nsub; s += SEL_THREADS / 32) {
-        int32_t lo = 0, hi = S - 1;
-        for (int f = l - 1; f >= 0; --f) {
-            const int32_t c = lo + ((hi - lo) >> 1);
-            if ((s >> f) & 1) lo = c + 1; else hi = c - 1;
-        }
-        const int n = hi - lo + 1;
-        if (n <= 0) continue;  // uniform per warp
-        if (n > 32) {
-            bad = true;
-            continue;
-        }
-        const bool in = lane < n;
-        KW w[MAXK];
-        uint32_t id = in ? IB(b)[lo + lane] : 0u;
-#pragma unroll
-        for (int d = 0; d < MAXK; ++d) w[d] = (in && d < k) ? KB(b)[d * T + lo + lane] : (KW)0;
-        uint32_t less[MAXK];
-#pragma unroll
-        for (int qd = 0; qd < MAXK; ++qd) less[qd] = 0;
-        // per source lane: which of its coordinate words are below / equal to
-        // this lane's (bit d); super key q then reads them rotated by q
-        const uint32_t full = (1u << k) - 1u;
-        for (int src = 0; src < n; ++src) {
-            uint32_t ltm = 0, eqm = 0;
-#pragma unroll
-            for (int d = 0; d < MAXK; ++d) {
-                if (d < k) {
-                    const KW o = __shfl_sync(0xffffffffu, w[d], src);
-                    ltm |= (o < w[d] ? 1u : 0u) << d;
-                    eqm |= (o == w[d] ? 1u : 0u) << d;
-                }
-            }
-#pragma unroll
-            for (int qd = 0; qd < MAXK; ++qd) {
-                if (qd < k) {
-                    const uint32_t ne = ~((eqm >> qd) | (eqm << (k - qd))) & full;
-                    const uint32_t lt = ((ltm >> qd) | (ltm << (k - qd))) & full;
-                    if (ne && ((lt >> (__ffs(ne) - 1)) & 1u)) less[qd] |= 1u << src;
-                }
-            }
-        }
-        uint32_t subm = __ballot_sync(0xffffffffu, in);
-        bool active = in;
-        int32_t mlo = lo, mhi = hi;
-        for (int lv = l; __any_sync(0xffffffffu, active); ++lv) {
-            if (active && (mhi < mlo || lv >= l + 32)) {  // inconsistent ranks: report, never spin
-                bad = true;
-                active = false;
-            }
-            const int p = (lam + lv) % k;
-            uint32_t lp = 0;
-#pragma unroll
-            for (int qd = 0; qd < MAXK; ++qd)
-                if (qd == p) lp = less[qd];
-            const int rank = __popc(lp & subm);
-            const int32_t c = mlo + ((mhi - mlo) >> 1);
-            const bool goL = active && rank < c - mlo;
-            const bool goR = active && rank > c - mlo;
-            if (active && rank == c - mlo) {
-                sf_emit<KW>(node, left, right, dim, ulo, mlo, mhi, c, id, in_off, p);
-                active = false;
-            }
-            const uint32_t Lm = __ballot_sync(0xffffffffu, goL);
-            const uint32_t Rm = __ballot_sync(0xffffffffu, goR);
-            if (goL) {
-                mhi = c - 1;
-                subm &= Lm;
-            } else if (goR) {
-                mlo = c + 1;
-                subm &= Rm;
-            }
-        }
-        (void)lt;
-    }
-    if (bad) atomicOr(err, ERR_INTERNAL);
 }
 
 // ------------------------------------------------------------ launchers
@@ -746,14 +562,9 @@ static SelBufs<KW> sel_bufs(void* const* id, void* const* key, int k) {
 
 size_t sel_seg_bytes(int key64) { return key64 ? sizeof(SelSeg<uint64_t>) : sizeof(SelSeg<uint32_t>); }
 
-// Largest finisher unit (2048, 1024 or 512 tuples) whose shared memory fits.
-int sel_finish_tile(int key64, int k) {
-    for (int T = 2048; T >= 512; T /= 2) {
-        const size_t b = key64 ? sel_finish_smem<uint64_t>(k, T) : sel_finish_smem<uint32_t>(k, T);
-        if (b <= 160 * 1024) return T;
-    }
-    return 512;
-}
+// Largest segment whose orders one block makes (and the presorting build's
+// finisher takes).
+int sel_order_tile(int k) { return k <= 4 ? 2048 : 1024; }
 
 template <typename KW>
 static cudaError_t sel_level(const SelBufs<KW>& B, int cur, int k, int32_t m, int L, int tile, void* segs,
@@ -787,7 +598,7 @@ static cudaError_t sel_level(const SelBufs<KW>& B, int cur, int k, int32_t m, in
 
 // One level of the selection build over every segment of level L, in tiles
 // of `tile` positions (a tile must touch at most LEVEL_NSMAX segments: with
-// segments of at least T tuples, 2048 for T >= 1024 and 1024 for T = 512).
+// segments of at least 1024 tuples, 2048).
 // phase 0: reset the segments' state; 3: the shared leading bytes of every
 // segment (*unresolved, as an int32, receives the smallest first byte to
 // select; it must hold the byte count before); 1: selection rounds
@@ -805,31 +616,41 @@ cudaError_t launch_sel_level(int key64, void* const* id, void* const* key, int c
                                node, in_off, err, s, round_begin, round_end, phase);
 }
 
-cudaError_t init_select_kernels() {
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_sel_finish<uint32_t>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+template <typename KW>
+static cudaError_t init_sel_order() {
+    // 160 KB covers every k: 2048 tuples up to k = 4, 1024 up to 8
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_sel_order<KW, 8, 8>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute((const void*)k_sel_finish<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 200 * 1024);
+        e = cudaFuncSetAttribute((const void*)k_sel_order<KW, 8, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 160 * 1024);
     return e;
 }
+cudaError_t init_select_kernels() {
+    const cudaError_t e = init_sel_order<uint32_t>();
+    return e == cudaSuccess ? init_sel_order<uint64_t>() : e;
+}
 
-// Finisher over the 2^lam units of level lam (each at most T tuples).
-cudaError_t launch_sel_finish(int key64, void* const* id, void* const* key, int cur, int k, int32_t m, int lam, int T,
-                              int32_t* node, int32_t* left, int32_t* right, uint8_t* dim, int64_t in_off, int* err,
-                              cudaStream_t s) {
-    if (m <= 0) return cudaSuccess;
+template <typename KW>
+static cudaError_t sel_order(const SelBufs<KW>& B, int cur, int k, int32_t m, int lam, const SelOrder& out, int* err,
+                             cudaStream_t s) {
     const unsigned units = 1u << lam;
-    if (key64) {
-        const size_t smem = sel_finish_smem<uint64_t>(k, T);
-        k_sel_finish<uint64_t><<<units, SEL_THREADS, smem, s>>>(sel_bufs<uint64_t>(id, key, k), cur, k, m, lam, T,
-                                                                node, left, right, dim, in_off, err);
-    } else {
-        const size_t smem = sel_finish_smem<uint32_t>(k, T);
-        k_sel_finish<uint32_t><<<units, SEL_THREADS, smem, s>>>(sel_bufs<uint32_t>(id, key, k), cur, k, m, lam, T,
-                                                                node, left, right, dim, in_off, err);
-    }
+    if (k <= 4) k_sel_order<KW, 8, 8><<<units, 256, sel_order_smem<KW, 8, 8>(k), s>>>(B, cur, k, m, lam, out, err);
+    else k_sel_order<KW, 8, 4><<<units, 256, sel_order_smem<KW, 8, 4>(k), s>>>(B, cur, k, m, lam, out, err);
     return cudaGetLastError();
+}
+
+// The orders of the 2^lam segments of level lam (each at most
+// sel_order_tile(k) tuples), in the buffer that does not hold the elements:
+// plane[p] over its key plane p, perm over its index plane.
+cudaError_t launch_sel_order(int key64, void* const* id, void* const* key, int cur, int k, int32_t m, int lam,
+                             uint32_t** plane, uint32_t** perm, int* err, cudaStream_t s) {
+    if (m <= 0) return cudaSuccess;
+    SelOrder out{};
+    for (int p = 0; p < k; ++p) plane[p] = out.plane[p] = static_cast<uint32_t*>(key[(cur ^ 1) * MAXK + p]);
+    *perm = out.perm = static_cast<uint32_t*>(id[cur ^ 1]);
+    if (key64) return sel_order<uint64_t>(sel_bufs<uint64_t>(id, key, k), cur, k, m, lam, out, err, s);
+    return sel_order<uint32_t>(sel_bufs<uint32_t>(id, key, k), cur, k, m, lam, out, err, s);
 }
 
 }  // namespace kd

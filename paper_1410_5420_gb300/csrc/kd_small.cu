@@ -11,7 +11,7 @@
 // kd_presort_noalloc is the first of them alone.
 #include <cstdint>
 
-#include "kd_internal.cuh"
+#include "kd_block_sort.cuh"
 
 namespace kd {
 
@@ -23,84 +23,6 @@ template <typename T>
 __device__ __forceinline__ auto small_key(T v) {
     int nan = 0;
     return key_of(v, &nan);
-}
-
-// One stable 8-bit LSD pass over the block's n elements, E rows of 32 per
-// warp: the element at place warp * 32 E + e * 32 + lane is (key[e], id[e]);
-// on return the arrays hold the new order and are reloaded from it.  Lanes
-// of equal digits are found by a ballot per digit bit (the match
-// instruction's cost grows with the distinct digits in a warp).
-template <int NW, int E>
-__device__ __forceinline__ void small_pass(uint32_t (&key)[E], uint32_t (&id)[E], int shift, int n, uint32_t* s_key,
-                                           uint16_t* s_idx, uint16_t (*wc)[RADIX], uint32_t* s_ws) {
-    constexpr int Q = NW / 8;  // threads per digit of the scan, each over 8 warps
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t lt = lanemask_lt();
-    reinterpret_cast<uint4*>(wc[warp])[lane] = make_uint4(0, 0, 0, 0);
-    __syncwarp();
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const bool in = warp * 32 * E + e * 32 + lane < n;
-        const uint32_t d = (key[e] >> shift) & 255u;
-        uint32_t peers = __ballot_sync(0xffffffffu, in);
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const uint32_t v = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-            peers &= (d >> b) & 1u ? v : ~v;
-        }
-        const uint32_t base = wc[warp][d];
-        id[e] |= (base + __popc(peers & lt)) << 16;  // the rank rides with the index (14 bits)
-        __syncwarp();
-        if (in && lane == 31 - __clz(peers)) wc[warp][d] = (uint16_t)(base + __popc(peers));
-        __syncwarp();
-    }
-    __syncthreads();
-    {
-        const int d = tid / Q, w0 = tid % Q * 8;
-        uint32_t c[8], sum = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            c[i] = wc[w0 + i][d];
-            sum += c[i];
-        }
-        uint32_t incl = sum;
-#pragma unroll
-        for (int o = 1; o < Q; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (tid % Q >= o) incl += y;
-        }
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, lane | (Q - 1));  // of digit d
-        uint32_t x = total;
-#pragma unroll
-        for (int o = Q; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_ws[warp] = x;
-        __syncthreads();
-        uint32_t run = __reduce_add_sync(0xffffffffu, lane < warp ? s_ws[lane] : 0u) + x - total + incl - sum;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            wc[w0 + i][d] = (uint16_t)run;
-            run += c[i];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        if (warp * 32 * E + e * 32 + lane < n) {
-            const uint32_t p = wc[warp][(key[e] >> shift) & 255u] + (id[e] >> 16);
-            s_key[p] = key[e];
-            s_idx[p] = (uint16_t)id[e];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int o = warp * 32 * E + e * 32 + lane;
-        key[e] = o < n ? s_key[o] : 0u;
-        id[e] = o < n ? s_idx[o] : 0u;
-    }
 }
 
 template <typename KW, int NW, int E>
@@ -121,13 +43,13 @@ struct SmallOut {
 };
 
 // Block d: the indices of n tuples (at most 32 NW E) by super key d.  First a
-// stable radix sort by x_d alone, over the bytes that differ (64-bit keys one
-// 32-bit word at a time); then runs of equal x_d are ordered by the other
-// coordinates and the index by compares, or, where a run exceeds SMALL_RUN,
-// everything is sorted again by the whole super key, least significant
-// coordinate first.  Bound by shared-memory latency and issue on its one SM;
-// 16384 float32 tuples of k = 3: 85 us for the three arrays (a bitonic sort
-// with super-key compares took 284), 42% of issue slots.
+// stable radix sort by the leading bits of x_d (16, or 24 above 2048
+// tuples); then runs of equal words are ordered by the super key and the
+// index by compares, or, where a run exceeds SMALL_RUN, everything is sorted
+// again by the whole super key, least significant coordinate first, over
+// the bytes that differ.  Bound by shared-memory latency and issue on its
+// one SM; 16384 float32 tuples of k = 3: 83 us for the three arrays (a bitonic
+// sort with super-key compares took 284).
 template <typename T, typename KW, int NW, int E>
 __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__ coords, int n, int k,
                                                            const SmallOut out) {
@@ -137,7 +59,8 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
     KW* s_full = reinterpret_cast<KW*>(ssm);                                  // ... then x_d in its order
     uint16_t* s_idx = reinterpret_cast<uint16_t*>(ssm + sizeof(KW) * NT * E);
     __shared__ __align__(16) uint16_t wc[NW][RADIX];
-    __shared__ uint32_t s_ws[32], s_and[2], s_or[2];
+    __shared__ uint32_t s_ws[32], s_w[4];
+    constexpr int BITS = NT * E <= 2048 ? 16 : 24;
     const int d = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int base = warp * 32 * E + lane;  // place of row 0's element
     if constexpr (sizeof(T) == 4 && T(0.5) != T(0)) {  // floats
@@ -152,55 +75,40 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
         }
     }
     uint32_t key[E], id[E];
-    // stable sort of the current order (identity: the input's) by x_c
-    auto sort_by = [&](int c, bool identity) {
-        if (tid < 2) {
-            s_and[tid] = 0xffffffffu;
-            s_or[tid] = 0;
-        }
+    // loads the current order (identity: the input's) and returns the bits in
+    // which its x_c differ
+    auto load = [&](int c, bool identity) {
         KW a = ~(KW)0, r = 0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int o = base + e * 32;
             id[e] = identity ? (uint32_t)o : (o < n ? s_idx[o] : 0u);
-            key[e] = 0;
             if (o < n) {
                 const KW x = small_key(coords[(int64_t)id[e] * k + c]);
                 a &= x;
                 r |= x;
-                key[e] = (uint32_t)x;
+                if (identity) s_idx[o] = (uint16_t)o;
             }
         }
+        return block_diff(a, r, s_w);
+    };
+    // key[]: bits from `shift` up of the elements' x_c
+    auto words = [&](int c, int shift) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            key[e] = base + e * 32 < n ? (uint32_t)(small_key(coords[(int64_t)id[e] * k + c]) >> shift) : 0u;
+    };
+    // stable sort of the current order by the whole of x_c
+    auto sort_by = [&](int c, bool identity) {
+        const KW differ = load(c, identity);
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < (int)sizeof(KW) / 4; ++w) {
-            const uint32_t aw = __reduce_and_sync(0xffffffffu, (uint32_t)(a >> (32 * w)));
-            const uint32_t ow = __reduce_or_sync(0xffffffffu, (uint32_t)(r >> (32 * w)));
-            if (lane == 0) {
-                atomicAnd(&s_and[w], aw);
-                atomicOr(&s_or[w], ow);
-            }
-        }
-        if (identity) {
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                if (base + e * 32 < n) s_idx[base + e * 32] = (uint16_t)(base + e * 32);
-        }
-        __syncthreads();
-        const uint32_t differ[2] = {s_and[0] ^ s_or[0], s_and[1] ^ s_or[1]};
-#pragma unroll
-        for (int w = 0; w < (int)sizeof(KW) / 4; ++w) {
-            if (differ[w] == 0) continue;
-            if (w > 0) {
-#pragma unroll
-                for (int e = 0; e < E; ++e)
-                    if (base + e * 32 < n)
-                        key[e] = (uint32_t)((uint64_t)small_key(coords[(int64_t)id[e] * k + c]) >> 32);
-            }
+        for (int w = 0; w < (int)sizeof(KW) * 8; w += 32) {
+            if ((uint32_t)(differ >> w) == 0) continue;
+            words(c, w);
             for (int b = 0; b < 32; b += 8)
-                if ((differ[w] >> b) & 255u) small_pass<NW, E>(key, id, b, n, s_key, s_idx, wc, s_ws);
+                if (((uint32_t)(differ >> w) >> b) & 255u) block_pass<NW, E>(key, id, b, n, s_key, s_idx, wc, s_ws);
         }
-        __syncthreads();  // (s_and and s_or are read before the next call resets them)
     };
     auto fill_keys = [&]() {  // s_full: x_d in the current order
 #pragma unroll
@@ -210,28 +118,39 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
         }
         __syncthreads();
     };
-    // tuple i before tuple j by x_{d+1}, ..., x_{d-1} and the index
+    // tuple i before tuple j by super key d and the index
     auto before = [&](int i, int j) {
-        for (int r = 1; r < k; ++r) {
+        for (int r = 0; r < k; ++r) {
             const int c = d + r < k ? d + r : d + r - k;
             const KW x = small_key(coords[(int64_t)i * k + c]), y = small_key(coords[(int64_t)j * k + c]);
             if (x != y) return x < y;
         }
         return i < j;
     };
-    sort_by(d, true);
+    const KW differ = load(d, true);
+    const int shift = word_shift<BITS>(differ);
+    if (differ != 0) {
+        words(d, shift);
+#pragma unroll
+        for (int e = 0; e < E; ++e) key[e] &= (1u << BITS) - 1u;
+        for (int b = 0; b < BITS; b += 8) block_pass<NW, E>(key, id, b, n, s_key, s_idx, wc, s_ws);
+    }
+    __syncthreads();
     fill_keys();
-    if (k > 1) {
+    auto word = [&](int o) { return sort_word<BITS>(s_full[o], shift); };
+    {
         bool tie = false, lng = false;
         for (int e = 0; e < E; ++e) {
             const int o = base + e * 32;
-            if (o + 1 >= n || s_full[o + 1] != s_full[o]) continue;
+            if (o + 1 >= n || word(o + 1) != word(o)) continue;
             tie = true;
-            lng |= o + SMALL_RUN < n && s_full[o + SMALL_RUN] == s_full[o];
+            lng |= o + SMALL_RUN < n && word(o + SMALL_RUN) == word(o);
         }
         if (__syncthreads_or(lng)) {
-            for (int r = k - 1; r >= 1; --r) sort_by(d + r < k ? d + r : d + r - k, r == k - 1);
-            sort_by(d, false);
+            for (int r = k - 1; r >= 0; --r) {
+                sort_by(d + r < k ? d + r : d + r - k, r == k - 1);
+                __syncthreads();
+            }
             fill_keys();
         } else if (__syncthreads_or(tie)) {
 #pragma unroll
@@ -240,10 +159,10 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
                 id[e] = 0;
                 key[e] = 0xffffffffu;  // the element's new place, if it is in a run
                 if (o >= n) continue;
-                const KW x = s_full[o];
+                const uint32_t x = word(o);
                 int s = o, f = o;
-                while (s > 0 && s_full[s - 1] == x) --s;
-                while (f + 1 < n && s_full[f + 1] == x) ++f;
+                while (s > 0 && word(s - 1) == x) --s;
+                while (f + 1 < n && word(f + 1) == x) ++f;
                 if (s == f) continue;
                 id[e] = s_idx[o];
                 int c = s;
@@ -255,6 +174,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
             for (int e = 0; e < E; ++e)
                 if (key[e] != 0xffffffffu) s_idx[key[e]] = (uint16_t)id[e];
             __syncthreads();
+            fill_keys();
         }
     }
     // a tuple equal to its predecessor goes (the smallest index comes first)
