@@ -120,7 +120,7 @@ kd_status kd_create(kd_ctx **out, const kd_config *cfg);
  * KD_EDEVICE, KD_ETIMEOUT.  Synchronises the stream three times: to read
  * the key-byte histograms (constant digits are skipped), the run lengths of
  * array 0 after its sort by x_0 (k >= 2: long or costly runs take the
- * whole-key sort), and m.  Clouds of at most 16384 tuples: once, to read m.
+ * whole-key sort), and m.  Clouds of at most 196608 tuples: once, to read m.
  */
 kd_status kd_presort(kd_ctx *ctx, const kd_cloud *cloud, kd_handle *out);
 
@@ -224,10 +224,9 @@ const char *kd_last_error(kd_ctx *ctx);
  * counterpart: it exists for callers that cannot let a library allocate
  * during a call, such as a process whose device memory is all owned by its
  * own allocator, or a latency-bound loop that cannot absorb a pool growth
- * or a device-wide synchronising free.  It works in shared memory; only a
- * call whose outputs overlap its coordinates uses a workspace, one static
- * device array of 1 MiB per device (KD_NOALLOC_MAX_N tuples of up to
- * KD_MAX_K coordinates).
+ * or a device-wide synchronising free.  Its workspace is one static device
+ * array of about 2 MiB per device, sized for KD_NOALLOC_MAX_N tuples of up
+ * to KD_MAX_K coordinates.
  *
  *  cloud       coordinates in device memory on the context's device
  *              (cloud->on_device must be 1), n <= KD_NOALLOC_MAX_N; larger
@@ -247,10 +246,10 @@ const char *kd_last_error(kd_ctx *ctx);
  * (KD_EINVAL) are found on the host before anything is enqueued.  The first
  * call on a device does a one-time set-up (the address of the static
  * workspace), so a caller that records its stream into a graph should make
- * one call before it starts recording.  Calls whose outputs overlap their
- * coordinates share the one workspace of the device: those whose work can
- * overlap on the device (different streams, or threads without ordering
- * between them) race and give wrong results; order them on one stream.
+ * one call before it starts recording.  Calls on a device share the one
+ * workspace: calls whose work can overlap on the device (different streams,
+ * or threads without ordering between them) race and give wrong results;
+ * order them on one stream.
  */
 #define KD_NOALLOC_MAX_N 16384
 kd_status kd_presort_noalloc(kd_ctx *ctx, const kd_cloud *cloud, int32_t *arrays_out, int32_t *m_out);

@@ -85,7 +85,8 @@ size_t finish_smem(int k, int smax);
 cudaError_t init_presort_kernels();
 cudaError_t init_small_kernels();
 int small_presort_max();
-size_t small_presort_words(int n, int k);
+size_t small_presort_words(int dtype, int n, int k, bool all_arrays);
+int small_sort_launches(int64_t n);
 cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, uint32_t* work, const AllPlanes& rec,
                                  uint32_t* perm0, void* sel_keys, int64_t sel_stride, int64_t* m_out, int* err,
                                  cudaStream_t s);
@@ -628,10 +629,12 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     int* const d_err = &d_info->err;
     int64_t* const d_n = &d_info->n;
     int32_t* const mcloud = (int32_t*)(d_info + 1);
-    // One cloud small enough for a block per super key: two launches and one
-    // read back instead of about 25 and three.  Whole builds (float32, k = 3),
-    // digit passes over the whole GPU against this: 256 tuples 410 -> 153 us,
-    // 2048 445 -> 194, 16384 483 -> 295.
+    // One cloud small enough to be sorted in blocks: two to four launches and
+    // one read back instead of about 25 and three.  Whole builds, digit passes
+    // over the whole GPU against this (float32, k = 3; int64, k = 6): 65536
+    // tuples 439 -> 259 and 745 -> 340 us, 131072 467 -> 320 and 803 -> 454,
+    // 196608 492 -> 408 and 881 -> 649; the merge of the chunks grows with the
+    // square of their number.
     if (count == 1 && N <= small_presort_max()) {
         const void* x = clouds[0].coords;
         if (!clouds[0].on_device) {
@@ -641,11 +644,11 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             x = cb;
         }
         uint32_t* work = nullptr;
-        if (all_arrays) CKS(S.get(&work, small_presort_words((int)N, k) * 4));
-        else CKS(dev_alloc(ctx, &H->sel_keys, (size_t)k * pad4(N) * w + 16));
+        CKS(S.get(&work, small_presort_words(dtype, (int)N, k, all_arrays) * 4));
+        if (!all_arrays) CKS(dev_alloc(ctx, &H->sel_keys, (size_t)k * pad4(N) * w + 16));
         {
             LaunchTimer lt(ctx, F_SORT, (double)N, nullptr, (double)k * (tsz + 4));
-            ctx->launches += 1;  // the sort, then the records (or the key planes)
+            ctx->launches += small_sort_launches(N);  // the sort's, then the records (or the key planes)
             CK(launch_small_presort(dtype, x, (int)N, k, work, H->rec, H->perm0, H->sel_keys, pad4(N), H->d_m, d_err,
                                     s));
         }

@@ -5,19 +5,21 @@
 // has already handed all device memory to its own allocator (a call would
 // then fail with KD_ENOMEM), or a latency-bound loop where a growing pool or
 // a cudaFree would stall the device for every stream.  kd_presort_noalloc
-// serves them for clouds of up to KD_NOALLOC_MAX_N tuples: its outputs go to
-// buffers the caller owns, and what it needs beside them fits the shared
-// memory of one thread block per super key (k_small_sort in kd_small.cu, one
-// launch).
+// serves them for clouds of up to KD_NOALLOC_MAX_N tuples: its only
+// workspace is one file-scope device array (NA_BYTES), set up once per
+// device, and its outputs go to buffers the caller owns.  The sorts are
+// those of kd_small.cu.
 //
 // It computes what kd_presort + kd_handle_arrays compute (Section 2.1: the
 // k index arrays sorted by the cyclic super keys x_d : x_{d+1} : ... and
 // duplicate tuples removed, the smallest index of a run surviving).
 //
-// The blocks read the coordinates until the last of them ends.  A call whose
-// outputs overlap its coordinates therefore first copies these to a
-// file-scope device array (1 MiB per device, set up once): two such calls on
-// one device whose work can overlap race on it.
+// The one static array per device is shared by every call on that device
+// that uses it (more than 2048 tuples, or outputs that overlap the
+// coordinates of a call that reads these while it writes, which it copies
+// there first): two such calls whose kernels can overlap (different streams,
+// or different threads without ordering between them) race on it.  Order
+// such calls on one stream.
 #include <mutex>
 #include <string>
 
@@ -30,30 +32,36 @@ int ctx_device(const kd_ctx* ctx);
 cudaStream_t ctx_stream(const kd_ctx* ctx);
 void ctx_set_error(kd_ctx* ctx, const std::string& msg);
 void ctx_add_launches(kd_ctx* ctx, int n);
-cudaError_t launch_small_arrays(int dtype, const void* coords, int n, int k, int32_t* rows, int32_t* m_out,
+cudaError_t launch_small_arrays(int dtype, const void* coords, int n, int k, void* work, int32_t* rows, int32_t* m_out,
                                 cudaStream_t s);
+size_t small_arrays_bytes(int n, int k);
+int small_sort_launches(int64_t n);
+bool small_reads_while_writing(int64_t n);
 }  // namespace kd
 
 namespace {
 
 constexpr int NA_MAX_N = KD_NOALLOC_MAX_N;
 
-// The coordinates of a call whose outputs overlap them.
-static __device__ __align__(256) uint64_t na_scratch[(size_t)KD_MAX_K * NA_MAX_N];
+// The chunked sort's workspace at the largest cloud of 64-bit keys (keys,
+// indices and places of k rows, a bit per place, a word per chunk), which
+// exceeds the coordinates of any cloud.
+constexpr size_t NA_BYTES = (size_t)KD_MAX_K * NA_MAX_N * (8 + 4 + 4) + (size_t)KD_MAX_K * NA_MAX_N / 8 + 1024;
+static __device__ __align__(256) unsigned char na_scratch[NA_BYTES];
 
 // Per-device set-up, once per device with that device current: the address
 // of the static array.
 std::mutex na_mu;
-uint64_t* na_ws[64] = {};
+unsigned char* na_ws[64] = {};
 
-cudaError_t noalloc_setup(int device, uint64_t** ws) {
+cudaError_t noalloc_setup(int device, unsigned char** ws) {
     std::lock_guard<std::mutex> lk(na_mu);
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     if (!na_ws[device]) {
         void* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, na_scratch);
         if (e != cudaSuccess) return e;
-        na_ws[device] = static_cast<uint64_t*>(p);
+        na_ws[device] = static_cast<unsigned char*>(p);
     }
     *ws = na_ws[device];
     return cudaSuccess;
@@ -103,7 +111,7 @@ extern "C" kd_status kd_presort_noalloc(kd_ctx* ctx, const kd_cloud* cloud, int3
     if (n > 0 && (!cloud->coords || !arrays_out || !on_device_memory(cloud->coords, dev) ||
                   !on_device_memory(arrays_out, dev)))
         return na_fail(ctx, KD_EINVAL, "coords and arrays_out must be non-null device memory on the context's device");
-    uint64_t* ws = nullptr;
+    unsigned char* ws = nullptr;
     e = noalloc_setup(dev, &ws);
     if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, std::string("set-up: ") + cudaGetErrorString(e));
     cudaStream_t s = kd::ctx_stream(ctx);
@@ -113,13 +121,15 @@ extern "C" kd_status kd_presort_noalloc(kd_ctx* ctx, const kd_cloud* cloud, int3
     }
     const void* coords = cloud->coords;
     const size_t bytes = (size_t)n * k * (cloud->dtype == KD_I64 ? 8 : 4);
-    if (overlap(coords, bytes, arrays_out, (size_t)n * k * 4) || overlap(coords, bytes, m_out, 4)) {
+    if (kd::small_reads_while_writing(n) &&
+        (overlap(coords, bytes, arrays_out, (size_t)n * k * 4) || overlap(coords, bytes, m_out, 4))) {
         e = cudaMemcpyAsync(ws, coords, bytes, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, cudaGetErrorString(e));
         coords = ws;
     }
-    e = kd::launch_small_arrays(cloud->dtype, coords, (int)n, k, arrays_out, m_out, s);
+    if (kd::small_arrays_bytes((int)n, k) > NA_BYTES) return na_fail(ctx, KD_EINVAL, "internal: workspace");
+    e = kd::launch_small_arrays(cloud->dtype, coords, (int)n, k, ws, arrays_out, m_out, s);
     if (e != cudaSuccess) return na_fail(ctx, KD_EDEVICE, std::string("launch: ") + cudaGetErrorString(e));
-    kd::ctx_add_launches(ctx, 1);
+    kd::ctx_add_launches(ctx, kd::small_sort_launches(n));
     return KD_OK;
 }

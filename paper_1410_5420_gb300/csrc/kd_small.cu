@@ -1,22 +1,33 @@
-// kd_small.cu -- presort of a small cloud, one thread block per super key.
+// kd_small.cu -- presort of a small cloud, one thread block per super key and
+// chunk of tuples.
 //
 // Section 2.1's presort (k index arrays sorted by the cyclic super keys,
 // duplicate tuples removed) for clouds of at most SMALL_MAX tuples, where a
 // sort pass over the whole GPU is all launch latency:
-//   k_small_sort  block d sorts the tuple indices by super key d in shared
-//                 memory and removes duplicates;
-//   k_small_recs  the rank records the build reads, from the arrays and
-//                 their inverses;
-//   k_small_keys  the key planes in array-0 order (median-selection build).
-// kd_presort_noalloc is the first of them alone.
+//   k_small_sort     at most SMALL_ONE tuples: block d sorts the tuple
+//                    indices by super key d in shared memory and removes
+//                    duplicates;
+//   k_small_chunks   more: block (c, d) sorts chunk c by super key d;
+//   k_small_merge    every tuple's place among all chunks, by binary search
+//                    in the others, and whether it is a duplicate;
+//   k_small_compact  the places without the duplicates';
+//   k_small_recs     the rank records the build reads, from the arrays and
+//                    their inverses;
+//   k_small_keys     the key planes in array-0 order (median-selection build).
+// kd_presort_noalloc is all but the last two: 16384 float32 tuples of k = 3 in
+// 29 us (in one block per super key 83; by a bitonic sort 284).
 #include <cstdint>
 
 #include "kd_block_sort.cuh"
 
 namespace kd {
 
-constexpr int SMALL_MAX = 16384;
-constexpr int SMALL_RUN = 32;  // longest run of equal x_d ordered by compares
+constexpr int SMALL_ONE = 2048;    // most tuples sorted by one block per super key
+constexpr int SMALL_MAX = 196608;  // most tuples sorted in chunks
+constexpr int SMALL_RUN = 32;      // longest run of equal x_d ordered by compares
+// Chunks of 2048 tuples up to 16384, 4096 up to 65536, 8192 above: a block's
+// sort takes longer with its chunk, the merge with the number of chunks.
+__host__ __device__ constexpr int small_chunk(int n) { return n <= 16384 ? 2048 : (n <= 65536 ? 4096 : 8192); }
 
 // Key of a coordinate (floats are checked for NaN before).
 template <typename T>
@@ -42,38 +53,42 @@ struct SmallOut {
     int* err;
 };
 
-// Block d: the indices of n tuples (at most 32 NW E) by super key d.  First a
-// stable radix sort by the leading bits of x_d (16, or 24 above 2048
-// tuples); then runs of equal words are ordered by the super key and the
+// Shared memory of one block's sort of at most 32 NW E tuples.
+template <typename KW, int NW, int E>
+struct SmallShared {
+    uint32_t* key;   // the word being sorted ...
+    KW* full;        // ... then x_d in its order (the same memory)
+    uint16_t* idx;   // the order
+    uint16_t (*wc)[RADIX];
+    uint32_t *ws, *w;  // 32 and 4 words
+};
+
+template <typename T>
+__device__ __forceinline__ bool small_nan(const T* __restrict__ coords, int count, int nt) {
+    bool nan = false;
+    if constexpr (sizeof(T) == 4 && T(0.5) != T(0))  // floats
+        for (int i = threadIdx.x; i < count; i += nt) nan |= coords[i] != coords[i];
+    return nan;
+}
+
+// The indices of n tuples (at most 32 NW E) by super key d.  First a stable
+// radix sort by the leading differing bits of x_d (16, or 24 above 1024
+// tuples: with 16, clustered floats leave runs too long for compares); then runs of equal words are ordered by the super key and the
 // index by compares, or, where a run exceeds SMALL_RUN, everything is sorted
 // again by the whole super key, least significant coordinate first, over
 // the bytes that differ.  Bound by shared-memory latency and issue on its
-// one SM; 16384 float32 tuples of k = 3: 83 us for the three arrays (a bitonic
-// sort with super-key compares took 284).
+// one SM.
 template <typename T, typename KW, int NW, int E>
-__global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__ coords, int n, int k,
-                                                           const SmallOut out) {
-    constexpr int NT = 32 * NW;
-    extern __shared__ __align__(16) unsigned char ssm[];
-    uint32_t* s_key = reinterpret_cast<uint32_t*>(ssm);                       // the word being sorted ...
-    KW* s_full = reinterpret_cast<KW*>(ssm);                                  // ... then x_d in its order
-    uint16_t* s_idx = reinterpret_cast<uint16_t*>(ssm + sizeof(KW) * NT * E);
-    __shared__ __align__(16) uint16_t wc[NW][RADIX];
-    __shared__ uint32_t s_ws[32], s_w[4];
-    constexpr int BITS = NT * E <= 2048 ? 16 : 24;
-    const int d = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+__device__ __forceinline__ void small_order(const T* __restrict__ coords, int n, int k, int d,
+                                            const SmallShared<KW, NW, E>& S) {
+    constexpr int NT = 32 * NW, BITS = NT * E <= 1024 ? 16 : 24;
+    uint32_t* const s_key = S.key;
+    KW* const s_full = S.full;
+    uint16_t* const s_idx = S.idx;
+    uint16_t(*const wc)[RADIX] = S.wc;
+    uint32_t *const s_ws = S.ws, *const s_w = S.w;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int base = warp * 32 * E + lane;  // place of row 0's element
-    if constexpr (sizeof(T) == 4 && T(0.5) != T(0)) {  // floats
-        bool nan = false;
-        for (int i = tid; i < n * k; i += NT) nan |= coords[i] != coords[i];
-        if (__syncthreads_or(nan)) {
-            if (d == 0 && tid == 0) {
-                if (out.err) atomicOr(out.err, ERR_NAN);
-                if (out.m32) *out.m32 = -6;
-            }
-            return;
-        }
-    }
     uint32_t key[E], id[E];
     // loads the current order (identity: the input's) and returns the bits in
     // which its x_c differ
@@ -177,6 +192,40 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
             fill_keys();
         }
     }
+}
+
+// Whether tuples i and j are equal.
+template <typename T>
+__device__ __forceinline__ bool small_equal(const T* __restrict__ coords, int k, int i, int j) {
+    for (int c = 0; c < k; ++c)
+        if (small_key(coords[(int64_t)i * k + c]) != small_key(coords[(int64_t)j * k + c])) return false;
+    return true;
+}
+
+#define SMALL_SHARED(KW, NW, E)                                                                                       \
+    extern __shared__ __align__(16) unsigned char ssm[];                                                              \
+    __shared__ __align__(16) uint16_t s_wc[NW][RADIX];                                                                \
+    __shared__ uint32_t s_ws[32], s_w[4];                                                                             \
+    uint16_t* const s_idx = reinterpret_cast<uint16_t*>(ssm + sizeof(KW) * 32 * NW * E);                              \
+    KW* const s_full = reinterpret_cast<KW*>(ssm);                                                                    \
+    const SmallShared<KW, NW, E> S{reinterpret_cast<uint32_t*>(ssm), s_full, s_idx, s_wc, s_ws, s_w}
+
+// Block d: super key d's array of at most 32 NW E tuples, complete.
+template <typename T, typename KW, int NW, int E>
+__global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__ coords, int n, int k,
+                                                           const SmallOut out) {
+    constexpr int NT = 32 * NW;
+    SMALL_SHARED(KW, NW, E);
+    const int d = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = warp * 32 * E + lane;
+    if (__syncthreads_or(small_nan(coords, n * k, NT))) {
+        if (d == 0 && tid == 0) {
+            if (out.err) atomicOr(out.err, ERR_NAN);
+            if (out.m32) *out.m32 = -6;
+        }
+        return;
+    }
+    small_order<T, KW, NW, E>(coords, n, k, d, S);
     // a tuple equal to its predecessor goes (the smallest index comes first)
     uint32_t keep[E], cnt = 0;
 #pragma unroll
@@ -184,11 +233,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
         const int o = base + e * 32;
         bool kp = o < n;
         if (kp && o > 0 && s_full[o - 1] == s_full[o]) {
-            const int i = s_idx[o - 1], j = s_idx[o];
-            bool same = true;
-            for (int c = 0; c < k && same; ++c)
-                same = small_key(coords[(int64_t)i * k + c]) == small_key(coords[(int64_t)j * k + c]);
-            kp = !same;
+            kp = !small_equal(coords, k, s_idx[o - 1], s_idx[o]);
         }
         keep[e] = __ballot_sync(0xffffffffu, kp);
         cnt += __popc(keep[e]);
@@ -214,6 +259,146 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
     }
 }
 
+// Workspace of the chunked sort (rows of n per super key).
+template <typename KW>
+struct SmallWork {
+    KW* key;         // x_d of every chunk's tuples in its order
+    uint32_t* id;    // their indices
+    uint32_t* raw;   // all indices in super-key-d order
+    uint32_t* dup;   // bit per place of raw: a duplicate (rows of `words`)
+    uint32_t* nan;   // per chunk: it holds a NaN
+    int words;
+};
+
+// Block (c, d): chunk c by super key d.
+template <typename T, typename KW, int NW, int E>
+__global__ void __launch_bounds__(32 * NW, 1) k_small_chunks(const T* __restrict__ coords, int n, int k,
+                                                             const SmallWork<KW> W) {
+    constexpr int CH = 32 * NW * E;
+    SMALL_SHARED(KW, NW, E);
+    const int c = blockIdx.x, d = blockIdx.y, tid = threadIdx.x;
+    const int first = c * CH, cnt = min(n - first, CH);
+    pdl_trigger();
+    const T* x = coords + (int64_t)first * k;
+    if (d == 0) {
+        const int nan = __syncthreads_or(small_nan(x, cnt * k, CH / E));
+        if (tid == 0) W.nan[c] = nan ? 1u : 0u;
+    }
+    for (int i = tid; i * 32 < cnt; i += CH / E) W.dup[(int64_t)d * W.words + first / 32 + i] = 0;
+    small_order<T, KW, NW, E>(x, cnt, k, d, S);
+    for (int i = tid; i < cnt; i += CH / E) {
+        W.key[(int64_t)d * n + first + i] = s_full[i];
+        W.id[(int64_t)d * n + first + i] = (uint32_t)(first + s_idx[i]);
+    }
+}
+
+// Row d: the place in super-key-d order of the tuple at place q of the
+// chunks' orders, and whether an equal tuple precedes it.  Equal x_d are
+// told apart by the other coordinates and the index (that of an earlier
+// chunk is smaller).
+constexpr int SMALL_WAYS = 4;  // chunks searched side by side
+template <typename T, typename KW>
+__global__ void __launch_bounds__(256) k_small_merge(const T* __restrict__ coords, int n, int k, int chunk,
+                                                     const SmallWork<KW> W) {
+    const int q = blockIdx.x * 256 + threadIdx.x, d = blockIdx.y;
+    pdl_wait();
+    pdl_trigger();
+    if (q >= n) return;
+    const KW* key = W.key + (int64_t)d * n;
+    const uint32_t* id = W.id + (int64_t)d * n;
+    const KW x = key[q];
+    const int me = (int)id[q], mc = q / chunk, nc = (n + chunk - 1) / chunk;
+    auto before = [&](int other) {  // equal x_d: the other tuple precedes this one
+        for (int r = 1; r < k; ++r) {
+            const int c = d + r < k ? d + r : d + r - k;
+            const KW a = small_key(coords[(int64_t)other * k + c]), b = small_key(coords[(int64_t)me * k + c]);
+            if (a != b) return a < b;
+        }
+        return other < me;
+    };
+    int rank = q - mc * chunk;
+    bool dup = rank > 0 && key[q - 1] == x && small_equal(coords, k, (int)id[q - 1], me);
+    for (int c0 = 0; c0 < nc; c0 += SMALL_WAYS) {
+        int pos[SMALL_WAYS], len[SMALL_WAYS];
+#pragma unroll
+        for (int u = 0; u < SMALL_WAYS; ++u) {
+            const int c = c0 + u;
+            pos[u] = 0;
+            len[u] = c < nc && c != mc ? min(n - c * chunk, chunk) : 0;
+        }
+        for (int step = chunk; step > 0; step >>= 1) {
+            KW y[SMALL_WAYS];
+#pragma unroll
+            for (int u = 0; u < SMALL_WAYS; ++u)
+                y[u] = pos[u] + step <= len[u] ? key[(c0 + u) * chunk + pos[u] + step - 1] : (KW)0;
+#pragma unroll
+            for (int u = 0; u < SMALL_WAYS; ++u)
+                if (pos[u] + step <= len[u] &&
+                    (y[u] < x || (y[u] == x && before((int)id[(c0 + u) * chunk + pos[u] + step - 1]))))
+                    pos[u] += step;
+        }
+#pragma unroll
+        for (int u = 0; u < SMALL_WAYS; ++u) {
+            rank += pos[u];
+            const int p = (c0 + u) * chunk + pos[u] - 1;  // the last tuple before this one
+            if (c0 + u < mc && pos[u] > 0 && key[p] == x) dup = dup || small_equal(coords, k, (int)id[p], me);
+        }
+    }
+    W.raw[(int64_t)d * n + rank] = (uint32_t)me;
+    if (dup) atomicOr(&W.dup[(int64_t)d * W.words + (rank >> 5)], 1u << (rank & 31));
+}
+
+// Row d: the kept tuples of 1024 places of raw to their places without the
+// duplicates before them.
+template <typename KW>
+__global__ void __launch_bounds__(256) k_small_compact(int n, int nchunks, const SmallWork<KW> W, const SmallOut out) {
+    __shared__ uint32_t s_sum[8], s_pre[32];
+    const int d = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int p0 = blockIdx.x * 1024, w0 = p0 / 32;
+    pdl_wait();
+    pdl_trigger();
+    if (__syncthreads_or(tid < nchunks && W.nan[tid])) {
+        if (d == 0 && blockIdx.x == 0 && tid == 0) {
+            if (out.err) atomicOr(out.err, ERR_NAN);
+            if (out.m32) *out.m32 = -6;
+        }
+        return;
+    }
+    const uint32_t* bits = W.dup + (int64_t)d * W.words;
+    uint32_t v = 0;  // duplicates before p0
+    for (int i = tid; i < w0; i += 256) v += __popc(bits[i]);
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) s_sum[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t own = (w0 + lane) * 32 < n ? __popc(bits[w0 + lane]) : 0u;
+        uint32_t x = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        const uint32_t pre = __reduce_add_sync(0xffffffffu, lane < 8 ? s_sum[lane] : 0u);
+        s_pre[lane] = pre + x - own;
+        if (lane == 31 && d == 0 && p0 + 1024 >= n) {
+            const uint32_t m = (uint32_t)n - (pre + x);
+            if (out.m64) *out.m64 = m;
+            if (out.m32) *out.m32 = (int32_t)m;
+        }
+    }
+    __syncthreads();
+    for (int r = 0; r < 4; ++r) {
+        const int w = r * 8 + warp, p = p0 + w * 32 + lane;
+        if (p >= n) break;
+        const uint32_t b = bits[w0 + w];
+        if ((b >> lane) & 1u) continue;
+        const uint32_t o = (uint32_t)p - (s_pre[w] + __popc(b & lanemask_lt()));
+        const uint32_t t = W.raw[(int64_t)d * n + p];
+        out.arr[d * out.arr_stride + o] = t;
+        if (out.inv) out.inv[d * out.inv_stride + t] = o;
+    }
+}
+
 // rec[d][p][i] = place in array p of the tuple at place i of array d (p != d;
 // array 0 also its own places), and perm0 = array 0.  Block row y: array d.
 __global__ void __launch_bounds__(256) k_small_recs(const int64_t* __restrict__ m_ptr, int k,
@@ -221,6 +406,7 @@ __global__ void __launch_bounds__(256) k_small_recs(const int64_t* __restrict__ 
                                                     int64_t stride, const __grid_constant__ AllPlanes rec,
                                                     uint32_t* __restrict__ perm0) {
     const int i = blockIdx.x * 256 + threadIdx.x, d = blockIdx.y;
+    pdl_wait();
     if (i >= *m_ptr) return;
     const uint32_t t = arr[d * stride + i];
     if (d == 0) perm0[i] = t;
@@ -244,6 +430,14 @@ __global__ void __launch_bounds__(256) k_small_keys(const int64_t* __restrict__ 
 // ------------------------------------------------------------ launchers
 int small_presort_max() { return SMALL_MAX; }
 
+// Words of the chunked sort's workspace for narrays super keys.
+static int64_t small_rows(int64_t n, int narrays) { return (int64_t)narrays * ((n + 3) & ~(int64_t)3); }
+static int small_dup_words(int n) { return (n + 31) / 32; }
+static size_t small_work_words(int dtype, int n, int narrays) {
+    const size_t rows = (size_t)small_rows(n, narrays);
+    return rows * ((dtype == 1 ? 2 : 1) + 2) + (size_t)narrays * small_dup_words(n) + 32;
+}
+
 template <typename T, typename KW, int NW, int E>
 static cudaError_t small_sort_as(const void* coords, int n, int k, int narrays, const SmallOut& out, cudaStream_t s) {
     // (the error of the launch call itself: one pending from earlier work is neither reported nor cleared)
@@ -254,40 +448,79 @@ static cudaError_t small_sort_as(const void* coords, int n, int k, int narrays, 
                             argv, small_smem<KW, NW, E>(), s);
 }
 
-// The fewest rows that hold n: a block of 8 warps up to 1024 tuples (its
-// barriers and scans are shorter), of 32 warps above.
+template <typename T, typename KW, int NW, int E>
+static cudaError_t small_chunks_as(const void* coords, int n, int k, int narrays, const SmallWork<KW>& W,
+                                   cudaStream_t s) {
+    const T* c = static_cast<const T*>(coords);
+    SmallWork<KW> w = W;
+    void* argv[] = {&c, &n, &k, &w};
+    const int ch = 32 * NW * E;
+    return cudaLaunchKernel(reinterpret_cast<const void*>(&k_small_chunks<T, KW, NW, E>),
+                            dim3((n + ch - 1) / ch, narrays), dim3(32 * NW), argv, small_smem<KW, NW, E>(), s);
+}
+
+// One block per super key up to SMALL_ONE tuples, of 8 warps up to 1024 (its
+// barriers and scans are shorter); chunks above (work: small_work_words).
 template <typename T, typename KW>
-static cudaError_t small_sort_of(const void* coords, int n, int k, int narrays, const SmallOut& out, cudaStream_t s) {
+static cudaError_t small_sort_of(const void* coords, int n, int k, int narrays, uint32_t* work, const SmallOut& out,
+                                 cudaStream_t s) {
     if (n <= 256) return small_sort_as<T, KW, 8, 1>(coords, n, k, narrays, out, s);
     if (n <= 1024) return small_sort_as<T, KW, 8, 4>(coords, n, k, narrays, out, s);
-    if (n <= 2048) return small_sort_as<T, KW, 32, 2>(coords, n, k, narrays, out, s);
-    if (n <= 4096) return small_sort_as<T, KW, 32, 4>(coords, n, k, narrays, out, s);
-    if (n <= 8192) return small_sort_as<T, KW, 32, 8>(coords, n, k, narrays, out, s);
-    return small_sort_as<T, KW, 32, 16>(coords, n, k, narrays, out, s);
+    if (n <= SMALL_ONE) return small_sort_as<T, KW, 32, 2>(coords, n, k, narrays, out, s);
+    const int64_t rows = small_rows(n, narrays);
+    SmallWork<KW> W;
+    W.key = reinterpret_cast<KW*>(work);
+    W.id = work + rows * (sizeof(KW) / 4);
+    W.raw = W.id + rows;
+    W.dup = W.raw + rows;
+    W.words = small_dup_words(n);
+    W.nan = W.dup + (int64_t)narrays * W.words;
+    const int chunk = small_chunk(n);
+    cudaError_t e = chunk == 2048 ? small_chunks_as<T, KW, 32, 2>(coords, n, k, narrays, W, s)
+                    : chunk == 4096 ? small_chunks_as<T, KW, 32, 4>(coords, n, k, narrays, W, s)
+                                    : small_chunks_as<T, KW, 32, 8>(coords, n, k, narrays, W, s);
+    if (e == cudaSuccess)
+        e = launch_dependent(k_small_merge<T, KW>, dim3((n + 255) / 256, narrays), dim3(256), 0, s, (const T*)coords, n,
+                             k, chunk, W);
+    if (e == cudaSuccess)
+        e = launch_dependent(k_small_compact<KW>, dim3((n + 1023) / 1024, narrays), dim3(256), 0, s, n,
+                             (n + chunk - 1) / chunk, W, out);
+    return e;
 }
 
-static cudaError_t small_sort(int dtype, const void* coords, int n, int k, int narrays, const SmallOut& out,
-                              cudaStream_t s) {
+static cudaError_t small_sort(int dtype, const void* coords, int n, int k, int narrays, uint32_t* work,
+                              const SmallOut& out, cudaStream_t s) {
     if (n < 1 || n > SMALL_MAX) return cudaErrorInvalidValue;
-    if (dtype == 0) return small_sort_of<int32_t, uint32_t>(coords, n, k, narrays, out, s);
-    if (dtype == 1) return small_sort_of<int64_t, uint64_t>(coords, n, k, narrays, out, s);
-    return small_sort_of<float, uint32_t>(coords, n, k, narrays, out, s);
+    if (dtype == 0) return small_sort_of<int32_t, uint32_t>(coords, n, k, narrays, work, out, s);
+    if (dtype == 1) return small_sort_of<int64_t, uint64_t>(coords, n, k, narrays, work, out, s);
+    return small_sort_of<float, uint32_t>(coords, n, k, narrays, work, out, s);
 }
 
-// kd_presort_noalloc: rows of n in out, m (or KD_ENAN) in m_out.
-cudaError_t launch_small_arrays(int dtype, const void* coords, int n, int k, int32_t* rows, int32_t* m_out,
+// Kernels launched by one sort.
+int small_sort_launches(int64_t n) { return n <= SMALL_ONE ? 1 : 3; }
+// Whether the sort reads the coordinates while it writes its outputs.
+bool small_reads_while_writing(int64_t n) { return n <= SMALL_ONE; }
+
+// kd_presort_noalloc: rows of n in out, m (or KD_ENAN) in m_out; work:
+// small_arrays_bytes(n, k) bytes.
+size_t small_arrays_bytes(int n, int k) { return n <= SMALL_ONE ? 0 : small_work_words(1, n, k) * 4; }
+cudaError_t launch_small_arrays(int dtype, const void* coords, int n, int k, void* work, int32_t* rows, int32_t* m_out,
                                 cudaStream_t s) {
     SmallOut o{};
     o.arr = reinterpret_cast<uint32_t*>(rows);
     o.arr_stride = n;
     o.m32 = m_out;
-    return small_sort(dtype, coords, n, k, k, o, s);
+    return small_sort(dtype, coords, n, k, k, static_cast<uint32_t*>(work), o, s);
 }
 
 // The handle of a small cloud: perm0, the rank records (rec, k >= 2) or, with
 // sel_keys, the key planes in array-0 order instead; m and the error bits.
-// work: small_presort_words(n, k) words.
-size_t small_presort_words(int n, int k) { return (size_t)2 * k * n; }
+// work: small_presort_words words (the sort's, then the arrays and their
+// inverses).
+size_t small_presort_words(int dtype, int n, int k, bool all_arrays) {
+    return (n <= SMALL_ONE ? 0 : (small_work_words(dtype, n, all_arrays ? k : 1) + 3) / 4 * 4) +
+           (all_arrays ? (size_t)2 * k * n : 0);
+}
 cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, uint32_t* work, const AllPlanes& rec,
                                  uint32_t* perm0, void* sel_keys, int64_t sel_stride, int64_t* m_out, int* err,
                                  cudaStream_t s) {
@@ -298,7 +531,7 @@ cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, ui
     const unsigned blocks = (unsigned)((n + 255) / 256);
     if (sel_keys) {
         o.arr = perm0;
-        cudaError_t e = small_sort(dtype, coords, n, k, 1, o, s);
+        cudaError_t e = small_sort(dtype, coords, n, k, 1, work, o, s);
         if (e != cudaSuccess) return e;
         if (dtype == 0)
             k_small_keys<int32_t, uint32_t><<<blocks, 256, 0, s>>>(m_out, k, (const int32_t*)coords, perm0,
@@ -311,24 +544,21 @@ cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, ui
                                                                  (uint32_t*)sel_keys, sel_stride);
         return cudaGetLastError();
     }
-    o.arr = work;
-    o.inv = work + (size_t)k * n;
-    cudaError_t e = small_sort(dtype, coords, n, k, k, o, s);
+    o.arr = work + small_presort_words(dtype, n, k, true) - (size_t)2 * k * n;
+    o.inv = o.arr + (size_t)k * n;
+    cudaError_t e = small_sort(dtype, coords, n, k, k, work, o, s);
     if (e != cudaSuccess) return e;
-    k_small_recs<<<dim3(blocks, k), 256, 0, s>>>(m_out, k, o.arr, o.inv, n, rec, perm0);
-    return cudaGetLastError();
+    return launch_dependent(k_small_recs, dim3(blocks, k), dim3(256), 0, s, (const int64_t*)m_out, k,
+                            (const uint32_t*)o.arr, (const uint32_t*)o.inv, (int64_t)n, rec, perm0);
 }
 
-template <typename T, typename KW, int NW, int E>
-static cudaError_t init_small_as() {
-    return cudaFuncSetAttribute((const void*)k_small_sort<T, KW, NW, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)small_smem<KW, NW, E>());
-}
 template <typename T, typename KW>
 static cudaError_t init_small_of() {
-    cudaError_t e = init_small_as<T, KW, 32, 4>();
-    if (e == cudaSuccess) e = init_small_as<T, KW, 32, 8>();
-    if (e == cudaSuccess) e = init_small_as<T, KW, 32, 16>();
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_small_chunks<T, KW, 32, 4>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem<KW, 32, 4>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void*)k_small_chunks<T, KW, 32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)small_smem<KW, 32, 8>());
     return e;
 }
 cudaError_t init_small_kernels() {

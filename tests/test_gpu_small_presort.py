@@ -1,8 +1,8 @@
-"""The presort of small clouds (one block per super key) through every entry
-point that uses it, against the oracle: the edges of its block sizes, runs
-of equal coordinates below and above the length ordered by compares, every
-type and dimension count, and outputs that overlap the coordinates.
-GPU only."""
+"""The presort of small clouds (one block per super key and chunk) through
+every entry point that uses it, against the oracle: the edges of its block
+and chunk sizes, runs of equal coordinates below and above the length ordered
+by compares, every type and dimension count, and outputs that overlap the
+coordinates.  GPU only."""
 import numpy as np
 import pytest
 
@@ -50,12 +50,19 @@ def test_block_size_edges(cuda_lib, n):
     _check(cuda_lib, kdgen.cloud_gmm(n, 2, n + 1))
 
 
+@pytest.mark.parametrize("n", [65536, 65537, 81921, 196608, 196609])
+def test_chunk_size_edges(cuda_lib, n):
+    _check(cuda_lib, kdgen.cloud_int_uniform(n, 3, 34, n, np.int64, dup_frac=0.01))
+    _check(cuda_lib, kdgen.cloud_gmm(n, 2, n + 1))
+
+
 @pytest.mark.parametrize("k", [1, 2, 4, 5, 8])
 @pytest.mark.parametrize("values", [1, 2, 40, 300, 3000])
 def test_runs_of_equal_coordinates(cuda_lib, k, values):
     """5000 tuples over few values per coordinate: runs of 5000, 2500, about
     125 (the whole super key is sorted), 17 and 2 (ordered by compares), with
-    many duplicates for small k; each type."""
+    many duplicates for small k, and equal tuples in different chunks; each
+    type."""
     rng = np.random.default_rng(k * 10000 + values)
     coords = rng.integers(0, values, (5000, k))
     _check(cuda_lib, (coords - values // 2).astype(np.int32))

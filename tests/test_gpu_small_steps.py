@@ -27,7 +27,7 @@ def _build(lib, coords, **cfg):
         ctx.close()
 
 
-@pytest.mark.parametrize("n", [1023, 1025, 2047, 2048, 2049, 4097, 20480, 65537])
+@pytest.mark.parametrize("n", [1025, 2049, 4097, 20480, 196609, 198656, 198657, 204799])
 @pytest.mark.parametrize("k", [2, 3, 4, 5, 8])
 def test_tile_edges(cuda_lib, n, k):
     coords = kdgen.cloud_int_uniform(n, k, 9, n + k, np.int64, dup_frac=0.01) if k % 2 else kdgen.cloud_gmm(n, k, n)
