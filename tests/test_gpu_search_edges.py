@@ -135,3 +135,33 @@ def test_region_offsets_over_chunks(cuda_lib, nq):
         cuda_lib.kd_index_destroy(ctx, ix)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("nq", [(1 << 17) - 1, 1 << 17, (1 << 19) + 3])
+def test_region_of_many_boxes(cuda_lib, nq):
+    """Boxes taken cell by cell, and boxes kept by the counting walk: none, up
+    to 16 and more than 16 tuples, and inverted boxes."""
+    import torch
+    rng = np.random.default_rng(nq)
+    coords = kdgen.cloud_gmm(70000, 3, 17)
+    centre = coords[rng.integers(0, len(coords), nq)]
+    half = (10.0 ** rng.uniform(-3, 0.7, (nq, 3))).astype(np.float32)
+    lo, hi = centre - half, centre + half
+    lo[::50], hi[::50] = hi[::50].copy(), lo[::50].copy()
+    ctx = cuda_lib.kd_create(0)
+    try:
+        ix, _ = _index(cuda_lib, ctx, coords)
+        L, H = torch.from_numpy(lo).cuda(), torch.from_numpy(hi).cuda()
+        offs, idx = (t.cpu().numpy() for t in cuda_lib.kd_region(ctx, ix, L, H))
+        pick = np.unique(np.concatenate([rng.integers(0, nq, 300), [0, nq - 1], np.argsort(np.diff(offs))[-20:]]))
+        ref = oracle.region(coords, lo[pick], hi[pick])
+        assert offs[-1] == len(idx) and max(len(r) for r in ref) > 16
+        for i, r in zip(pick, ref):
+            np.testing.assert_array_equal(np.sort(idx[offs[i]:offs[i + 1]]), r)
+        L[5, 1] = float("nan")
+        with pytest.raises(cuda_lib.KdError) as e:
+            cuda_lib.kd_region(ctx, ix, L, H)
+        assert e.value.code == -6
+        cuda_lib.kd_index_destroy(ctx, ix)
+    finally:
+        ctx.close()
