@@ -30,6 +30,7 @@
 #include <memory>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "kd_internal.cuh"
@@ -122,9 +123,10 @@ __global__ void __launch_bounds__(256) k_index_gather(const T* __restrict__ coor
 // while the rest of the GPU had finished.  Here candidates are kept by a
 // float distance and only the at most 32 survivors get the double one; the
 // boxes bound by the distance to the tuples themselves.  Eight neighbours of
-// each of 2^22 int64 tuples: 33.9 -> 8.1 ms, now bound by instruction issue
-// (71%, 1570 warp instructions per query); five of 100003 float32 queries
-// among 10^6 clustered tuples: 3.5-28 ms (by the cluster geometry) -> 0.65.
+// each of 2^22 int64 tuples: 33.9 -> 7.05 ms, now bound by instruction issue
+// (5.7 blocks, 4.7 nodes and 1.1 sorts per query); five of 100003 float32
+// queries among 10^6 clustered tuples: 3.5-28 ms (by the cluster geometry)
+// -> 0.6.
 //
 // Float distances.  a = the float sum of the squared float |p - q| differs
 // from the exact distance t by less than 2^-20 t (roundings of at most
@@ -157,22 +159,32 @@ struct KnnTree {
     int32_t nbox[BOX_LEVELS];
 };
 
-// |a - b| as a float, within 2^-23 of it.  (64 bits: from its two halves,
-// three roundings; the conversion instruction for 64-bit integers runs on
-// the FP64 pipe, which it kept 92% busy.)
-__device__ __forceinline__ float diff_f(int32_t a, int32_t b) {
-    return __uint2float_rn(a > b ? (uint32_t)a - (uint32_t)b : (uint32_t)b - (uint32_t)a);
-}
-__device__ __forceinline__ float diff_f(int64_t a, int64_t b) {
-    const uint64_t u = a > b ? (uint64_t)a - (uint64_t)b : (uint64_t)b - (uint64_t)a;
+// An unsigned difference as a float, within 2^-23 of it.  (64 bits: from the
+// two halves, three roundings; the conversion instruction for 64-bit
+// integers runs on the FP64 pipe, which it kept 92% busy.)
+__device__ __forceinline__ float udiff_f(uint32_t u) { return __uint2float_rn(u); }
+__device__ __forceinline__ float udiff_f(uint64_t u) {
     return fmaf(__uint2float_rn((uint32_t)(u >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)u));
 }
-__device__ __forceinline__ float diff_f(float a, float b) { return __fsub_rn(a, b); }
+// |a - b| as such a float (the float difference for floats).
+template <typename T>
+__device__ __forceinline__ float diff_f(T a, T b) {
+    using U = typename std::make_unsigned<T>::type;
+    return udiff_f(a > b ? (U)((U)a - (U)b) : (U)((U)b - (U)a));
+}
+template <>
+__device__ __forceinline__ float diff_f<float>(float a, float b) { return __fsub_rn(a, b); }
 
 // Distance of q from the interval [lo, hi], as diff_f.
 template <typename T>
 __device__ __forceinline__ float gap_f(T q, T lo, T hi) {
-    return q < lo ? diff_f(lo, q) : (q > hi ? diff_f(q, hi) : 0.0f);
+    using U = typename std::make_unsigned<T>::type;
+    const U below = (U)lo - (U)q, above = (U)q - (U)hi;
+    return udiff_f(q < lo ? below : (q > hi ? above : (U)0));
+}
+template <>
+__device__ __forceinline__ float gap_f<float>(float q, float lo, float hi) {
+    return q < lo ? __fsub_rn(lo, q) : (q > hi ? __fsub_rn(q, hi) : 0.0f);
 }
 
 __device__ __forceinline__ uint32_t knn_bound(float a) {
@@ -272,6 +284,13 @@ __device__ __forceinline__ void knn_block(const KnnTree<T>& X, KnnQuery<T, K>& Q
             uint32_t nk = pass ? key : KNN_NONE;
             int32_t na = a;
             warp_sort(nk, na);
+            if (Q.bound == KNN_OPEN && __shfl_sync(0xffffffffu, Q.key, 0) == KNN_NONE) {  // the list is empty
+                Q.key = nk;
+                Q.addr = na;
+                const uint32_t A0 = __shfl_sync(0xffffffffu, Q.key, Q.kn - 1);
+                if (A0 != KNN_NONE) Q.bound = knn_bound(__uint_as_float(A0));
+                return;
+            }
             nk = __shfl_xor_sync(0xffffffffu, nk, 31);
             na = __shfl_xor_sync(0xffffffffu, na, 31);
             const bool take = nk < Q.key;
@@ -384,8 +403,10 @@ __device__ __forceinline__ void knn_emit(const KnnTree<T>& X, const T* __restric
 // distances of all their candidates at once, one per lane: with kn = 8 and
 // one query at a time, 24 of the 32 lanes of every FP64 instruction idled
 // while that pipe was 89% busy.
+// Five blocks per SM (a few spills up to k = 4): 7.2 -> 7.05 ms for all eight
+// neighbours of 2^22 int64 tuples, 1.57 -> 1.37 for 2^20 float32; six: 7.3, 1.39.
 template <typename T, int K>
-__global__ void __launch_bounds__(KNN_THREADS) k_knn(const __grid_constant__ KnnTree<T> X,
+__global__ void __launch_bounds__(KNN_THREADS, K <= 4 ? 5 : 2) k_knn(const __grid_constant__ KnnTree<T> X,
                                                      const T* __restrict__ queries, int64_t nq, int kn, int width,
                                                      int32_t* __restrict__ idx_out, double* __restrict__ d_out,
                                                      int* __restrict__ err) {
