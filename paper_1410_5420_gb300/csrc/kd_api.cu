@@ -36,6 +36,15 @@ cudaError_t launch_sort_pass(int key64, const int64_t* count_ptr, int64_t max_co
 bool sort_pass_small(int64_t max_count);
 size_t sort_small_words(int64_t max_count);
 cudaError_t launch_digit_bases(const uint32_t* hist, int nrows, uint32_t* bases, cudaStream_t s);
+cudaError_t launch_word_sample(const void* keys, int64_t n, int k, int64_t stride, const uint32_t* hist, uint32_t* out,
+                               cudaStream_t s);
+cudaError_t launch_chain_next(int key64, const int64_t* count_ptr, int64_t max_count, const uint32_t* perm, int nplanes,
+                              const uint32_t* const* src, uint32_t* const* dst, const uint32_t* id_src,
+                              uint32_t* id_dst, const void* plane, uint32_t* words, int shift, int* err,
+                              cudaStream_t s);
+cudaError_t launch_word_runs(const int64_t* count_ptr, int64_t max_count, const uint32_t* words, const uint32_t* perm,
+                             const uint32_t* ids, const void* plane, uint32_t* out, int32_t* redo, int* err,
+                             cudaStream_t s);
 cudaError_t launch_pack_clouds(const PackDesc* d, int count, void* dst, cudaStream_t s);
 cudaError_t launch_gather(int key64, const int64_t* count_ptr, int64_t max_count, const void* plane,
                           const uint32_t* ids, void* out, int* err, cudaStream_t s);
@@ -107,6 +116,9 @@ namespace {
 // compares, unless the runs of more than 32 tuples would cost more than this
 // many compares per tuple (sum of their L^2 over n); then by the whole key.
 constexpr uint64_t RUN_COST_PER_TUPLE = 128;
+// Expected other tuples in a tuple's run of equal words (the sample's
+// estimate) up to which the chain sorts by words.
+constexpr double WORD_MATES = 4.0;
 
 enum Family {
     F_TRANSFORM = 0, F_SORT, F_DEDUP, F_RECORDS, F_LEVEL, F_FINISH, F_TOP, F_OTHER, F_GATHER,
@@ -497,7 +509,9 @@ struct Tables {
 struct InfoBlock {
     int64_t m;             // kept tuples
     int64_t n;             // tuples
-    int32_t err, pad[3];   // error bits
+    int32_t err;           // error bits
+    int32_t redo;          // a run of equal words was too long (k_word_runs)
+    int32_t pad[2];
     uint32_t run_meta[4];  // of launch_run_stats
 };
 
@@ -715,7 +729,7 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         CKS(S.get(&cloud_plane, (size_t)NS * 4 + 16));
         CKS(S.get(&cstart, (size_t)(count + 1) * 8));
     }
-    CKS(S.get(&hist, (size_t)nrows * RADIX * 4 + 4));
+    CKS(S.get(&hist, ((size_t)nrows * RADIX + 1 + k) * 4));  // then the error bits and the word samples
     uint32_t *bases_all = nullptr, *bases_kept = nullptr;  // digit bases over all / kept tuples
     CKS(S.get(&bases_all, (size_t)nrows * RADIX * 4));
     CKS(S.get(&bases_kept, (size_t)nrows * RADIX * 4));
@@ -752,12 +766,28 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         LaunchTimer lt(ctx, F_OTHER, 0.0);
         CK(launch_digit_bases(hist, nrows, bases_all, s));
     }
-    // which digits are constant (the histograms end with the error bits)
+    // The chain's sorts by words (see kd_presort.cu): 64-bit keys, or so many
+    // dimensions that the carried rank planes outweigh their gathers, and
+    // planes that L2 holds while they are gathered.  Whole builds, by keys
+    // against by words: int64 k = 3, 2^20 tuples 912 -> 901 us, 2^22 2272 ->
+    // 2092, 2^24 7809 -> 7668; k = 4, 2^19 834 -> 799; k = 6, 2^22 6346 ->
+    // 5328; float32 k = 4, 2^22 2550 -> 2564, k = 6, 2^20 1587 -> 1601, 2^21
+    // 2801 -> 2590, 2^22 4872 -> 4323.
+    const bool words_fit = count == 1 && all_arrays && N <= (int64_t)1 << 24 &&
+                           (key64 ? k >= 3 && (k - 2) * N >= (int64_t)1 << 20 : k >= 5 && N >= (int64_t)1 << 21);
+    if (words_fit && key64) {
+        LaunchTimer lt(ctx, F_OTHER, 0.0);
+        CK(launch_word_sample(keys, N, k, NS, hist, hist + (size_t)nrows * RADIX + 1, s));
+    }
+    bool by_words = words_fit;
+    // which digits are constant (the histograms end with the error bits and
+    // the word samples, whose collisions must leave a tuple about WORD_MATES
+    // others in its run of equal words)
     std::vector<uint8_t> constant(nrows);
     {
         const unsigned char* h = nullptr;
         CK(cudaMemcpyAsync(hist + (size_t)nrows * RADIX, d_err, 4, cudaMemcpyDeviceToDevice, s));
-        CKS(fetch(ctx, hist, (size_t)nrows * RADIX * 4 + 4, &h));  // synchronises
+        CKS(fetch(ctx, hist, ((size_t)nrows * RADIX + 1 + k) * 4, &h));  // synchronises
         const uint32_t* h_hist = reinterpret_cast<const uint32_t*>(h);
         CKS(err_status(ctx, (int)h_hist[(size_t)nrows * RADIX]));
         for (int r = 0; r < nrows; ++r) {
@@ -765,6 +795,10 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             for (int b = 0; b < RADIX; ++b) nz += h_hist[(size_t)r * RADIX + b] != 0;
             constant[r] = nz <= 1;
         }
+        // mates of a tuple in its run: 2 c N / sample^2
+        for (int d = 1; d < k && words_fit && key64; ++d)
+            by_words = by_words &&
+                       2.0 * h_hist[(size_t)nrows * RADIX + 1 + d] * (double)N <= WORD_MATES * 4096.0 * 4096.0;
     }
     auto trivial = [&](int row) { return constant[row] != 0; };
     auto row_of = [&](int plane, int digit) { return plane >= 0 ? plane * D + digit : k * D + digit; };
@@ -928,8 +962,8 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     // key buffer the chain's first sort reads) and, for 32-bit keys and
     // k >= 3, x_{k-2} (carried through that sort for the next one), both in
     // array-0 order, so neither needs a gather
-    const bool y_first = count == 1 && k >= 2 && all_arrays;
-    const bool y_second = y_first && k >= 3 && !key64;
+    bool y_first = count == 1 && k >= 2 && all_arrays && !by_words;
+    bool y_second = y_first && k >= 3 && !key64;
     unsigned char* y2c = nullptr;
     if (y_second) CKS(S.get(&y2c, (size_t)NS * w + 16));
     {
@@ -977,8 +1011,77 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         }
     }
     // chain: array d = stable sort of array d+1 by x_d (then cloud) --------
+    // by words: the source positions are the one payload, and the last pass
+    // (or k_word_runs) leaves them as rank plane d+1 of array d
+    auto chain_by_words = [&]() -> kd_status {
+        uint32_t* words = (uint32_t*)kbuf[0];
+        uint32_t* wbuf[2] = {(uint32_t*)kbuf[0], (uint32_t*)kbuf[1]};
+        const uint32_t* id = H->perm0;
+        // bytes of x_d's word: from `first`, as many as differ (inexact: three)
+        auto word_bytes = [&](int d, int* first) {
+            int top = D - 1;
+            while (top > 0 && trivial(row_of(d, top))) --top;
+            *first = top < 4 ? 0 : top - 2;
+            return top < 4 ? top + 1 : 3;
+        };
+        int first = 0;
+        word_bytes(k - 1, &first);
+        {
+            LaunchTimer lt(ctx, F_GATHER, 0.0, H->d_m, 8.0 + w);
+            CK(launch_chain_next(key64, H->d_m, N, nullptr, 0, nullptr, nullptr, id, nullptr, plane_ptr(k - 1), words,
+                                 8 * first, d_err, s));
+        }
+        std::vector<int> carried;  // rank planes of the previous array beside its own positions
+        for (int d = k - 1; d >= 1; --d) {
+            const int from = (d + 1) % k;
+            const int nb = word_bytes(d, &first);
+            const bool exact = first == 0;
+            uint32_t* const sorted = H->rec.p[d][from];
+            std::vector<int> digits;
+            for (int b = 0; b < nb; ++b)
+                if (!trivial(row_of(d, first + b))) digits.push_back(b);
+            if (digits.empty()) digits.push_back(0);
+            int wc = 0;
+            const uint32_t* src = nullptr;
+            for (size_t i = 0; i < digits.size(); ++i) {
+                const bool last = i + 1 == digits.size();
+                PayloadArgs pay{};
+                pay.n = 1;
+                pay.src[0] = src;
+                pay.dst[0] = last && exact ? sorted : pbuf[i & 1][0];
+                void* kdst = last && exact ? nullptr : (void*)wbuf[wc ^ 1];
+                LaunchTimer lt(ctx, F_SORT, 0.0, H->d_m, (kdst ? 8.0 : 4.0) + 8.0);
+                ctx->launches += pass_extra;  // count and scan kernels of the pass
+                CK(launch_sort_pass(0, H->d_m, N, wbuf[wc], kdst, pay,
+                                    bases_kept + (size_t)row_of(d, first + digits[i]) * RADIX, 8 * digits[i], status,
+                                    ++pass_no, d_err, s, ctx->spin_limit));
+                src = pay.dst[0];
+                wc ^= 1;
+            }
+            if (!exact) {
+                LaunchTimer lt(ctx, F_SORT, 0.0, H->d_m, 12.0);
+                CK(launch_word_runs(H->d_m, N, wbuf[wc], src, id, plane_ptr(d), sorted, &d_info->redo, d_err, s));
+            }
+            const uint32_t* gsrc[MAXK];
+            uint32_t* gdst[MAXK];
+            for (size_t j = 0; j < carried.size(); ++j) {
+                gsrc[j] = H->rec.p[from][carried[j]];
+                gdst[j] = H->rec.p[d][carried[j]];
+            }
+            uint32_t* const next_id = d > 1 ? (id == ibuf[0] ? ibuf[1] : ibuf[0]) : nullptr;
+            if (d > 1) word_bytes(d - 1, &first);
+            if (d > 1 || !carried.empty()) {
+                LaunchTimer lt(ctx, F_GATHER, 0.0, H->d_m, 4.0 + 8.0 * carried.size() + (d > 1 ? 12.0 + w : 0.0));
+                CK(launch_chain_next(key64, H->d_m, N, sorted, (int)carried.size(), gsrc, gdst, id, next_id,
+                                     d > 1 ? plane_ptr(d - 1) : nullptr, words, 8 * first, d_err, s));
+            }
+            if (d > 1) id = next_id;
+            carried.push_back(from);
+        }
+        return KD_OK;
+    };
     // payload plane list: [id (while a later gather needs it)], R_0, R_{k-1}, ..., R_{d+1}
-    if (k >= 2 && all_arrays) {
+    auto chain_by_keys = [&]() -> kd_status {
         const uint32_t* id_src = H->perm0;  // array 0 order
         // the first sort's keys come from duplicate removal; the second's are
         // carried through the first sort (see above)
@@ -1052,6 +1155,9 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             id_src = cur_id;
             ranks_prev = ranks;
         }
+        return KD_OK;
+    };
+    auto records = [&]() -> kd_status {
         // Remaining rank planes: array d (d != 1) lacks the ranks R_p of the
         // planes the chain did not carry; they are a permutation of array 1's
         // planes by destination R_d.  Each is done as one grouping pass on the
@@ -1114,6 +1220,11 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             LaunchTimer lt(ctx, F_RECORDS, 0.0, H->d_m, 4.0);
             CK(launch_own_ranks(H->d_m, N, k, H->rec, s));
         }
+        return KD_OK;
+    };
+    if (k >= 2 && all_arrays) {
+        CKS(by_words ? chain_by_words() : chain_by_keys());
+        CKS(records());
     }
     // learn m ----------------------------------------------------------------
     const unsigned char* h_info = nullptr;
@@ -1121,6 +1232,13 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     InfoBlock info;
     memcpy(&info, h_info, sizeof(info));
     CKS(err_status(ctx, info.err));
+    if (info.redo) {  // a run the sample did not show: once more by whole keys
+        CKS(chain_by_keys());
+        CKS(records());
+        CKS(fetch(ctx, d_info, sizeof(InfoBlock) + (size_t)count * 4, &h_info));
+        memcpy(&info, h_info, sizeof(info));
+        CKS(err_status(ctx, info.err));
+    }
     const int32_t* mc = reinterpret_cast<const int32_t*>(h_info + sizeof(InfoBlock));
     const int64_t M = info.m;
     H->M = M;

@@ -24,7 +24,7 @@
 //                 keys equals comparing these ranks.
 #include <algorithm>
 
-#include "kd_internal.cuh"
+#include "kd_block_sort.cuh"
 
 namespace kd {
 
@@ -1435,6 +1435,170 @@ __global__ void __launch_bounds__(256) k_run_cross(const uint32_t* __restrict__ 
     }
 }
 
+// --------------------------------------------------------- chain by words
+// The chain (array d = stable sort of array d+1 by x_d) with few and narrow
+// passes: instead of the whole key, a 32-bit word of it, and instead of every
+// rank plane, one payload, the source position; the planes then follow by
+// one gather.  A word is exact where the input's x_d differ in their low
+// four bytes alone; otherwise it holds the three leading bytes that differ,
+// and the runs of equal words are put right afterwards (k_word_runs).
+//   k_word_sample  before the first sort: how many of a sample's words
+//                  coincide, so that inputs with long runs keep whole keys;
+//   k_chain_next   array d from the sorted positions: rank planes, ids, and
+//                  the words of the next sort;
+//   k_word_runs    runs of equal words ordered by the whole x_d (equal ones
+//                  keep their order).
+constexpr int WORD_SAMPLE = 4096;
+constexpr int WORD_RUN = 64;  // longest run of equal words put right
+
+// Collisions among the leading three differing bytes of WORD_SAMPLE evenly
+// spaced keys of plane blockIdx.x (0 where the low four bytes hold all
+// differences).
+template <typename KW>
+__global__ void __launch_bounds__(1024) k_word_sample(const KW* __restrict__ keys, int64_t n, int64_t stride,
+                                                      const uint32_t* __restrict__ hist, uint32_t* __restrict__ out) {
+    constexpr int D = sizeof(KW), E = WORD_SAMPLE / 1024;
+    __shared__ uint32_t s_key[WORD_SAMPLE];
+    __shared__ uint16_t s_idx[WORD_SAMPLE];
+    __shared__ __align__(16) uint16_t wc[32][RADIX];
+    __shared__ uint32_t s_ws[32];
+    const int tid = threadIdx.x, d = blockIdx.x;
+    int top = 0;  // highest byte that differs
+    for (int b = 1; b < D; ++b)
+        if (__syncthreads_count(tid < RADIX && hist[(d * D + b) * RADIX + (tid & (RADIX - 1))] != 0) > 1) top = b;
+    if (top < 4) {
+        if (tid == 0) out[d] = 0;
+        return;
+    }
+    const int m = (int)(n < WORD_SAMPLE ? n : WORD_SAMPLE);
+    uint32_t key[E], id[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int o = (tid >> 5) * 32 * E + e * 32 + (tid & 31);
+        id[e] = (uint32_t)o;
+        key[e] = o < m ? (uint32_t)(keys[d * stride + o * n / m] >> (8 * (top - 2))) & 0xffffffu : 0u;
+    }
+    for (int b = 0; b < 24; b += 8) block_pass<32, E>(key, id, b, m, s_key, s_idx, wc, s_ws);
+    int c = 0;
+    for (int i = tid; i + 1 < m; i += 1024) c += s_key[i] == s_key[i + 1] ? 1 : 0;
+    c = (int)__reduce_add_sync(0xffffffffu, (uint32_t)c);
+    __syncthreads();
+    if ((tid & 31) == 0) s_ws[tid >> 5] = (uint32_t)c;
+    __syncthreads();
+    if (tid < 32) {
+        c = (int)__reduce_add_sync(0xffffffffu, s_ws[tid]);
+        if (tid == 0) out[d] = (uint32_t)c;
+    }
+}
+
+// Array d from the places perm[i] of its tuples in array d+1 (nullptr: the
+// same places): nplanes rank planes and the ids move along, and words[i]
+// receives the next sort's word, (key >> shift) of the tuple.
+struct ChainNext {
+    const uint32_t* src[MAXK];
+    uint32_t* dst[MAXK];
+    int nplanes;
+    const uint32_t* id_src;
+    uint32_t* id_dst;  // nullptr: not wanted
+    const void* plane;  // nullptr: no next sort
+    uint32_t* words;
+    int shift;
+};
+constexpr int CN_ITEMS = 4;
+template <typename KW>
+__global__ void __launch_bounds__(256) k_chain_next(const int64_t* __restrict__ count_ptr,
+                                                    const uint32_t* __restrict__ perm, int64_t id_limit,
+                                                    const __grid_constant__ ChainNext C, int* __restrict__ err) {
+    const int64_t count = *count_ptr;
+    const int64_t base = (int64_t)blockIdx.x * 256 * CN_ITEMS + threadIdx.x;
+    if (base >= count) return;
+    uint32_t p[CN_ITEMS];
+#pragma unroll
+    for (int e = 0; e < CN_ITEMS; ++e) {
+        const int64_t i = base + (int64_t)e * 256;
+        p[e] = i < count ? (perm ? perm[i] : (uint32_t)i) : 0u;
+        if ((int64_t)p[e] >= count) {  // only from inconsistent sorts
+            atomicOr(err, ERR_INTERNAL);
+            p[e] = 0;
+        }
+    }
+    if (C.plane) {
+        uint32_t id[CN_ITEMS];
+#pragma unroll
+        for (int e = 0; e < CN_ITEMS; ++e) {
+            id[e] = C.id_src[p[e]];
+            if ((int64_t)id[e] >= id_limit) {
+                atomicOr(err, ERR_INTERNAL);
+                id[e] = 0;
+            }
+        }
+        KW x[CN_ITEMS];
+#pragma unroll
+        for (int e = 0; e < CN_ITEMS; ++e) x[e] = static_cast<const KW*>(C.plane)[id[e]];
+#pragma unroll
+        for (int e = 0; e < CN_ITEMS; ++e) {
+            const int64_t i = base + (int64_t)e * 256;
+            if (i >= count) break;
+            C.words[i] = (uint32_t)(x[e] >> C.shift);
+            if (C.id_dst) C.id_dst[i] = id[e];
+        }
+    }
+    for (int q = 0; q < C.nplanes; ++q) {
+        uint32_t v[CN_ITEMS];
+#pragma unroll
+        for (int e = 0; e < CN_ITEMS; ++e) v[e] = C.src[q][p[e]];
+#pragma unroll
+        for (int e = 0; e < CN_ITEMS; ++e) {
+            const int64_t i = base + (int64_t)e * 256;
+            if (i < count) C.dst[q][i] = v[e];
+        }
+    }
+}
+
+// perm (sorted by the 24 low bits of words) to out, runs of equal words by
+// the whole x_d of the tuples (their ids in the order before the sort in
+// ids).  A run above WORD_RUN is left as it is and sets *redo.
+template <typename KW>
+__global__ void __launch_bounds__(256) k_word_runs(const int64_t* __restrict__ count_ptr,
+                                                   const uint32_t* __restrict__ words,
+                                                   const uint32_t* __restrict__ perm, const uint32_t* __restrict__ ids,
+                                                   const KW* __restrict__ plane, int64_t id_limit,
+                                                   uint32_t* __restrict__ out, int32_t* __restrict__ redo,
+                                                   int* __restrict__ err) {
+    const int64_t count = *count_ptr;
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= count) return;
+    const uint32_t w = words[i] & 0xffffffu, me = perm[i];
+    auto word = [&](int64_t j) { return words[j] & 0xffffffu; };
+    int64_t s = i, f = i;
+    while (s > 0 && i - s < WORD_RUN && word(s - 1) == w) --s;
+    while (f + 1 < count && f - i < WORD_RUN && word(f + 1) == w) ++f;
+    if (f - s + 1 > WORD_RUN) {
+        *redo = 1;
+        s = f = i;
+    }
+    if (s == f) {
+        out[i] = me;
+        return;
+    }
+    auto key = [&](uint32_t at) -> KW {
+        const uint32_t id = (int64_t)at < count ? ids[at] : 0xffffffffu;
+        if ((int64_t)id >= id_limit) {
+            atomicOr(err, ERR_INTERNAL);
+            return 0;
+        }
+        return plane[id];
+    };
+    const KW x = key(me);
+    int64_t o = s;
+    for (int64_t j = s; j <= f; ++j) {
+        if (j == i) continue;
+        const KW y = key(perm[j]);
+        o += y < x || (y == x && j < i) ? 1 : 0;
+    }
+    out[o] = me;
+}
+
 // -------------------------------------------------------------- records
 // rec[d][p][i]: rank in super-key-p order of the tuple at position i of index
 // array d.  After deduplication super keys are unique, so comparing super
@@ -1716,6 +1880,41 @@ cudaError_t launch_gather(int key64, const int64_t* count_ptr, int64_t max_count
     else
         k_gather<uint32_t, GI><<<(unsigned)blocks, 256, 0, s>>>(count_ptr, (const uint32_t*)plane, ids, max_count,
                                                                (uint32_t*)out, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_word_sample(const void* keys, int64_t n, int k, int64_t stride, const uint32_t* hist, uint32_t* out,
+                               cudaStream_t s) {
+    k_word_sample<uint64_t><<<k, 1024, 0, s>>>((const uint64_t*)keys, n, stride, hist, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_chain_next(int key64, const int64_t* count_ptr, int64_t max_count, const uint32_t* perm, int nplanes,
+                              const uint32_t* const* src, uint32_t* const* dst, const uint32_t* id_src,
+                              uint32_t* id_dst, const void* plane, uint32_t* words, int shift, int* err,
+                              cudaStream_t s) {
+    ChainNext C{};
+    for (int q = 0; q < nplanes; ++q) {
+        C.src[q] = src[q];
+        C.dst[q] = dst[q];
+    }
+    C.nplanes = nplanes;
+    C.id_src = id_src;
+    C.id_dst = id_dst;
+    C.plane = plane;
+    C.words = words;
+    C.shift = shift;
+    const unsigned blocks = (unsigned)((max_count + 256 * CN_ITEMS - 1) / (256 * CN_ITEMS));
+    if (key64) k_chain_next<uint64_t><<<blocks, 256, 0, s>>>(count_ptr, perm, max_count, C, err);
+    else k_chain_next<uint32_t><<<blocks, 256, 0, s>>>(count_ptr, perm, max_count, C, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_word_runs(const int64_t* count_ptr, int64_t max_count, const uint32_t* words, const uint32_t* perm,
+                             const uint32_t* ids, const void* plane, uint32_t* out, int32_t* redo, int* err,
+                             cudaStream_t s) {
+    k_word_runs<uint64_t><<<(unsigned)((max_count + 255) / 256), 256, 0, s>>>(
+        count_ptr, words, perm, ids, (const uint64_t*)plane, max_count, out, redo, err);
     return cudaGetLastError();
 }
 
