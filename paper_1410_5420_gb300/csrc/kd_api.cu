@@ -1735,7 +1735,9 @@ kd_status select_build(kd_ctx* ctx, kd_presorted* H, kd_tree* out) {
     CKS(S.get(&unresolved, 16));
     const int nbytes = k * w;
     int cur = 0;
-    for (int L = 0; L < lam; ++L) {
+    // (level 0: array 0 is in super-key-0 order, so its median is in place and
+    // so are its halves; launch_top_nodes writes the root)
+    for (int L = 1; L < lam; ++L) {
         LaunchTimer lt(ctx, F_SELECT, (double)M, nullptr, 0.0);
         CK(launch_sel_level(key64, ids, keys, cur, k, (int32_t)M, L, stile, segs, ghist, gany, unresolved, node, 0, d_err, s,
                             0, 0, 0));

@@ -135,34 +135,60 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_hist(const __grid_constant_
     constexpr int B = sizeof(KW);
     const int j = r / B, sh = sel_shift<KW>(r);
     const int p = L % k;
+    // the leading words of all rows in flight before the first is used
+    KW x0[SEL_IPT];
+    int slot[SEL_IPT];
+    const bool one = T.ns == 1;
+    const int32_t lo0 = T.lo[0], hi0 = T.hi[0];
+#pragma unroll
     for (int e = 0; e < SEL_IPT; ++e) {
         const int o = e * SEL_THREADS + tid;
         const int32_t pos = pos0 + o;
-        int sj = o < npos ? tile_slot(T.lo, T.hi, T.ns, pos) : -1;
+        slot[e] = -1;
+        if (o < npos) {
+            if (one) slot[e] = pos >= lo0 && pos <= hi0 ? 0 : -1;
+            else slot[e] = tile_slot(T.lo, T.hi, T.ns, pos);
+        }
+        x0[e] = slot[e] >= 0 ? bufs.key[cur][p][pos] : (KW)0;
+    }
+#pragma unroll
+    for (int e = 0; e < SEL_IPT; ++e) {
+        const int32_t pos = pos0 + e * SEL_THREADS + tid;
+        const int sj = slot[e];
         bool cand = sj >= 0 && T.pos[sj] == -1 && r >= T.start[sj];
         uint32_t dig = 0;
         if (cand) {
             // the words of the super key up to word j, compared with the prefix
-            KW wj = 0;
-#pragma unroll
-            for (int jj = 0; jj < MAXK; ++jj) {
-                if (jj > j) break;
-                int d = p + jj;
-                if (d >= k) d -= k;
-                const KW x = bufs.key[cur][d][pos];
-                if (jj < j) cand = cand && x == T.prefix[sj][jj];
-                else wj = x;
+            KW wj = x0[e];
+            if (j > 0) {
+                cand = wj == T.prefix[sj][0];
+                for (int jj = 1; jj <= j && cand; ++jj) {
+                    int d = p + jj;
+                    if (d >= k) d -= k;
+                    wj = bufs.key[cur][d][pos];
+                    if (jj < j) cand = wj == T.prefix[sj][jj];
+                }
             }
             if (cand && sh + 8 < 8 * B) cand = (wj >> (sh + 8)) == (T.prefix[sj][j] >> (sh + 8));
             dig = (uint32_t)(wj >> sh) & 255u;
         }
-        // candidates of one segment and digit in this warp add once (long runs of
-        // equal top bytes would otherwise serialise on one counter)
-        const uint32_t key = cand ? ((uint32_t)sj << 8 | dig) : 0xffffffffu;
-        const uint32_t peers = __match_any_sync(0xffffffffu, key);
-        if (cand && (threadIdx.x & 31) == __ffs(peers) - 1) {
-            atomicAdd(&h[sj][dig], (uint32_t)__popc(peers));
-            any[sj][dig] = pos;
+        // the lanes that share the first candidate's segment and digit add once
+        // (a run of equal top bytes would serialise on one counter); the others
+        // add for themselves.  (Grouping every digit by a match instruction kept
+        // that pipe 82% busy on spread digits; a round over 2^22 int64 tuples
+        // 21 -> 16 us on average.)
+        const uint32_t cands = __ballot_sync(0xffffffffu, cand);
+        if (cands == 0) continue;
+        const int first = __ffs(cands) - 1;
+        const uint32_t key = (uint32_t)sj << 8 | dig;
+        const uint32_t lead = __shfl_sync(0xffffffffu, key, first);  // (every lane takes part)
+        const uint32_t same = __ballot_sync(0xffffffffu, cand && key == lead);
+        if (cand) {
+            const bool mine = (same >> (tid & 31)) & 1u;
+            if (!mine || (tid & 31) == first) {
+                atomicAdd(&h[sj][dig], mine ? (uint32_t)__popc(same) : 1u);
+                any[sj][dig] = pos;
+            }
         }
     }
     __syncthreads();
@@ -215,10 +241,17 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_span(const __grid_constant_
     sel_load_tile(T, pos0, npos, m, L, segs, err);  // (synchronises the block)
     const int p = L % k;
     // warp, then block, then one global update per segment of the tile
+    KW x0[SEL_IPT];
+#pragma unroll
+    for (int e = 0; e < SEL_IPT; ++e) {
+        const int o = e * SEL_THREADS + tid;
+        x0[e] = o < npos ? bufs.key[cur][p][pos0 + o] : (KW)0;
+    }
+#pragma unroll
     for (int e = 0; e < SEL_IPT; ++e) {
         const int o = e * SEL_THREADS + tid;
         const int sj = o < npos ? tile_slot(T.lo, T.hi, T.ns, pos0 + o) : -1;
-        const KW w = sj >= 0 ? bufs.key[cur][p][pos0 + o] : (KW)0;
+        const KW w = sj >= 0 ? x0[e] : (KW)0;
         const uint32_t peers = __match_any_sync(0xffffffffu, (uint32_t)sj);  // lanes of one segment
         KW a, b;
         sel_warp_and_or(peers, w, a, b);
@@ -339,41 +372,52 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_move(const __grid_constant_
     }
     if (tid < LEVEL_NSMAX * 2) (&scnt[0][0])[tid] = 0;
     __syncthreads();
-    int flag[SEL_IPT];
+    // half and slot of every row's element, packed: -1 none, else slot * 2 + half.
+    // The loads of all rows are in flight before the first is used, here and
+    // plane by plane below (row by row, each waited for its own): a level over
+    // 2^22 int64 tuples of k = 3, 91 -> 49 us.
+    int where[SEL_IPT];
     uint32_t local[SEL_IPT];
-    int slot[SEL_IPT];
+    KW x0[SEL_IPT];
 #pragma unroll
     for (int e = 0; e < SEL_IPT; ++e) {
         const int o = e * SEL_THREADS + tid;
-        flag[e] = -1;
-        slot[e] = -1;
-        local[e] = 0;
-        if (o >= npos) continue;
-        const int32_t pos = pos0 + o;
-        const int sj = tile_slot(T.lo, T.hi, T.ns, pos);
-        if (sj < 0) continue;
-        if (T.pos[sj] < T.lo[sj] || T.pos[sj] > T.hi[sj]) {
-            atomicOr(err, ERR_INTERNAL);
-            continue;
-        }
-        int c = 0;
+        x0[e] = o < npos ? bufs.key[cur][p][pos0 + o] : (KW)0;
+    }
 #pragma unroll
-        for (int j = 0; j < MAXK; ++j) {
-            if (j >= k || c != 0) break;
-            int d = p + j;
-            if (d >= k) d -= k;
-            const KW x = bufs.key[cur][d][pos], y = med[sj][j];
-            if (x != y) c = x < y ? -1 : 1;
+    for (int e = 0; e < SEL_IPT; ++e) {
+        const int o = e * SEL_THREADS + tid;
+        where[e] = -1;
+        const int32_t pos = pos0 + o;
+        const int sj = o < npos ? tile_slot(T.lo, T.hi, T.ns, pos) : -1;
+        if (sj >= 0) {
+            const int32_t mp = T.pos[sj];
+            if (mp < T.lo[sj] || mp > T.hi[sj]) {
+                atomicOr(err, ERR_INTERNAL);
+            } else {
+                KW x = x0[e], y = med[sj][0];
+                for (int j = 1; j < k && x == y; ++j) {
+                    int d = p + j;
+                    if (d >= k) d -= k;
+                    x = bufs.key[cur][d][pos];
+                    y = med[sj][j];
+                }
+                if (x == y) {
+                    if (pos != mp) atomicOr(err, ERR_INTERNAL);
+                    const int32_t mid = T.lo[sj] + ((T.hi[sj] - T.lo[sj]) >> 1);
+                    node[mid] = (int32_t)((int64_t)bufs.id[cur][pos] - in_off);
+                } else {
+                    where[e] = sj * 2 + (x > y ? 1 : 0);
+                }
+            }
         }
-        slot[e] = sj;
-        if (c == 0) {
-            if (pos != T.pos[sj]) atomicOr(err, ERR_INTERNAL);
-            const int32_t mid = T.lo[sj] + ((T.hi[sj] - T.lo[sj]) >> 1);
-            node[mid] = (int32_t)((int64_t)bufs.id[cur][pos] - in_off);
-            continue;
-        }
-        flag[e] = c > 0 ? 1 : 0;
-        local[e] = atomicAdd(&scnt[sj][flag[e]], 1u);
+        // the lanes of a row that go to the same half claim their places together
+        const uint32_t peers = __match_any_sync(0xffffffffu, where[e]);
+        const int leader = __ffs(peers) - 1;
+        uint32_t at = 0;
+        if (where[e] >= 0 && (tid & 31) == leader) at = atomicAdd(&(&scnt[0][0])[where[e]], (uint32_t)__popc(peers));
+        at = __shfl_sync(0xffffffffu, at, leader);
+        local[e] = at + __popc(peers & lanemask_lt());
     }
     __syncthreads();
     if (tid < T.ns * 2) {
@@ -381,19 +425,38 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_move(const __grid_constant_
         sbase[x][f] = atomicAdd(&segs[T.idx[x]].cnt[f], scnt[x][f]);
     }
     __syncthreads();
+    int32_t dest[SEL_IPT];
 #pragma unroll
     for (int e = 0; e < SEL_IPT; ++e) {
-        if (flag[e] < 0) continue;
-        const int sj = slot[e];
+        dest[e] = -1;
+        if (where[e] < 0) continue;
+        const int sj = where[e] >> 1, f = where[e] & 1;
         const int32_t lo = T.lo[sj], hi = T.hi[sj], mid = lo + ((hi - lo) >> 1);
-        const int32_t dst = (flag[e] ? mid + 1 : lo) + (int32_t)(sbase[sj][flag[e]] + local[e]);
-        if (flag[e] ? (dst <= mid || dst > hi) : (dst >= mid)) {
+        const int32_t dst = (f ? mid + 1 : lo) + (int32_t)(sbase[sj][f] + local[e]);
+        if (f ? (dst <= mid || dst > hi) : (dst >= mid)) {
             atomicOr(err, ERR_INTERNAL);
             continue;
         }
-        const int32_t pos = pos0 + e * SEL_THREADS + tid;  // < pos0 + npos: flag[e] >= 0
-        bufs.id[cur ^ 1][dst] = bufs.id[cur][pos];
-        for (int d = 0; d < k; ++d) bufs.key[cur ^ 1][d][dst] = bufs.key[cur][d][pos];
+        dest[e] = dst;
+        bufs.key[cur ^ 1][p][dst] = x0[e];
+    }
+    const int32_t first = pos0 + tid;
+    {
+        uint32_t v[SEL_IPT];
+#pragma unroll
+        for (int e = 0; e < SEL_IPT; ++e) v[e] = dest[e] >= 0 ? bufs.id[cur][first + e * SEL_THREADS] : 0u;
+#pragma unroll
+        for (int e = 0; e < SEL_IPT; ++e)
+            if (dest[e] >= 0) bufs.id[cur ^ 1][dest[e]] = v[e];
+    }
+    for (int d = 0; d < k; ++d) {
+        if (d == p) continue;
+        KW v[SEL_IPT];
+#pragma unroll
+        for (int e = 0; e < SEL_IPT; ++e) v[e] = dest[e] >= 0 ? bufs.key[cur][d][first + e * SEL_THREADS] : (KW)0;
+#pragma unroll
+        for (int e = 0; e < SEL_IPT; ++e)
+            if (dest[e] >= 0) bufs.key[cur ^ 1][d][dest[e]] = v[e];
     }
 }
 
