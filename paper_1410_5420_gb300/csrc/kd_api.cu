@@ -120,6 +120,10 @@ constexpr uint64_t RUN_COST_PER_TUPLE = 128;
 // estimate) up to which the chain sorts by words.
 constexpr double WORD_MATES = 4.0;
 
+// Destinations of one cloud's missing rank planes that are scattered at once:
+// three quarters of the 129 MB L2 (both sides measured where it is used).
+constexpr int64_t SCATTER_BYTES = 96000000;
+
 enum Family {
     F_TRANSFORM = 0, F_SORT, F_DEDUP, F_RECORDS, F_LEVEL, F_FINISH, F_TOP, F_OTHER, F_GATHER,
     F_SELECT,         // median-selection build: selection rounds and partitions of the levels
@@ -1160,8 +1164,18 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     auto records = [&]() -> kd_status {
         // Remaining rank planes: array d (d != 1) lacks the ranks R_p of the
         // planes the chain did not carry; they are a permutation of array 1's
-        // planes by destination R_d.  Each is done as one grouping pass on the
-        // top bits of R_d (ranges that fit in L2) and an in-range scatter.
+        // planes by destination R_d: scattered at once where the destinations of
+        // a cloud stay in L2 (SCATTER_BYTES), else after one grouping pass on the
+        // top bits of R_d (ranges that fit in L2).  The pass reads and writes
+        // nv + 1 planes and costs two launches; the scatter alone takes as long as
+        // the scatter after it, as long as its lines are evicted full.  Uniform
+        // ranks, grouped and at once: 6 million tuples of k = 6 (96 MB for the
+        // largest array) 7.78 and 7.64 ms, 2^22 of k = 6 (80 MB) 5.30 and 5.06,
+        // 2^22 of k = 2 (17 MB) 1.24 and 1.20, 4096 clouds of up to 2^16 15.06
+        // and 14.66; past the line 6 million with 120 MB at once 7.70 against
+        // 7.64, 2^25 of k = 2 (134 MB) 7.19 against 6.99, 2^26 14.65 against 13.82.
+        int64_t span = 0;  // tuples of the largest cloud: array order keeps clouds apart
+        for (int i = 0; i < count; ++i) span = std::max(span, H->n_c[i]);
         uint32_t* pbases = nullptr;
         CKS(S.get(&pbases, RADIX * 4));
         uint64_t present = 0;  // 8 bits per array: planes already written
@@ -1180,6 +1194,19 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
                 if (q != d && !((bits >> q) & 1u)) miss.push_back(q);
             if (!miss.empty()) {
                 const int nv = (int)miss.size();
+                PayloadArgs sc{};
+                sc.n = nv;
+                if (span * nv * 4 <= SCATTER_BYTES) {
+                    for (int j = 0; j < nv; ++j) {
+                        sc.src[j] = miss[j] == 1 ? nullptr : H->rec.p[1][miss[j]];  // R_1 of array 1 = position
+                        sc.dst[j] = H->rec.p[d][miss[j]];
+                    }
+                    LaunchTimer lt(ctx, F_RECORDS, 0.0, H->d_m, 4.0 + 8.0 * nv);
+                    CK(launch_perm_scatter(H->d_m, N, H->rec.p[1][d], sc, s));
+                    for (int q : miss) bits |= 1u << q;
+                    present |= bits << (d * MAXK);
+                    continue;
+                }
                 // destination ranges of about 16 MB of scattered words: the
                 // scatter's random 4-byte writes then merge in L2 (2^26
                 // tuples: 1.92 ms for the records against 2.01 ms with 48 MB
@@ -1204,8 +1231,6 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
                     CK(launch_sort_pass(0, H->d_m, N, H->rec.p[1][d], gdest, pay, pbases, shift, status, ++pass_no, d_err, s,
                                         ctx->spin_limit));
                 }
-                PayloadArgs sc{};
-                sc.n = nv;
                 for (int j = 0; j < nv; ++j) {
                     sc.src[j] = pbuf[0][j];
                     sc.dst[j] = H->rec.p[d][miss[j]];

@@ -1626,7 +1626,8 @@ __global__ void k_perm_bases(const int64_t* __restrict__ m_ptr, int shift, uint3
     bases[threadIdx.x] = block_excl_scan256((uint32_t)c, s_warp, nullptr);
 }
 
-// Scatter of nval planes by destination: dst[j][dest[i]] = src[j][i].  Each
+// Scatter of nval planes by destination: dst[j][dest[i]] = src[j][i], a NULL
+// source standing for the position i.  Each
 // thread moves PS_ITEMS elements with all their loads in flight at once.
 constexpr int PS_ITEMS = 4;  // 4: 1.88 ms for the records per 2^26 step, 8: 1.93, 16: 1.96
 __global__ void __launch_bounds__(256) k_perm_scatter(const int64_t* __restrict__ m_ptr,
@@ -1646,7 +1647,7 @@ __global__ void __launch_bounds__(256) k_perm_scatter(const int64_t* __restrict_
 #pragma unroll
         for (int e = 0; e < PS_ITEMS; ++e) {
             const int64_t i = base + (int64_t)e * 256;
-            v[e] = i < m ? pa.src[j][i] : 0u;
+            v[e] = i < m ? (pa.src[j] ? pa.src[j][i] : (uint32_t)i) : 0u;
         }
 #pragma unroll
         for (int e = 0; e < PS_ITEMS; ++e)
