@@ -46,6 +46,8 @@ cudaError_t launch_word_runs(const int64_t* count_ptr, int64_t max_count, const 
                              const uint32_t* ids, const void* plane, uint32_t* out, int32_t* redo, int* err,
                              cudaStream_t s);
 cudaError_t launch_pack_clouds(const PackDesc* d, int count, void* dst, cudaStream_t s);
+cudaError_t launch_cloud_ids(const int64_t* count_ptr, int64_t n, const uint32_t* plane, const int64_t* start, int ncloud,
+                             const uint32_t* ids, uint32_t* out, int* err, cudaStream_t s);
 cudaError_t launch_gather(int key64, const int64_t* count_ptr, int64_t max_count, const void* plane,
                           const uint32_t* ids, void* out, int* err, cudaStream_t s);
 size_t dedup_scratch_words(int64_t n);
@@ -993,7 +995,7 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         const void* ksrc = P.mode == KEY_BUF ? (const void*)kbuf[kc] : plane_ptr(-1);
         if (P.mode == KEY_GATHER) {
             LaunchTimer lg(ctx, F_GATHER, 0.0, H->d_m, 12.0);
-            CK(launch_gather(0, H->d_m, N, plane_ptr(-1), ibuf[ic], kbuf[kc], d_err, s));
+            CK(launch_cloud_ids(H->d_m, N, cloud_plane, cstart, count, ibuf[ic], (uint32_t*)kbuf[kc], d_err, s));
             ksrc = kbuf[kc];
         }
         LaunchTimer lt(ctx, F_SORT, 0.0, H->d_m, pass_bytes(P, !last, 1));
@@ -1142,7 +1144,10 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
                 void* kdst = (last || next_gathers) ? nullptr : (void*)kbuf[kc ^ 1];
                 if (gather) {
                     LaunchTimer lg(ctx, F_GATHER, 0.0, H->d_m, 4.0 + 2.0 * P.w);
-                    CK(launch_gather(plane64(P.plane), H->d_m, N, plane_ptr(P.plane), cur_id, kbuf[kc], d_err, s));
+                    if (P.plane < 0)
+                        CK(launch_cloud_ids(H->d_m, N, cloud_plane, cstart, count, cur_id, (uint32_t*)kbuf[kc], d_err, s));
+                    else
+                        CK(launch_gather(plane64(P.plane), H->d_m, N, plane_ptr(P.plane), cur_id, kbuf[kc], d_err, s));
                     ksrc = kbuf[kc];
                 }
                 LaunchTimer lt(ctx, F_SORT, 0.0, H->d_m, pass_bytes(P, kdst != nullptr, pay.n));

@@ -30,6 +30,16 @@ namespace kd {
 
 // -------------------------------------------------------------- helpers
 // ------------------------------------------------------------ transform
+// Largest c in [lo, hi) with start[c] <= p, given that start[lo] <= p.
+template <typename P, typename Q>
+__device__ __forceinline__ int cloud_of(const P* start, int lo, int hi, Q p) {
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (start[mid] <= p) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // hist layout: row (d * D + b) for coordinate d, key byte b; then rows
 // (k * D + b) for the cloud-id plane of a batch.  Dynamic smem: the block's
 // histogram rows followed by a 256-point staging tile of coordinates.
@@ -45,13 +55,35 @@ __global__ void __launch_bounds__(256) k_transform(const T* __restrict__ coords,
     const int nrows = k * D + cloud_digits;
     uint32_t* sh = smem;
     T* sc = reinterpret_cast<T*>(smem + nrows * RADIX);
+    __shared__ int s_cloud[2];  // the 256 points' clouds lie between these
     const int tid = threadIdx.x;
     for (int i = tid; i < nrows * RADIX; i += 256) sh[i] = 0;
     int nan = 0;
+    // A batch: the block's tiles are consecutive, so that each tile's clouds are
+    // found from the last one's (38.9 million tuples in 4096 clouds: 599 -> 384
+    // us).  One cloud: the blocks' tiles alternate, so that the blocks read and
+    // write side by side (2^26 tuples: 486 us, consecutive 553).
+    const int64_t tiles = (n + 255) / 256;
+    int64_t base = (int64_t)blockIdx.x * 256, past = n, stride_pts = (int64_t)gridDim.x * 256;
+    if (ncloud > 1) {
+        base = tiles * blockIdx.x / gridDim.x * 256;
+        past = min(tiles * (blockIdx.x + 1) / gridDim.x * 256, n);
+        stride_pts = 256;
+        if (tid == 0) s_cloud[1] = cloud_of(cloud_start, 0, ncloud, base);
+    }
     __syncthreads();
-    for (int64_t base = (int64_t)blockIdx.x * 256; base < n; base += (int64_t)gridDim.x * 256) {
+    for (; base < past; base += stride_pts) {
         const int cnt = (int)(n - base < 256 ? n - base : 256);
         for (int i = tid; i < cnt * k; i += 256) sc[i] = coords[base * k + i];
+        if (ncloud > 1 && tid == 0) {
+            int lo = s_cloud[1], hi = lo + 1;
+            s_cloud[0] = lo;
+            for (int step = 1; hi < ncloud && cloud_start[hi] <= base + cnt - 1; step *= 2) {
+                lo = hi;
+                hi = min(hi + step, ncloud);
+            }
+            s_cloud[1] = cloud_of(cloud_start, lo, hi, base + cnt - 1);
+        }
         __syncthreads();
         if (tid < cnt) {
             const int64_t p = base + tid;
@@ -64,14 +96,10 @@ __global__ void __launch_bounds__(256) k_transform(const T* __restrict__ coords,
                     atomicAdd(&sh[(d * D + b) * RADIX + (uint32_t)((key >> (8 * b)) & 255u)], 1u);
             }
             if (ncloud > 1) {
-                int lo = 0, hi = ncloud;  // largest c with cloud_start[c] <= p
-                while (hi - lo > 1) {
-                    int mid = (lo + hi) >> 1;
-                    if (cloud_start[mid] <= p) lo = mid; else hi = mid;
-                }
-                cloud_plane[p] = (uint32_t)lo;
+                const int c = cloud_of(cloud_start, s_cloud[0], s_cloud[1] + 1, p);
+                cloud_plane[p] = (uint32_t)c;
                 for (int b = 0; b < cloud_digits; ++b)
-                    atomicAdd(&sh[(k * D + b) * RADIX + ((lo >> (8 * b)) & 255)], 1u);
+                    atomicAdd(&sh[(k * D + b) * RADIX + ((c >> (8 * b)) & 255)], 1u);
             }
         }
         __syncthreads();
@@ -793,6 +821,61 @@ __global__ void __launch_bounds__(256) k_gather(const int64_t* __restrict__ coun
     for (int j = 0; j < GI; ++j) {
         const int64_t p = base + (int64_t)j * 256;
         if (p < count) out[p] = v[j];
+    }
+}
+
+// The cloud of every tuple id: out[pos] = largest c with start[c] <= ids[pos],
+// positions in [0, *count_ptr), from the clouds' starts in shared memory and a
+// table of CLOUD_CELLS equal ranges of ids with the clouds they begin and end
+// in, most of which leave none or one halving.  The ids come in the order of
+// the last coordinate sorted by, so a gather of the cloud-id plane reads a
+// 32-byte sector for each 4 bytes, past L2 from 32 million tuples: 38.9 million
+// tuples, 4096 clouds 425 us, this 107 (2.9 TB/s streamed, bound by the
+// shared-memory reads).  The tables cost each block some 12 us first: whole
+// builds of batches, gather against this, 2.4 million tuples 1.52 and 1.54 ms,
+// 9.7 million 3.94 and 3.90, 19 million 7.26 and 7.12, 78 million 29.8 and
+// 26.9.
+constexpr int CLOUD_CELLS = 4096;
+constexpr int CLOUD_THREADS = 512;
+constexpr int CLOUD_ITEMS = 8;
+constexpr int64_t CLOUD_MIN_TUPLES = (int64_t)1 << 23;
+constexpr int CLOUD_MAX = 8192;  // starts and cells in the 48 KB a block has without asking
+__global__ void __launch_bounds__(CLOUD_THREADS, 4)
+    k_cloud_ids(const int64_t* __restrict__ count_ptr, const int64_t* __restrict__ start, int ncloud, int64_t n, int shift,
+                const uint32_t* __restrict__ ids, uint32_t* __restrict__ out, int* __restrict__ err) {
+    extern __shared__ uint32_t smem[];
+    uint32_t* s_start = smem;                                         // [ncloud]
+    uint16_t* s_cell = reinterpret_cast<uint16_t*>(smem + ncloud);  // [CLOUD_CELLS + 1]
+    const int tid = threadIdx.x;
+    for (int c = tid; c < ncloud; c += CLOUD_THREADS) s_start[c] = (uint32_t)start[c];
+    __syncthreads();
+    for (int j = tid; j <= CLOUD_CELLS; j += CLOUD_THREADS) {
+        const int64_t p = (int64_t)j << shift;
+        s_cell[j] = (uint16_t)cloud_of(s_start, 0, ncloud, (uint32_t)(p < n ? p : n - 1));
+    }
+    __syncthreads();
+    const int64_t count = *count_ptr;
+    constexpr int TILE = CLOUD_THREADS * CLOUD_ITEMS;
+    for (int64_t base = (int64_t)blockIdx.x * TILE; base < count; base += (int64_t)gridDim.x * TILE) {
+        uint32_t id[CLOUD_ITEMS];
+#pragma unroll
+        for (int j = 0; j < CLOUD_ITEMS; ++j) {
+            const int64_t p = base + j * CLOUD_THREADS + tid;
+            id[j] = p < count ? ids[p] : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < CLOUD_ITEMS; ++j) {
+            const int64_t p = base + j * CLOUD_THREADS + tid;
+            if (p >= count) continue;
+            int c = 0;
+            if ((int64_t)id[j] < n) {
+                const uint32_t cell = id[j] >> shift;
+                c = cloud_of(s_start, s_cell[cell], s_cell[cell + 1] + 1, id[j]);
+            } else {
+                atomicOr(err, ERR_INTERNAL);
+            }
+            out[p] = (uint32_t)c;
+        }
     }
 }
 
@@ -1683,18 +1766,30 @@ constexpr size_t TRANSFORM_SMEM_MAX = (size_t)(MAXK * 8 + 4) * RADIX * 4 + 256 *
 
 // Concatenation of device clouds: block b copies the 32-bit words of the
 // clouds whose descriptors it strides over (src, words, destination word).
+// Bound by the loads in flight and by the largest clouds' blocks: eight loads
+// a thread and eight blocks a cloud (38.9 million tuples of 12 bytes in 4096
+// clouds of up to 2^16: 256 -> 154 us, 6.1 TB/s read and written).
+constexpr int PACK_LOADS = 8;
 __global__ void __launch_bounds__(256) k_pack_clouds(const PackDesc* __restrict__ d, int count,
                                                      uint32_t* __restrict__ dst) {
     for (int c = blockIdx.x; c < count; c += gridDim.x) {
         const PackDesc e = d[c];
         const uint32_t* src = static_cast<const uint32_t*>(e.src);
-        for (int64_t i = threadIdx.x; i < e.words; i += 256) dst[e.dst_word + i] = src[i];
+        for (int64_t i = (int64_t)blockIdx.y * 256 * PACK_LOADS + threadIdx.x; i < e.words;
+             i += (int64_t)gridDim.y * 256 * PACK_LOADS) {
+            uint32_t v[PACK_LOADS];
+#pragma unroll
+            for (int j = 0; j < PACK_LOADS; ++j) v[j] = i + 256 * j < e.words ? src[i + 256 * j] : 0u;
+#pragma unroll
+            for (int j = 0; j < PACK_LOADS; ++j)
+                if (i + 256 * j < e.words) dst[e.dst_word + i + 256 * j] = v[j];
+        }
     }
 }
 
 cudaError_t launch_pack_clouds(const PackDesc* d, int count, void* dst, cudaStream_t s) {
     if (count == 0) return cudaSuccess;
-    k_pack_clouds<<<std::min(count, 152 * 16), 256, 0, s>>>(d, count, static_cast<uint32_t*>(dst));
+    k_pack_clouds<<<dim3(std::min(count, 152 * 16), 8), 256, 0, s>>>(d, count, static_cast<uint32_t*>(dst));
     return cudaGetLastError();
 }
 
@@ -1881,6 +1976,17 @@ cudaError_t launch_gather(int key64, const int64_t* count_ptr, int64_t max_count
     else
         k_gather<uint32_t, GI><<<(unsigned)blocks, 256, 0, s>>>(count_ptr, (const uint32_t*)plane, ids, max_count,
                                                                (uint32_t*)out, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cloud_ids(const int64_t* count_ptr, int64_t n, const uint32_t* plane, const int64_t* start, int ncloud,
+                             const uint32_t* ids, uint32_t* out, int* err, cudaStream_t s) {
+    if (ncloud > CLOUD_MAX || n < CLOUD_MIN_TUPLES) return launch_gather(0, count_ptr, n, plane, ids, out, err, s);
+    int shift = 0;
+    while ((n - 1) >> shift >= CLOUD_CELLS) ++shift;
+    const size_t smem = (size_t)ncloud * 4 + (CLOUD_CELLS + 1) * 2;
+    k_cloud_ids<<<grid_for(n, CLOUD_THREADS * CLOUD_ITEMS, 152 * 4), CLOUD_THREADS, smem, s>>>(
+        count_ptr, start, ncloud, n, shift, ids, out, err);
     return cudaGetLastError();
 }
 
