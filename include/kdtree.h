@@ -261,8 +261,11 @@ kd_status kd_presort_noalloc(kd_ctx *ctx, const kd_cloud *cloud, int32_t *arrays
  * kd_index_create: a search index for tree `tree` built from `cloud` (the
  * same coordinates, host or device; the tree's node_tuple array host or
  * device).  The index keeps the tuples in the tree's address order on the
- * device (m x k coordinates and m tuple indices), allocated from the
- * context; destroy it with kd_index_destroy before destroying the context.
+ * device (m x k coordinates, one plane each, bounding boxes of about 1/16 of
+ * their size, and m tuple indices), allocated from the context; where its
+ * budget has no room for the boxes the index does without, with the same
+ * results and slower searches.  Destroy it with kd_index_destroy before
+ * destroying the context.
  */
 typedef struct kd_index_s *kd_index;
 kd_status kd_index_create(kd_ctx *ctx, const kd_cloud *cloud, const kd_tree *tree, kd_index *out);
