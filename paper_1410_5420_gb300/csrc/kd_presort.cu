@@ -679,7 +679,6 @@ __global__ void __launch_bounds__(RS_THREADS)
     __shared__ uint32_t s_ticket;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        s_ticket = atomicAdd(ctr, 1u);  // (cleared long before the previous pass)
         mbar_init(&full, 1);
         fence_mbar_init();
     }
@@ -687,10 +686,13 @@ __global__ void __launch_bounds__(RS_THREADS)
         (&s_wc[0][0])[i] = 0;
         (&s_match[0][0])[i] = 0;
     }
+    // the previous pass's keys and payloads, and the counters: the first pass
+    // follows the memset that clears them, whose writes are visible only now
+    pdl_wait();
+    pdl_trigger();
+    if (tid == 0) s_ticket = atomicAdd(ctr, 1u);
     __syncthreads();
     const int64_t t = s_ticket;
-    pdl_wait();  // the previous pass's keys and payloads
-    pdl_trigger();
     const int64_t count = *count_ptr;
     const int64_t base = t * TILE;
     if (base >= count) return;
