@@ -515,9 +515,10 @@ __device__ __forceinline__ void knn_insert(double* bd, int32_t* bi, int kn, doub
 // near side first.  queries as for k_knn.
 template <typename T>
 __global__ void __launch_bounds__(SEARCH_THREADS) k_knn_walk(const T* __restrict__ pts, int64_t stride,
-                                                             const int32_t* __restrict__ tuple, int32_t m, int k, const T* __restrict__ queries, int64_t nq,
-                                                        int kn, int32_t* __restrict__ idx_out,
-                                                        double* __restrict__ d_out, int* __restrict__ err) {
+                                                             const int32_t* __restrict__ tuple, int32_t m, int k,
+                                                             const T* __restrict__ queries, int64_t nq, int kn,
+                                                             int32_t* __restrict__ idx_out,
+                                                             double* __restrict__ d_out, int* __restrict__ err) {
     const int64_t qi = (int64_t)blockIdx.x * SEARCH_THREADS + threadIdx.x;
     if (qi >= nq) return;
     const int32_t self = queries ? -1 : tuple[qi];
@@ -1005,8 +1006,8 @@ void cells_as(kd_index_s* ix, int levels, const void* lo, int64_t nq, uint32_t* 
 template <typename T>
 void knn_of(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err,
             cudaStream_t s) {
-    if (ix->m > 0 && !ix->boxes)
-        k_knn_walk<T><<<grid_of(nq, SEARCH_THREADS), SEARCH_THREADS, 0, s>>>(
+    if (ix->m > 0 && !ix->boxes)  // (a thread per query, so a grid that no cap of grid_of cuts)
+        k_knn_walk<T><<<(unsigned)((nq + SEARCH_THREADS - 1) / SEARCH_THREADS), SEARCH_THREADS, 0, s>>>(
             (const T*)ix->pts, ix->m, ix->node_tuple, (int32_t)ix->m, ix->k, (const T*)queries, nq, kn, di, dd, err);
     else
         KD_SEARCH_K(knn_as, T, ix, queries, nq, kn, di, dd, err, s)
