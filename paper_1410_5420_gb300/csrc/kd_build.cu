@@ -1381,8 +1381,12 @@ __global__ void __launch_bounds__(FIN_THREADS, fin_min_blocks(SMAX, K))
         uint32_t sub = __ballot_sync(0xffffffffu, in);
         bool active = in;
         int32_t mlo = a0, mhi = b0;
-        int p = p0;  // the dimension of level l
-        for (int l = dl; __any_sync(0xffffffffu, active); ++l, p = p + 1 == K ? 0 : p + 1) {
+        int p = p0;  // the dimension of the level
+        // (a segment of at most 32 tuples is done in six levels; ranks that
+        // contradict each other, from inconsistent inputs, would leave a lane
+        // active for ever: its node stays unset and is reported below)
+#pragma unroll 1
+        for (int l = 0; l < 6 && __any_sync(0xffffffffu, active); ++l, p = p + 1 == K ? 0 : p + 1) {
             uint32_t lp = 0;
 #pragma unroll
             for (int q = 0; q < K; ++q)
