@@ -65,7 +65,8 @@ typedef struct {
                                 (kd_kernel_stats); bit 4: finisher phase counters; bit 8
                                 (failure-detection tests): bound the device waits to a few
                                 thousand polls and make the next presort's first look-back
-                                wait run out once, which it reports as KD_ETIMEOUT */
+                                wait run out once, which it reports as KD_ETIMEOUT; bit 16:
+                                the same for the next build's first level step */
     const char *tune_cache;  /* autotuner cache file (read by kd_create, rewritten by kd_autotune); NULL: none */
     int schedule;            /* level schedule of kd_build (same tree under each):
                                 KD_SCHEDULE_MULTI (0, default): an array is partitioned only when it is

@@ -84,14 +84,15 @@ bool level_tile_supported(int k, int tile);
 int level_status_stride(int k);
 cudaError_t launch_level_pass(int k, int tile, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
                               const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, uint32_t* status,
-                              int* err, cudaStream_t s);
+                              int* err, cudaStream_t s, uint32_t spin_limit, int withhold);
 size_t level_status_words(int k, int ntiles);
 int level_small_tile();
 bool level_steps_small(int64_t m);
 size_t level_small_bytes(int k, int64_t max_ntiles, int nsteps);
 cudaError_t launch_level_small(int k, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
                                const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, void* area,
-                               int64_t max_ntiles, int step, int* err, cudaStream_t s);
+                               int64_t max_ntiles, int step, int* err, cudaStream_t s, uint32_t spin_limit,
+                               int withhold);
 size_t finish_smem(int k, int smax);
 cudaError_t init_presort_kernels();
 cudaError_t init_small_kernels();
@@ -203,6 +204,7 @@ struct kd_ctx {
     // chunks' waits run out and the call reports KD_ETIMEOUT.
     uint32_t spin_limit = SPIN_LIMIT;
     bool inject_timeout = false;
+    bool inject_level_timeout = false;  // bit 16: the same for the next build's first level step
     std::string last_error;
     std::recursive_mutex mu;
     std::unordered_map<void*, size_t> sizes;
@@ -1646,14 +1648,21 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
         const int F = step_jobs[st][0].lev_out - step_jobs[st][0].lev_in;
         // array q moves k planes (array 0) or k - 1 (its own rank is not carried)
         LaunchTimer lt(ctx, F_LEVEL, step_elems[st], nullptr, 8.0 * (k - (step_q[st] != 0)) + 4.0 * F);
+        const int withhold = ctx->inject_level_timeout ? 1 : 0;
         if (small_steps) {
             CK(launch_level_small(k, bufs, step_q[st], d_jobs + job_off[st], (int)step_jobs[st].size(),
-                                  (int)step_ntiles[st], d_cd, medr, H->perm0, d_status, max_ntiles, (int)st, d_err, s));
-            continue;
+                                  (int)step_ntiles[st], d_cd, medr, H->perm0, d_status, max_ntiles, (int)st, d_err, s,
+                                  ctx->spin_limit, withhold));
+        } else {
+            ctx->launches += 3;  // tile records, count pass and scan
+            CK(launch_level_pass(k, tile, bufs, step_q[st], d_jobs + job_off[st], (int)step_jobs[st].size(),
+                                 (int)step_ntiles[st], d_cd, medr, H->perm0, d_status, d_err, s, ctx->spin_limit,
+                                 withhold));
         }
-        ctx->launches += 3;  // tile records, count pass and scan
-        CK(launch_level_pass(k, tile, bufs, step_q[st], d_jobs + job_off[st], (int)step_jobs[st].size(),
-                             (int)step_ntiles[st], d_cd, medr, H->perm0, d_status, d_err, s));
+        if (withhold) {  // the injected wait: report it before anything else runs
+            ctx->inject_level_timeout = false;
+            CKS(check_device_err(ctx, d_err));
+        }
     }
     if (nunits > 0) {
         unsigned long long* phase = nullptr;
@@ -1991,9 +2000,10 @@ kd_status kd_create(kd_ctx** out, const kd_config* cfg) {
     if (c.tune_cache) ctx->tune_cache = c.tune_cache;
     ctx->cfg.tune_cache = ctx->tune_cache.empty() ? nullptr : ctx->tune_cache.c_str();  // owned copy for workers
     tuning_load(ctx.get());
-    if (c.debug & 8) {
+    if (c.debug & (8 | 16)) {
         ctx->spin_limit = 4096;
-        ctx->inject_timeout = true;
+        ctx->inject_timeout = (c.debug & 8) != 0;
+        ctx->inject_level_timeout = (c.debug & 16) != 0;
     }
     if (cudaSetDevice(c.device) != cudaSuccess) return KD_EDEVICE;
     // kernel attributes are per device: set them once for each device used

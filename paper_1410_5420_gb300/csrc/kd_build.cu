@@ -382,7 +382,10 @@ __global__ void __launch_bounds__(LEVEL_BLOCK)
 // at once and scans them in registers; the threads' (flag, value) pairs are
 // scanned across the block; a chunk then publishes what it carries out
 // (inclusive at once when it holds a head) and takes what comes in by a
-// decoupled look-back over the earlier chunks of its bucket.
+// decoupled look-back over the earlier chunks of its bucket.  spin_limit
+// bounds the look-back's polls; a block whose wait runs out stores nothing
+// and reports ERR_TIMEOUT.  withhold (failure-detection tests only): chunk 0
+// never publishes.
 constexpr int LS_V = 4;
 constexpr int LS_CHUNK = 1024 * LS_V;
 __host__ __device__ __forceinline__ int level_scan_chunks(int ntiles) { return (ntiles + LS_CHUNK - 1) / LS_CHUNK; }
@@ -390,9 +393,10 @@ __host__ __device__ __forceinline__ int level_scan_chunks(int ntiles) { return (
 __global__ void __launch_bounds__(1024) k_level_scan(int ntiles, int ncol, int stride, const uint32_t* __restrict__ cnt,
                                                      const uint32_t* __restrict__ head, uint32_t* __restrict__ incl,
                                                      uint32_t* __restrict__ lb, uint32_t* __restrict__ ticket,
-                                                     int* __restrict__ err) {
+                                                     int* __restrict__ err, uint32_t spin_limit, int withhold) {
     __shared__ uint32_t s_f[32], s_v[32];
     __shared__ uint32_t s_ctl, s_id, s_carry;
+    __shared__ bool s_late;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     pdl_wait();
     pdl_trigger();
@@ -466,7 +470,8 @@ __global__ void __launch_bounds__(1024) k_level_scan(int ntiles, int ncol, int s
     // what the chunk carries out, ignoring what comes in: inclusive when the
     // chunk holds a head (or is the first)
     const bool blk_head = s_f[31] != 0u;
-    if (tid == 0) {
+    if (tid == 0) s_late = false;
+    if (tid == 0 && !(withhold && c == 0)) {
         if (c == 0 || blk_head) {
             inc[c] = s_v[31];
             publish_flag(flags, c, FLAG_INC);
@@ -477,7 +482,10 @@ __global__ void __launch_bounds__(1024) k_level_scan(int ntiles, int ncol, int s
     }
     uint32_t carry = 0;
     if (c > 0) {
-        const uint32_t ex = block_lookback<uint32_t>(flags, agg, inc, 1, c, &s_ctl, err, 1);
+        __syncthreads();  // s_late
+        const uint32_t ex =
+            block_lookback<uint32_t>(flags, agg, inc, 1, c, &s_ctl, err, 1, spin_limit, &s_late);
+        if (s_late) return;  // uniform: set by the look-back for the whole block
         if (tid == 0) {
             s_carry = ex;
             if (!blk_head) {
@@ -748,9 +756,12 @@ __device__ __forceinline__ void st_status(uint64_t* p, uint32_t epoch, uint32_t 
 // Sums of nbl (a power of two, at most 32) buckets over the tiles t - 1,
 // t - 2, ..., t_head (where the segment starts); status points to the first
 // of them.  Called by a whole warp; with fewer than 32 buckets the lanes hold
-// several tiles of a row.  Lane i < nbl returns bucket i's sum.
+// several tiles of a row.  Lane i < nbl returns bucket i's sum.  After
+// spin_limit polls that find a tile without a word the warp sets ERR_TIMEOUT
+// and *late, and the sums are meaningless.
 __device__ __forceinline__ uint32_t level_lookback(const uint64_t* __restrict__ status, int nbp, int nbl, int t,
-                                                   int t_head, uint32_t epoch, int* err) {
+                                                   int t_head, uint32_t epoch, uint32_t spin_limit, bool* late_out,
+                                                   int* err) {
     const int lane = threadIdx.x & 31;
     const int tpw = 32 / nbl, off = lane / nbl;
     const uint64_t* col = status + (lane & (nbl - 1));
@@ -790,8 +801,9 @@ __device__ __forceinline__ uint32_t level_lookback(const uint64_t* __restrict__ 
         if (__all_sync(0xffffffffu, done)) break;
         hi -= rows * tpw;
         if (stuck) {
-            if (++spins > SPIN_LIMIT) {
+            if (++spins > spin_limit) {
                 if (lane == 0) atomicOr(err, ERR_TIMEOUT);
+                *late_out = true;
                 break;
             }
             __nanosleep(100);
@@ -820,7 +832,8 @@ template <int K>
 __global__ void __launch_bounds__(LEVEL_THREADS)
     k_level_small(const __grid_constant__ AllBufs bufs, int q, const LevelJob* __restrict__ jobs, int njobs,
                   const CloudDev* __restrict__ clouds, uint32_t* __restrict__ medr, const uint32_t* __restrict__ perm0,
-                  uint64_t* __restrict__ status, uint32_t epoch, uint32_t* __restrict__ ctr, int* __restrict__ err) {
+                  uint64_t* __restrict__ status, uint32_t epoch, uint32_t* __restrict__ ctr, int* __restrict__ err,
+                  uint32_t spin_limit, int withhold) {
     constexpr int IPT = SMALL_IPT, TILE = SMALL_TILE;
     constexpr int NBMAX = 1 << (K - 1);
     constexpr int NDMAX = LEVEL_NSMAX * NBMAX;
@@ -929,21 +942,23 @@ __global__ void __launch_bounds__(LEVEL_THREADS)
             c += x;
         }
         if (d == tid) total = c;
-        if (sj == ns - 1) st_status(row + b, epoch, starts ? LB_INC : LB_AGG, c);
+        if (sj == ns - 1 && !(withhold && t == 0)) st_status(row + b, epoch, starts ? LB_INC : LB_AGG, c);
         s_dmid[d] = (J.write_med & LEVEL_MED) ? a + ((z - a) >> 1) : -2;
     }
+    bool late = false;
     if (cont && warp * 32 < NB) {
         __syncwarp();
         // tiles of this job back to the one holding the segment's first position
         const int t_head = t - (pos0 - tlo[0] + TILE - 1) / TILE;
-        const uint32_t before = level_lookback(status + warp * 32, NBMAX, NB < 32 ? NB : 32, t, t_head, epoch, err);
-        if (tid < NB) {
+        const uint32_t before = level_lookback(status + warp * 32, NBMAX, NB < 32 ? NB : 32, t, t_head, epoch,
+                                               spin_limit, &late, err);
+        if (tid < NB && !late) {
             if (ns == 1) st_status(row + tid, epoch, LB_INC, before + total);
 #pragma unroll
             for (int w = 0; w < LEVEL_WARPS; ++w) s_wc[w][tid] += before;
         }
     }
-    __syncthreads();
+    if (__syncthreads_or(late)) return;  // a wait ran out: no count is published as final, nothing stored
     int32_t dest[IPT];
 #pragma unroll
     for (int j = 0; j < IPT; ++j) {
@@ -1534,7 +1549,7 @@ size_t level_status_words(int k, int ntiles) {
 template <int K, int IPT>
 static cudaError_t level_step(const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
                               const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, const LevelStatus& L,
-                              int* err, cudaStream_t s) {
+                              int* err, cudaStream_t s, uint32_t spin_limit, int withhold) {
     const int v = IPT == 8 ? 1 : 0;
     const int nbmax = 1 << (K - 1);
     const int nch = level_scan_chunks(ntiles);
@@ -1548,7 +1563,8 @@ static cudaError_t level_step(const AllBufs& bufs, int q, const LevelJob* jobs, 
                              bufs, q, jobs, njobs, ntiles, clouds, (const uint32_t*)L.trec, L.cnt, L.head, L.ctrs, err);
     if (e == cudaSuccess)
         e = launch_dependent(k_level_scan, dim3(nbmax * nch), dim3(1024), 0, s, ntiles, nbmax, level_nbp(K),
-                             (const uint32_t*)L.cnt, (const uint32_t*)L.head, L.incl, L.lb, L.ctrs + 2, err);
+                             (const uint32_t*)L.cnt, (const uint32_t*)L.head, L.incl, L.lb, L.ctrs + 2, err,
+                             spin_limit, withhold);
     if (e == cudaSuccess)
         e = launch_dependent(k_level_pass<K, IPT>, dim3(gm), dim3(LEVEL_BLOCK), level_smem_bytes<K, IPT>(true), s, bufs,
                              q, jobs, njobs, ntiles, clouds, medr, perm0, (const uint32_t*)L.trec,
@@ -1560,23 +1576,23 @@ static cudaError_t level_step(const AllBufs& bufs, int q, const LevelJob* jobs, 
 // (1024, or 2048 for k <= 4).
 cudaError_t launch_level_pass(int k, int tile, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs,
                               int ntiles, const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0,
-                              uint32_t* status, int* err, cudaStream_t s) {
+                              uint32_t* status, int* err, cudaStream_t s, uint32_t spin_limit, int withhold) {
     if (ntiles == 0) return cudaSuccess;
     if (k < 2 || k > MAXK || g_num_sms == 0 || !level_tile_supported(k, tile)) return cudaErrorInvalidValue;
     const LevelStatus L = level_status_layout(k, ntiles, status);
     const bool big = tile == LEVEL_THREADS * 8;
     cudaError_t e = cudaSuccess;
     switch (k) {
-        case 2: e = big ? level_step<2, 8>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s)
-                        : level_step<2, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
-        case 3: e = big ? level_step<3, 8>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s)
-                        : level_step<3, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
-        case 4: e = big ? level_step<4, 8>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s)
-                        : level_step<4, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
-        case 5: e = level_step<5, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
-        case 6: e = level_step<6, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
-        case 7: e = level_step<7, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
-        case 8: e = level_step<8, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s); break;
+        case 2: e = big ? level_step<2, 8>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold)
+                        : level_step<2, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
+        case 3: e = big ? level_step<3, 8>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold)
+                        : level_step<3, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
+        case 4: e = big ? level_step<4, 8>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold)
+                        : level_step<4, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
+        case 5: e = level_step<5, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
+        case 6: e = level_step<6, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
+        case 7: e = level_step<7, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
+        case 8: e = level_step<8, 4>(bufs, q, jobs, njobs, ntiles, clouds, medr, perm0, L, err, s, spin_limit, withhold); break;
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
@@ -1601,7 +1617,8 @@ size_t level_small_bytes(int k, int64_t max_ntiles, int nsteps) {
 // positions; `step` numbers the build's calls.
 cudaError_t launch_level_small(int k, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
                                const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, void* area,
-                               int64_t max_ntiles, int step, int* err, cudaStream_t s) {
+                               int64_t max_ntiles, int step, int* err, cudaStream_t s, uint32_t spin_limit,
+                               int withhold) {
     if (ntiles == 0) return cudaSuccess;
     uint64_t* status = static_cast<uint64_t*>(area);
     uint32_t* ctr =
@@ -1609,7 +1626,7 @@ cudaError_t launch_level_small(int k, const AllBufs& bufs, int q, const LevelJob
 #define KD_SMALL(K)                                                                                                \
     case K:                                                                                                        \
         return launch_dependent(k_level_small<K>, dim3(ntiles), dim3(LEVEL_THREADS), 0, s, bufs, q, jobs, njobs,   \
-                                clouds, medr, perm0, status, (uint32_t)step + 1u, ctr, err);
+                                clouds, medr, perm0, status, (uint32_t)step + 1u, ctr, err, spin_limit, withhold);
     switch (k) {
         KD_SMALL(2) KD_SMALL(3) KD_SMALL(4) KD_SMALL(5) KD_SMALL(6) KD_SMALL(7) KD_SMALL(8)
         default: return cudaErrorInvalidValue;
