@@ -16,6 +16,8 @@
 //   k_boxes         bounding boxes over blocks of 32 consecutive addresses
 //   k_knn           one warp per query: walk of the box tree, nearest first,
 //                   the best candidates sorted across the warp
+//   k_knn_exact     the queries k_knn has left (distances that 32-bit floats
+//                   do not tell apart), by double distances alone
 //   k_knn_walk      one thread per query: depth-first walk of the tree, for
 //                   an index without boxes
 //   k_region        one thread per box: depth-first walk visiting a side
@@ -130,13 +132,21 @@ __global__ void __launch_bounds__(256) k_index_gather(const T* __restrict__ coor
 //
 // Float distances.  a = the float sum of the squared float |p - q| differs
 // from the exact distance t by less than 2^-20 t (roundings of at most
-// (K + 4) 2^-24 in all), unless it underflows (below KNN_TINY) or overflows to +inf.  So
-// with A the kn-th smallest a, every one of the kn nearest tuples has
+// (K + 4) 2^-24 in all), unless it underflows (below KNN_TINY) or overflows to
+// +inf.  So with A the kn-th smallest a, every one of the kn nearest tuples has
 // a <= A (1 + 2^-18) = the bound, and a box whose float distance, less
 // 2^-18 of itself, exceeds the bound holds none of them.  All candidates up
 // to the bound are ranked by (double distance, tuple index).  If more than
 // the list's 32 lie below it (ties, or near ties, around kn), the query is
-// answered again with double distances for every candidate (`exact`).
+// answered again with double distances for every candidate (EXACT).  Where
+// that is certain because the bound cannot fall any more (KNN_TINY) or tells
+// nothing apart (+inf), the walk gives up and leaves the query to
+// k_knn_exact, which prunes by double distances of the boxes too: each of
+// their rounded steps grows with its operands, so that no tuple of a box comes
+// out nearer than the box.  2^17 normal float32 tuples scaled by 1e-20 or by
+// 1e22, whose squares leave the float's range, eight neighbours of each: 3.0
+// ms (both float walks over every block of the index 754 ms, the walk by one
+// thread per query 8.0, unscaled 0.23).
 constexpr int BOX_W = 32;        // tuples per block, children per node
 constexpr int BOX_LEVELS = 5;    // level 4 has at most 32 boxes for 2^30 tuples
 constexpr int KNN_THREADS = 256;
@@ -144,6 +154,8 @@ constexpr float KNN_MARGIN = 3.814697265625e-6f;  // 2^-18
 constexpr float KNN_TINY = 1e-35f;
 constexpr uint32_t KNN_NONE = 0xffffffffu;  // no candidate / child done
 constexpr uint32_t KNN_OPEN = 0xfffffffeu;  // bound while the list holds fewer than kn
+constexpr uint32_t KNN_INF = 0x7f800000u;   // float bits of +inf
+constexpr int32_t KNN_LEFT = INT32_MIN;     // first index of a row that is left to k_knn_exact
 
 template <typename T>
 struct KnnTree {
@@ -190,6 +202,19 @@ __device__ __forceinline__ float gap_f<float>(float q, float lo, float hi) {
 __device__ __forceinline__ uint32_t knn_bound(float a) {
     return __float_as_uint(fmaxf(a * (1.0f + KNN_MARGIN), KNN_TINY));
 }
+// More candidates up to the bound than the list holds, and a bound that
+// cannot fall any more or that tells nothing apart.  Asked once per 32 blocks
+// of floats, once per 1024 of 64-bit integers (whose differences overflow only
+// to the far ends of the type), never of 32-bit ones.  (In knn_block, or with a
+// bound that also says so, k_knn has more spills and all neighbours of 2^22
+// int64 tuples take 7.09 -> 7.33 to 7.49 ms; once per 32 blocks 7.16 -> 7.21.)
+template <typename T>
+constexpr bool knn_may_stick(int level) {
+    return std::is_same<T, float>::value || (sizeof(T) == 8 && level > 1);
+}
+__device__ __forceinline__ bool knn_stuck(uint32_t lost, uint32_t bound) {
+    return lost <= bound && (bound <= __float_as_uint(KNN_TINY) || bound >= KNN_INF);
+}
 
 // The query of one warp and its candidates (lane j: the j-th best).
 template <typename T, int K>  // K: the dimensions, or MAXK: at most that many
@@ -210,7 +235,7 @@ __device__ __forceinline__ double exact_dist(const KnnTree<T>& X, const T (&q)[K
     double acc = 0.0;
 #pragma unroll
     for (int d = 0; d < K; ++d) {
-            if (K == MAXK && d >= X.k) break;
+        if (K == MAXK && d >= X.k) break;
         const double u = abs_diff<T>(X.pts[d * X.stride + a], q[d]);
         acc = __dadd_rn(acc, __dmul_rn(u, u));
     }
@@ -358,8 +383,95 @@ __device__ __forceinline__ void knn_node(const KnnTree<T>& X, KnnQuery<T, K>& Q,
         if (best > Q.bound) break;
         const int c = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
         if (lane == c) key = KNN_NONE;
-        if constexpr (L > 0) knn_node<T, K, EXACT, L - 1>(X, Q, node * BOX_W + c);
-        else knn_block<T, K, EXACT>(X, Q, node * BOX_W + c);
+        if constexpr (L > 0) {
+            knn_node<T, K, EXACT, L - 1>(X, Q, node * BOX_W + c);
+            if constexpr (!EXACT && knn_may_stick<T>(L))
+                if (knn_stuck(Q.lost, Q.bound)) break;
+        } else {
+            knn_block<T, K, EXACT>(X, Q, node * BOX_W + c);
+        }
+    }
+}
+
+// ---- by double distances alone: one query, its list (distance bits, tuple
+// index) sorted across the warp.
+template <typename T, int K>
+struct KnnExact {
+    T q[K];
+    int32_t self;
+    int kn;
+    uint64_t last;  // distance of the kn-th best (~0: fewer so far)
+    uint64_t dkey;
+    int32_t tup;
+};
+
+__device__ __forceinline__ uint64_t warp_min64(uint64_t x) {
+    const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(x >> 32));
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, (uint32_t)(x >> 32) == hi ? (uint32_t)x : 0xffffffffu);
+    return (uint64_t)hi << 32 | lo;
+}
+
+template <typename T, int K>
+__device__ __forceinline__ void knn_exact_block(const KnnTree<T>& X, KnnExact<T, K>& Q, int32_t blk) {
+    const int lane = threadIdx.x & 31;
+    const int32_t a = blk * BOX_W + lane;
+    double dist = 0.0;
+    int32_t tp = 0;
+    bool pass = a < X.m && a != Q.self;
+    if (pass) {
+        dist = exact_dist<T, K>(X, Q.q, a);
+        tp = X.tuple[a];
+    }
+    const uint64_t dk = (uint64_t)__double_as_longlong(dist);
+    pass = pass && dist == dist && dk <= Q.last;
+    for (uint32_t mask = __ballot_sync(0xffffffffu, pass); mask; mask &= mask - 1) {
+        const int src = __ffs(mask) - 1;
+        const uint64_t d = __shfl_sync(0xffffffffu, dk, src);
+        const int32_t t = __shfl_sync(0xffffffffu, tp, src);
+        const int pos = __popc(__ballot_sync(0xffffffffu, Q.dkey < d || (Q.dkey == d && Q.tup < t)));
+        if (pos >= Q.kn) continue;
+        const uint64_t ud = __shfl_up_sync(0xffffffffu, Q.dkey, 1);
+        const int32_t ut = __shfl_up_sync(0xffffffffu, Q.tup, 1);
+        if (lane > pos) {
+            Q.dkey = ud;
+            Q.tup = ut;
+        } else if (lane == pos) {
+            Q.dkey = d;
+            Q.tup = t;
+        }
+    }
+    Q.last = __shfl_sync(0xffffffffu, Q.dkey, Q.kn - 1);
+}
+
+template <typename T, int K, int L>
+__device__ __forceinline__ void knn_exact_node(const KnnTree<T>& X, KnnExact<T, K>& Q, int32_t node) {
+    if constexpr (L > 0) {
+        if (L > X.top) {
+            knn_exact_node<T, K, L - 1>(X, Q, 0);
+            return;
+        }
+    }
+    const int lane = threadIdx.x & 31;
+    uint64_t key = ~0ull;
+    if (node * BOX_W + lane < X.nbox[L]) {
+        const T* b = X.box[L] + (int64_t)node * (2 * (K == MAXK ? X.k : K) * BOX_W) + lane;
+        double acc = 0.0;
+#pragma unroll
+        for (int d = 0; d < K; ++d) {
+            if (K == MAXK && d >= X.k) break;
+            const T lo = b[d * BOX_W], hi = b[((K == MAXK ? X.k : K) + d) * BOX_W];
+            const double u = Q.q[d] < lo ? abs_diff<T>(lo, Q.q[d]) : (Q.q[d] > hi ? abs_diff<T>(Q.q[d], hi) : 0.0);
+            acc = __dadd_rn(acc, __dmul_rn(u, u));
+        }
+        key = (uint64_t)__double_as_longlong(acc);
+    }
+    for (int i = 0; i < BOX_W; ++i) {
+        const uint64_t best = warp_min64(key);
+        if (best == ~0ull || best > Q.last) break;
+        const int c = __ffs(__ballot_sync(0xffffffffu, key == best)) - 1;
+        if (lane == c) key = ~0ull;
+        if constexpr (L > 0) knn_exact_node<T, K, L - 1>(X, Q, node * BOX_W + c);
+        else knn_exact_block<T, K>(X, Q, node * BOX_W + c);
     }
 }
 
@@ -403,6 +515,7 @@ __device__ __forceinline__ void knn_emit(const KnnTree<T>& X, const T* __restric
 // distances of all their candidates at once, one per lane: with kn = 8 and
 // one query at a time, 24 of the 32 lanes of every FP64 instruction idled
 // while that pipe was 89% busy.
+// err: the error bits, then whether queries are left to k_knn_exact.
 // Five blocks per SM (a few spills up to k = 4): 7.2 -> 7.05 ms for all eight
 // neighbours of 2^22 int64 tuples, 1.57 -> 1.37 for 2^20 float32; six: 7.3, 1.39.
 template <typename T, int K>
@@ -439,7 +552,12 @@ __global__ void __launch_bounds__(KNN_THREADS, K <= 4 ? 5 : 2) k_knn(const __gri
             if (X.m > 0) knn_node<T, K, false, BOX_LEVELS - 1>(X, Q, 0);
             const int32_t c = Q.key != KNN_NONE && Q.key <= Q.bound ? Q.addr : -1;  // the first lanes
             const int cnt = __popc(__ballot_sync(0xffffffffu, c >= 0));
-            if (Q.lost <= Q.bound || cnt == 0) {
+            if (knn_stuck(Q.lost, Q.bound)) {  // left to k_knn_exact
+                if (lane == 0) {
+                    idx_out[qi * kn] = KNN_LEFT;
+                    err[1] = 1;
+                }
+            } else if (Q.lost <= Q.bound || cnt == 0) {
                 // more candidates up to the bound than the list holds, or none at all
                 Q.bound = KNN_OPEN;
                 if (cnt > 0) knn_node<T, K, true, BOX_LEVELS - 1>(X, Q, 0);
@@ -458,6 +576,44 @@ __global__ void __launch_bounds__(KNN_THREADS, K <= 4 ? 5 : 2) k_knn(const __gri
         }
         if (__any_sync(0xffffffffu, cand >= 0))
             knn_emit<T, K>(X, queries, q0 + lane / width, cand, width, kn, idx_out, d_out);
+    }
+}
+
+// The queries k_knn has left (KNN_LEFT).  Each warp looks at `per` (at most
+// 32) rows.
+template <typename T, int K>
+__global__ void __launch_bounds__(KNN_THREADS, 2) k_knn_exact(const __grid_constant__ KnnTree<T> X,
+                                                              const T* __restrict__ queries, int64_t nq, int kn,
+                                                              int per, int32_t* __restrict__ idx_out,
+                                                              double* __restrict__ d_out) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t q0 = ((int64_t)blockIdx.x * (KNN_THREADS / 32) + (threadIdx.x >> 5)) * per; q0 < nq;
+         q0 += (int64_t)gridDim.x * (KNN_THREADS / 32) * per) {
+        const int32_t v = lane < per && q0 + lane < nq ? idx_out[(q0 + lane) * kn] : 0;
+        for (uint32_t left = __ballot_sync(0xffffffffu, v == KNN_LEFT); left; left &= left - 1) {
+            const int r = __ffs(left) - 1;
+            const int64_t qi = q0 + r;
+            KnnExact<T, K> Q;
+            bool nan = false;
+#pragma unroll
+            for (int d = 0; d < K; ++d) {
+                if (K == MAXK && d >= X.k) break;
+                Q.q[d] = queries ? queries[qi * (K == MAXK ? X.k : K) + d] : X.pts[d * X.stride + qi];
+                nan |= is_nan(Q.q[d]);
+            }
+            if (nan) continue;  // (its row was left unwritten, whatever it holds)
+            Q.self = queries ? -1 : (int32_t)qi;
+            Q.kn = kn;
+            Q.last = Q.dkey = ~0ull;
+            Q.tup = INT32_MAX;
+            knn_exact_node<T, K, BOX_LEVELS - 1>(X, Q, 0);
+            if (lane < kn) {
+                const bool none = Q.dkey == ~0ull;
+                idx_out[qi * kn + lane] = none ? -1 : Q.tup;
+                if (d_out)
+                    d_out[qi * kn + lane] = __longlong_as_double(none ? 0x7ff0000000000000ll : (long long)Q.dkey);
+            }
+        }
     }
 }
 
@@ -914,11 +1070,15 @@ kd_status to_device(kd_ctx* ctx, CallScratch& S, const void* src, size_t bytes, 
     return KD_OK;
 }
 
-kd_status read_err(kd_ctx* ctx, int* d_err, cudaStream_t s) {
-    int h = 0;
-    if (cudaMemcpyAsync(&h, d_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+// The error word after everything on the stream; left (if given): the word
+// after it.
+kd_status read_err(kd_ctx* ctx, int* d_err, cudaStream_t s, int* left = nullptr) {
+    int words[2] = {0, 0};
+    if (cudaMemcpyAsync(words, d_err, (left ? 2 : 1) * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return sfail(ctx, KD_EDEVICE, std::string("search: ") + cudaGetErrorString(cudaGetLastError()));
+    const int h = words[0];
+    if (left) *left = words[1];
     if (h & ERR_NAN) return sfail(ctx, KD_ENAN, "a query coordinate is NaN");
     if (h) return sfail(ctx, KD_EDEVICE, "inconsistent tree or index (device error flags " + std::to_string(h) + ")");
     return KD_OK;
@@ -957,7 +1117,7 @@ void index_fill(kd_ctx* ctx, kd_index_s* ix, const void* coords, int64_t n, int*
 }
 
 template <typename T, int K>
-void knn_as(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err,
+void knn_as(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err, bool exact,
             cudaStream_t s) {
     KnnTree<T> X{};
     X.pts = (const T*)ix->pts;
@@ -969,6 +1129,12 @@ void knn_as(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di
     for (int l = 0; l <= ix->top; ++l) {
         X.box[l] = (const T*)ix->boxes + ix->box_off[l];
         X.nbox[l] = ix->nbox[l];
+    }
+    if (exact) {
+        const int per = (int)std::max<int64_t>(1, std::min<int64_t>(32, nq / (152 * 32 * 4)));
+        k_knn_exact<T, K><<<grid_of(nq, KNN_THREADS / 32 * per), KNN_THREADS, 0, s>>>(X, (const T*)queries, nq, kn, per,
+                                                                                     di, dd);
+        return;
     }
     // several queries per warp only where there are warps enough without it (152 SMs x 32 warps)
     int width = 32;
@@ -1004,21 +1170,22 @@ void cells_as(kd_index_s* ix, int levels, const void* lo, int64_t nq, uint32_t* 
     }
 
 template <typename T>
-void knn_of(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err,
+void knn_of(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err, bool exact,
             cudaStream_t s) {
     if (ix->m > 0 && !ix->boxes)  // (a thread per query, so a grid that no cap of grid_of cuts)
         k_knn_walk<T><<<(unsigned)((nq + SEARCH_THREADS - 1) / SEARCH_THREADS), SEARCH_THREADS, 0, s>>>(
             (const T*)ix->pts, ix->m, ix->node_tuple, (int32_t)ix->m, ix->k, (const T*)queries, nq, kn, di, dd, err);
     else
-        KD_SEARCH_K(knn_as, T, ix, queries, nq, kn, di, dd, err, s)
+        KD_SEARCH_K(knn_as, T, ix, queries, nq, kn, di, dd, err, exact, s)
 }
 
-// The kn nearest tuples of nq queries (nullptr: of every address).
+// The kn nearest tuples of nq queries (nullptr: of every address); exact: of
+// those of them that such a call has left (err[1], which it sets).
 void launch_knn(kd_ctx* ctx, kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd,
-                int* err, cudaStream_t s) {
-    if (ix->dtype == KD_I32) knn_of<int32_t>(ix, queries, nq, kn, di, dd, err, s);
-    else if (ix->dtype == KD_I64) knn_of<int64_t>(ix, queries, nq, kn, di, dd, err, s);
-    else knn_of<float>(ix, queries, nq, kn, di, dd, err, s);
+                int* err, bool exact, cudaStream_t s) {
+    if (ix->dtype == KD_I32) knn_of<int32_t>(ix, queries, nq, kn, di, dd, err, exact, s);
+    else if (ix->dtype == KD_I64) knn_of<int64_t>(ix, queries, nq, kn, di, dd, err, exact, s);
+    else knn_of<float>(ix, queries, nq, kn, di, dd, err, exact, s);
     kd::ctx_add_launches(ctx, 1);
 }
 
@@ -1030,6 +1197,22 @@ void launch_region(kd_ctx* ctx, kd_index_s* ix, const void* lo, const void* hi, 
     else if (ix->dtype == KD_I64) KD_SEARCH_K(region_as, int64_t, ix, lo, hi, nq, order, norder, counts, kept, offs, out, err, s)
     else KD_SEARCH_K(region_as, float, ix, lo, hi, nq, order, norder, counts, kept, offs, out, err, s)
     kd::ctx_add_launches(ctx, 1);
+}
+
+// launch_knn with the copies of host outputs, to its end; once more for the
+// queries it has left, if any.
+kd_status run_knn(kd_ctx* ctx, kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd,
+                  int* d_err, int on_device, int32_t* idx_out, double* dist_out, cudaStream_t s) {
+    for (bool exact = false;; exact = true) {
+        launch_knn(ctx, ix, queries, nq, kn, di, dd, d_err, exact, s);
+        if (!on_device) {
+            cudaMemcpyAsync(idx_out, di, (size_t)nq * kn * 4, cudaMemcpyDeviceToHost, s);
+            if (dist_out) cudaMemcpyAsync(dist_out, dd, (size_t)nq * kn * 8, cudaMemcpyDeviceToHost, s);
+        }
+        int left = 0;
+        const kd_status st = read_err(ctx, d_err, s, &left);
+        if (exact || !left || (st != KD_OK && st != KD_ENAN)) return st;
+    }
 }
 
 int64_t offsets_chunks(int64_t n) { return std::max<int64_t>(1, (n + OFF_CHUNK - 1) / OFF_CHUNK); }
@@ -1163,15 +1346,10 @@ kd_status kd_knn(kd_ctx* ctx, kd_index ix, const void* queries, int64_t nq, int 
         st = S.get((void**)&di, (size_t)nq * kn * 4);
         if (st == KD_OK && dist_out) st = S.get((void**)&dd, (size_t)nq * kn * 8);
     }
-    if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
+    if (st == KD_OK) st = S.get((void**)&d_err, 2 * sizeof(int));
     if (st != KD_OK) return st;
-    cudaMemsetAsync(d_err, 0, sizeof(int), s);
-    launch_knn(ctx, ix, q, nq, kn, di, dd, d_err, s);
-    if (!on_device) {
-        cudaMemcpyAsync(idx_out, di, (size_t)nq * kn * 4, cudaMemcpyDeviceToHost, s);
-        if (dist_out) cudaMemcpyAsync(dist_out, dd, (size_t)nq * kn * 8, cudaMemcpyDeviceToHost, s);
-    }
-    return read_err(ctx, d_err, s);
+    cudaMemsetAsync(d_err, 0, 2 * sizeof(int), s);
+    return run_knn(ctx, ix, q, nq, kn, di, dd, d_err, on_device, idx_out, dist_out, s);
 }
 
 kd_status kd_knn_all(kd_ctx* ctx, kd_index ix, int kn, int on_device, int32_t* idx_out, double* dist_out) {
@@ -1191,15 +1369,10 @@ kd_status kd_knn_all(kd_ctx* ctx, kd_index ix, int kn, int on_device, int32_t* i
         st = S.get((void**)&di, (size_t)ix->m * kn * 4);
         if (st == KD_OK && dist_out) st = S.get((void**)&dd, (size_t)ix->m * kn * 8);
     }
-    if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
+    if (st == KD_OK) st = S.get((void**)&d_err, 2 * sizeof(int));
     if (st != KD_OK) return st;
-    cudaMemsetAsync(d_err, 0, sizeof(int), s);
-    launch_knn(ctx, ix, nullptr, ix->m, kn, di, dd, d_err, s);
-    if (!on_device) {
-        cudaMemcpyAsync(idx_out, di, (size_t)ix->m * kn * 4, cudaMemcpyDeviceToHost, s);
-        if (dist_out) cudaMemcpyAsync(dist_out, dd, (size_t)ix->m * kn * 8, cudaMemcpyDeviceToHost, s);
-    }
-    return read_err(ctx, d_err, s);
+    cudaMemsetAsync(d_err, 0, 2 * sizeof(int), s);
+    return run_knn(ctx, ix, nullptr, ix->m, kn, di, dd, d_err, on_device, idx_out, dist_out, s);
 }
 
 kd_status kd_reverse_knn(kd_ctx* ctx, kd_index ix, int kn, int on_device, int64_t* offsets, int32_t* rev_out) {
@@ -1215,7 +1388,7 @@ kd_status kd_reverse_knn(kd_ctx* ctx, kd_index ix, int kn, int on_device, int64_
     int64_t *cnt = nullptr, *offs = offsets, *cursor = nullptr;
     int* d_err = nullptr;
     int64_t n = 0;  // tuple indices are below the largest one + 1; the inverse map spans them
-    kd_status st = S.get((void**)&d_err, sizeof(int));
+    kd_status st = S.get((void**)&d_err, 2 * sizeof(int));
     if (st != KD_OK) return st;
     if (m == 0) {
         int64_t z = 0;
@@ -1242,10 +1415,11 @@ kd_status kd_reverse_knn(kd_ctx* ctx, kd_index ix, int kn, int on_device, int64_
         if (st == KD_OK) st = S.get((void**)&rev, (size_t)std::max<int64_t>(total, 1) * 4);
     }
     if (st != KD_OK) return st;
-    cudaMemsetAsync(d_err, 0, sizeof(int), s);
+    cudaMemsetAsync(d_err, 0, 2 * sizeof(int), s);
     cudaMemsetAsync(inv, 0xff, (size_t)n * 4, s);
     cudaMemsetAsync(cnt, 0, (size_t)m * 8, s);
-    launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, s);
+    launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, false, s);
+    if (ix->boxes) launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, true, s);  // (finds none to do, mostly)
     k_inv_map<<<grid_of(m, 256), 256, 0, s>>>(ix->node_tuple, m, n, inv, d_err);
     k_rev_count<<<grid_of(total, 256), 256, 0, s>>>(nn, total, inv, n, cnt, d_err);
     launch_offsets(ctx, cnt, m, cursor, offs, s);  // (the cursors' words hold the chunk sums meanwhile)
