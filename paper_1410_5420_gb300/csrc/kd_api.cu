@@ -100,8 +100,8 @@ int small_presort_max();
 size_t small_presort_words(int dtype, int n, int k, bool all_arrays);
 int small_sort_launches(int64_t n);
 cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, uint32_t* work, const AllPlanes& rec,
-                                 uint32_t* perm0, void* sel_keys, int64_t sel_stride, int64_t* m_out, int* err,
-                                 cudaStream_t s);
+                                 uint32_t* perm0, void* sel_keys, int64_t sel_stride, int64_t* m_out, int32_t* runs,
+                                 int* err, cudaStream_t s);
 cudaError_t init_build_kernels();
 int finish_kmax(int smax);
 cudaError_t launch_finish(const AllBufs& bufs, int k, const int64_t* unit_prefix, int ncloud, int64_t unit_base,
@@ -530,7 +530,7 @@ struct InfoBlock {
     int64_t n;             // tuples
     int32_t err;           // error bits
     int32_t redo;          // a run of equal words was too long (k_word_runs)
-    int32_t pad[2];
+    int32_t runs[2];       // of launch_small_presort
     uint32_t run_meta[4];  // of launch_run_stats
 };
 
@@ -668,22 +668,25 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     // tuples 439 -> 259 and 745 -> 340 us, 131072 467 -> 320 and 803 -> 454,
     // 196608 492 -> 408 and 881 -> 649; the merge of the chunks grows with the
     // square of their number.
+    kd_cloud there{};  // the cloud's copy on the device
     if (count == 1 && N <= small_presort_max()) {
-        const void* x = clouds[0].coords;
-        if (!clouds[0].on_device) {
+        there = clouds[0];
+        if (!there.on_device) {
             unsigned char* cb = nullptr;
             CKS(S.get(&cb, (size_t)N * k * tsz));
-            CK(cudaMemcpyAsync(cb, x, (size_t)N * k * tsz, cudaMemcpyHostToDevice, s));
-            x = cb;
+            CK(cudaMemcpyAsync(cb, there.coords, (size_t)N * k * tsz, cudaMemcpyHostToDevice, s));
+            there.coords = cb;
+            there.on_device = 1;
         }
+        Scratch W(ctx);
         uint32_t* work = nullptr;
-        CKS(S.get(&work, small_presort_words(dtype, (int)N, k, all_arrays) * 4));
+        CKS(W.get(&work, small_presort_words(dtype, (int)N, k, all_arrays) * 4));
         if (!all_arrays) CKS(dev_alloc(ctx, &H->sel_keys, (size_t)k * pad4(N) * w + 16));
         {
             LaunchTimer lt(ctx, F_SORT, (double)N, nullptr, (double)k * (tsz + 4));
             ctx->launches += small_sort_launches(N);  // the sort's, then the records (or the key planes)
-            CK(launch_small_presort(dtype, x, (int)N, k, work, H->rec, H->perm0, H->sel_keys, pad4(N), H->d_m, d_err,
-                                    s));
+            CK(launch_small_presort(dtype, there.coords, (int)N, k, work, H->rec, H->perm0, H->sel_keys, pad4(N), H->d_m,
+                                    d_info->runs, d_err, s));
         }
         ctx->inject_timeout = false;  // (no look-back to withhold a flag from)
         const unsigned char* h = nullptr;
@@ -691,11 +694,14 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
         CKS(fetch(ctx, d_info, sizeof(info), &h));
         memcpy(&info, h, sizeof(info));
         CKS(err_status(ctx, info.err));
-        H->M = info.m;
-        H->m_c[0] = H->m_off[1] = H->M;
-        guard.armed = false;
-        *out = H.release();
-        return KD_OK;
+        if (!info.runs[1]) {
+            H->M = info.m;
+            H->m_c[0] = H->m_off[1] = H->M;
+            guard.armed = false;
+            *out = H.release();
+            return KD_OK;
+        }
+        clouds = &there;  // few values per coordinate: by digit passes
     }
     // coordinates on the device, clouds back to back
     const void* coords = nullptr;

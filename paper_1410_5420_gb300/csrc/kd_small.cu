@@ -25,6 +25,13 @@ namespace kd {
 constexpr int SMALL_ONE = 2048;    // most tuples sorted by one block per super key
 constexpr int SMALL_MAX = 196608;  // most tuples sorted in chunks
 constexpr int SMALL_RUN = 32;      // longest run of equal x_d ordered by compares
+// Runs that are not merged (small_runs): long ones of all but one super key
+// from so many coordinates, ...
+constexpr int64_t SMALL_LONG_RUNS = 350000;
+// ... of half of them from so many tuples, and there all runs from so many
+// coordinates.
+constexpr int SMALL_MANY = 150000;
+constexpr int64_t SMALL_RUNS = 1100000;
 // Chunks of 2048 tuples up to 16384, 4096 up to 65536, 8192 above: a block's
 // sort takes longer with its chunk, the merge with the number of chunks.
 __host__ __device__ constexpr int small_chunk(int n) { return n <= 16384 ? 2048 : (n <= 65536 ? 4096 : 8192); }
@@ -77,10 +84,12 @@ __device__ __forceinline__ bool small_nan(const T* __restrict__ coords, int coun
 // index by compares, or, where a run exceeds SMALL_RUN, everything is sorted
 // again by the whole super key, least significant coordinate first, over
 // the bytes that differ.  Bound by shared-memory latency and issue on its
-// one SM.
-template <typename T, typename KW, int NW, int E>
+// one SM.  Where a run exceeds SMALL_RUN, or most threads hold a tuple of a
+// run, thread 0 calls report(whether it is the former), and stops what is left
+// to do where that returns true.
+template <typename T, typename KW, int NW, int E, typename R>
 __device__ __forceinline__ void small_order(const T* __restrict__ coords, int n, int k, int d,
-                                            const SmallShared<KW, NW, E>& S) {
+                                            const SmallShared<KW, NW, E>& S, const R& report) {
     constexpr int NT = 32 * NW, BITS = NT * E <= 1024 ? 16 : 24;
     uint32_t* const s_key = S.key;
     KW* const s_full = S.full;
@@ -162,12 +171,14 @@ __device__ __forceinline__ void small_order(const T* __restrict__ coords, int n,
             lng |= o + SMALL_RUN < n && word(o + SMALL_RUN) == word(o);
         }
         if (__syncthreads_or(lng)) {
+            if (__syncthreads_or(threadIdx.x == 0 && report(true))) return;
             for (int r = k - 1; r >= 0; --r) {
                 sort_by(d + r < k ? d + r : d + r - k, r == k - 1);
                 __syncthreads();
             }
             fill_keys();
-        } else if (__syncthreads_or(tie)) {
+        } else if (const int ties = __syncthreads_count(tie)) {
+            if (2 * ties > NT && threadIdx.x == 0) report(false);
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int o = base + e * 32;
@@ -225,7 +236,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
         }
         return;
     }
-    small_order<T, KW, NW, E>(coords, n, k, d, S);
+    small_order(coords, n, k, d, S, [](bool) { return false; });
     // a tuple equal to its predecessor goes (the smallest index comes first)
     uint32_t keep[E], cnt = 0;
 #pragma unroll
@@ -259,6 +270,18 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_sort(const T* __restrict__
     }
 }
 
+// The super keys whose order in some chunk had runs (small_order): bit d a run
+// of more than SMALL_RUN, bit 8 + d most tuples in runs.  Where `need` of the
+// super keys under `mask` did, rows[1] is set and the merge, which tells equal
+// x_d apart by the other coordinates at most steps of its searches, leaves the
+// sort to the caller.  rows NULL: it takes any.
+struct SmallRuns {
+    int32_t* rows;
+    uint32_t mask;
+    int need;
+};
+__device__ __forceinline__ bool small_leave(const SmallRuns& R) { return R.rows && R.rows[1]; }
+
 // Workspace of the chunked sort (rows of n per super key).
 template <typename KW>
 struct SmallWork {
@@ -268,6 +291,7 @@ struct SmallWork {
     uint32_t* dup;   // bit per place of raw: a duplicate (rows of `words`)
     uint32_t* nan;   // per chunk: it holds a NaN
     int words;
+    SmallRuns runs;
 };
 
 // Block (c, d): chunk c by super key d.
@@ -285,7 +309,14 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_chunks(const T* __restrict
         if (tid == 0) W.nan[c] = nan ? 1u : 0u;
     }
     for (int i = tid; i * 32 < cnt; i += CH / E) W.dup[(int64_t)d * W.words + first / 32 + i] = 0;
-    small_order<T, KW, NW, E>(x, cnt, k, d, S);
+    small_order(x, cnt, k, d, S, [&](bool longer) {
+        if (!W.runs.rows) return false;
+        const uint32_t bit = 1u << (longer ? d : 8 + d);
+        const uint32_t r = ((uint32_t)atomicOr(W.runs.rows, (int32_t)bit) | bit) & W.runs.mask;
+        const bool enough = __popc((r | r >> 8) & 0xffu) >= W.runs.need;
+        if (enough) W.runs.rows[1] = 1;
+        return enough;  // no merge will follow
+    });
     for (int i = tid; i < cnt; i += CH / E) {
         W.key[(int64_t)d * n + first + i] = s_full[i];
         W.id[(int64_t)d * n + first + i] = (uint32_t)(first + s_idx[i]);
@@ -297,6 +328,8 @@ __global__ void __launch_bounds__(32 * NW, 1) k_small_chunks(const T* __restrict
 // told apart by the other coordinates and the index (that of an earlier
 // chunk is smaller).
 constexpr int SMALL_WAYS = 4;  // chunks searched side by side
+// (Six blocks per SM: at five, of 48 registers, 65536 tuples of k = 3 over 16
+// values took 378 us, 319 at six.)
 template <typename T, typename KW>
 __global__ void __launch_bounds__(256) k_small_merge(const T* __restrict__ coords, int n, int k, int chunk,
                                                      const SmallWork<KW> W) {
@@ -307,7 +340,10 @@ __global__ void __launch_bounds__(256) k_small_merge(const T* __restrict__ coord
     const KW* key = W.key + (int64_t)d * n;
     const uint32_t* id = W.id + (int64_t)d * n;
     const KW x = key[q];
-    const int me = (int)id[q], mc = q / chunk, nc = (n + chunk - 1) / chunk;
+    const int me = (int)id[q], mc = q / chunk;
+    // (no chunks rather than a return, whose extra registers cost a block per SM:
+    // 196000 float32 tuples of k = 8 319 -> 380 us here)
+    const int nc = small_leave(W.runs) ? 0 : (n + chunk - 1) / chunk;
     auto before = [&](int other) {  // equal x_d: the other tuple precedes this one
         for (int r = 1; r < k; ++r) {
             const int c = d + r < k ? d + r : d + r - k;
@@ -317,7 +353,7 @@ __global__ void __launch_bounds__(256) k_small_merge(const T* __restrict__ coord
         return other < me;
     };
     int rank = q - mc * chunk;
-    bool dup = rank > 0 && key[q - 1] == x && small_equal(coords, k, (int)id[q - 1], me);
+    bool dup = nc > 0 && rank > 0 && key[q - 1] == x && small_equal(coords, k, (int)id[q - 1], me);
     for (int c0 = 0; c0 < nc; c0 += SMALL_WAYS) {
         int pos[SMALL_WAYS], len[SMALL_WAYS];
 #pragma unroll
@@ -357,6 +393,7 @@ __global__ void __launch_bounds__(256) k_small_compact(int n, int nchunks, const
     const int p0 = blockIdx.x * 1024, w0 = p0 / 32;
     pdl_wait();
     pdl_trigger();
+    if (small_leave(W.runs)) return;
     if (__syncthreads_or(tid < nchunks && W.nan[tid])) {
         if (d == 0 && blockIdx.x == 0 && tid == 0) {
             if (out.err) atomicOr(out.err, ERR_NAN);
@@ -463,7 +500,7 @@ static cudaError_t small_chunks_as(const void* coords, int n, int k, int narrays
 // barriers and scans are shorter); chunks above (work: small_work_words).
 template <typename T, typename KW>
 static cudaError_t small_sort_of(const void* coords, int n, int k, int narrays, uint32_t* work, const SmallOut& out,
-                                 cudaStream_t s) {
+                                 const SmallRuns& runs, cudaStream_t s) {
     if (n <= 256) return small_sort_as<T, KW, 8, 1>(coords, n, k, narrays, out, s);
     if (n <= 1024) return small_sort_as<T, KW, 8, 4>(coords, n, k, narrays, out, s);
     if (n <= SMALL_ONE) return small_sort_as<T, KW, 32, 2>(coords, n, k, narrays, out, s);
@@ -475,6 +512,7 @@ static cudaError_t small_sort_of(const void* coords, int n, int k, int narrays, 
     W.dup = W.raw + rows;
     W.words = small_dup_words(n);
     W.nan = W.dup + (int64_t)narrays * W.words;
+    W.runs = runs;
     const int chunk = small_chunk(n);
     cudaError_t e = chunk == 2048 ? small_chunks_as<T, KW, 32, 2>(coords, n, k, narrays, W, s)
                     : chunk == 4096 ? small_chunks_as<T, KW, 32, 4>(coords, n, k, narrays, W, s)
@@ -489,11 +527,11 @@ static cudaError_t small_sort_of(const void* coords, int n, int k, int narrays, 
 }
 
 static cudaError_t small_sort(int dtype, const void* coords, int n, int k, int narrays, uint32_t* work,
-                              const SmallOut& out, cudaStream_t s) {
+                              const SmallOut& out, const SmallRuns& runs, cudaStream_t s) {
     if (n < 1 || n > SMALL_MAX) return cudaErrorInvalidValue;
-    if (dtype == 0) return small_sort_of<int32_t, uint32_t>(coords, n, k, narrays, work, out, s);
-    if (dtype == 1) return small_sort_of<int64_t, uint64_t>(coords, n, k, narrays, work, out, s);
-    return small_sort_of<float, uint32_t>(coords, n, k, narrays, work, out, s);
+    if (dtype == 0) return small_sort_of<int32_t, uint32_t>(coords, n, k, narrays, work, out, runs, s);
+    if (dtype == 1) return small_sort_of<int64_t, uint64_t>(coords, n, k, narrays, work, out, runs, s);
+    return small_sort_of<float, uint32_t>(coords, n, k, narrays, work, out, runs, s);
 }
 
 // Kernels launched by one sort.
@@ -510,9 +548,29 @@ cudaError_t launch_small_arrays(int dtype, const void* coords, int n, int k, voi
     o.arr = reinterpret_cast<uint32_t*>(rows);
     o.arr_stride = n;
     o.m32 = m_out;
-    return small_sort(dtype, coords, n, k, k, static_cast<uint32_t*>(work), o, s);
+    return small_sort(dtype, coords, n, k, k, static_cast<uint32_t*>(work), o, SmallRuns{}, s);
 }
 
+// Which runs send a whole presort (all k arrays) back to the caller: the work
+// of the merge grows with the tuples, the chunks and the dimensions, that of
+// the digit passes hardly, and constant bytes save them passes.  Whole builds,
+// by digit passes and merged: 65536 int64 tuples of k = 8 over 2 values per
+// coordinate 0.63 and 1.72 ms (16 values 0.66 and 0.88, 64 values 0.65 and 0.71),
+// 196000 of k = 3 over 64 values 0.45 and 0.83, of k = 8 over 2 values 0.90 and
+// 6.89; 40000 of k = 8 over 16 values 0.66 and 0.58.  With three values in half
+// of the coordinates: 196000 of k = 6 0.75 and 1.45, 100000 float32 of k = 8 0.99
+// and 0.94.  Over 1000 values (short runs): 196000 int64 of k = 8 1.00 and 1.53,
+// 140000 float32 of k = 8 1.14 and 0.95.  What is left has cost its block sorts
+// and a read back, 0.06 to 0.1 ms.
+static SmallRuns small_runs(int n, int k, int32_t* rows) {
+    const int64_t nk = (int64_t)n * k;
+    const bool many = n > SMALL_MANY;
+    SmallRuns r{};
+    r.mask = k < 3 ? 0u : (nk > SMALL_LONG_RUNS ? 0xffu : 0u) | (many && nk > SMALL_RUNS ? 0xff00u : 0u);
+    r.need = many ? (k + 1) / 2 : k - 1;
+    r.rows = r.mask ? rows : nullptr;
+    return r;
+}
 // The handle of a small cloud: perm0, the rank records (rec, k >= 2) or, with
 // sel_keys, the key planes in array-0 order instead; m and the error bits.
 // work: small_presort_words words (the sort's, then the arrays and their
@@ -522,8 +580,8 @@ size_t small_presort_words(int dtype, int n, int k, bool all_arrays) {
            (all_arrays ? (size_t)2 * k * n : 0);
 }
 cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, uint32_t* work, const AllPlanes& rec,
-                                 uint32_t* perm0, void* sel_keys, int64_t sel_stride, int64_t* m_out, int* err,
-                                 cudaStream_t s) {
+                                 uint32_t* perm0, void* sel_keys, int64_t sel_stride, int64_t* m_out, int32_t* runs,
+                                 int* err, cudaStream_t s) {
     SmallOut o{};
     o.arr_stride = o.inv_stride = n;
     o.m64 = m_out;
@@ -531,7 +589,7 @@ cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, ui
     const unsigned blocks = (unsigned)((n + 255) / 256);
     if (sel_keys) {
         o.arr = perm0;
-        cudaError_t e = small_sort(dtype, coords, n, k, 1, work, o, s);
+        cudaError_t e = small_sort(dtype, coords, n, k, 1, work, o, SmallRuns{}, s);
         if (e != cudaSuccess) return e;
         if (dtype == 0)
             k_small_keys<int32_t, uint32_t><<<blocks, 256, 0, s>>>(m_out, k, (const int32_t*)coords, perm0,
@@ -546,7 +604,7 @@ cudaError_t launch_small_presort(int dtype, const void* coords, int n, int k, ui
     }
     o.arr = work + small_presort_words(dtype, n, k, true) - (size_t)2 * k * n;
     o.inv = o.arr + (size_t)k * n;
-    cudaError_t e = small_sort(dtype, coords, n, k, k, work, o, s);
+    cudaError_t e = small_sort(dtype, coords, n, k, k, work, o, small_runs(n, k, runs), s);
     if (e != cudaSuccess) return e;
     return launch_dependent(k_small_recs, dim3(blocks, k), dim3(256), 0, s, (const int64_t*)m_out, k,
                             (const uint32_t*)o.arr, (const uint32_t*)o.inv, (int64_t)n, rec, perm0);
