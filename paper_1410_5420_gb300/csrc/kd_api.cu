@@ -669,7 +669,8 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
     // 196608 492 -> 408 and 881 -> 649; the merge of the chunks grows with the
     // square of their number.
     kd_cloud there{};  // the cloud's copy on the device
-    if (count == 1 && N <= small_presort_max()) {
+    // (The injected wait needs the digit passes: the block sorts have none.)
+    if (count == 1 && N <= small_presort_max() && !ctx->inject_timeout) {
         there = clouds[0];
         if (!there.on_device) {
             unsigned char* cb = nullptr;
@@ -688,7 +689,6 @@ kd_status presort_batch(kd_ctx* ctx, const kd_cloud* clouds, int count, kd_preso
             CK(launch_small_presort(dtype, there.coords, (int)N, k, work, H->rec, H->perm0, H->sel_keys, pad4(N), H->d_m,
                                     d_info->runs, d_err, s));
         }
-        ctx->inject_timeout = false;  // (no look-back to withhold a flag from)
         const unsigned char* h = nullptr;
         InfoBlock info;
         CKS(fetch(ctx, d_info, sizeof(info), &h));
