@@ -57,8 +57,9 @@ typedef struct {
     int device;              /* CUDA device ordinal */
     void *cuda_stream;       /* cudaStream_t to order work on; NULL: the library makes its own */
     size_t mem_budget_bytes; /* cap on the library's device workspace; 0: no cap */
-    int level_tile;          /* positions per level-step tile: 1024, or 2048 (k <= 4); 0: tuned, else 2048 for
-                                k <= 4 and 1024 above */
+    int level_tile;          /* positions per level-step tile: 1024, or 2048 (k <= 4); 0: builds of at most
+                                2^21 tuples in all take steps of one launch on tiles of 1024, larger ones
+                                the tuned tile, else 2048 for k <= 4 and 1024 above */
     int switch_threshold;    /* subtree size finished on chip (rounded up to 1024, 2048 or 4096, capped by k);
                                 0: tuned, else 1024 */
     int debug;               /* bit 1: synchronise after the presort; bit 2: time every launch
@@ -196,10 +197,12 @@ kd_status kd_serving_stats(kd_ctx *ctx, int64_t *completed, double *p50_us, doub
  * allows) and the level-step tile (1024 or 2048 positions) are chosen per
  * (k, dtype, size bucket = floor(log2 n) of the largest cloud of a build).
  * kd_autotune presorts a synthetic cloud of n tuples (uniform coordinates,
- * generated on the device), times kd_build with every candidate pair (reps
+ * generated on the device), times kd_build with the candidate pairs (reps
  * runs each, median of CUDA-event times on the context's stream), records
  * the fastest for the bucket in the context, rewrites cfg->tune_cache when
- * one was given, and returns it.  Later builds whose bucket has an entry use
+ * one was given, and returns it.  (Up to 2^21 tuples: the fastest subtree size
+ * with the steps such a build takes, and the fastest tile for the batches of
+ * such clouds that exceed 2^21 tuples in all.)  Later builds whose bucket has an entry use
  * it unless cfg->switch_threshold or cfg->level_tile fix a value.  Every
  * candidate builds the same tree.  Errors: KD_EINVAL (k, n, dtype or reps
  * out of range), KD_ENOMEM, KD_EDEVICE.  Synchronises the stream.
@@ -208,7 +211,8 @@ kd_status kd_autotune(kd_ctx *ctx, int k, kd_dtype dtype, int64_t n, int reps, i
                       int *level_tile_out);
 
 /* The subtree size and level tile a build of clouds of at most n tuples
- * (k, dtype) would use on this context now. */
+ * (k, dtype) would use on this context now (the tile: of a build of more than
+ * 2^21 tuples in all, or where cfg->level_tile fixes it). */
 kd_status kd_tuning_get(kd_ctx *ctx, int k, kd_dtype dtype, int64_t n, int *switch_threshold_out,
                         int *level_tile_out);
 

@@ -197,7 +197,6 @@ struct kd_ctx {
     std::string tune_cache;
     int force_smax = 0, force_ltile = 0;  // the candidate kd_autotune is timing
     int schedule = KD_SCHEDULE_MULTI;     // level schedule (kd_config.schedule)
-    int last_smax = 0, last_ltile = 0;    // what the last build used
     // Failure-detection tests (debug bit 8): the look-back polls are bounded
     // by a few thousand instead of 2^24, and the next presort's first sort
     // pass has its chunk 0 withhold its flag (once), so that the other
@@ -1402,10 +1401,9 @@ kd_status build_batch(kd_ctx* ctx, kd_presorted* H, kd_tree* outs) {
         for (int i = 0; i < count; ++i) nmax = std::max(nmax, H->n_c[i]);
         choose_params(ctx, k, H->dtype, nmax, &smax, &tile);
     }
-    ctx->last_smax = smax;
-    ctx->last_ltile = tile;
-    // few tuples: every level step is one launch
-    const bool small_steps = level_steps_small(M);
+    // few tuples: every level step is one launch, of its own tile, unless the
+    // context fixes one (or the autotuner times it)
+    const bool small_steps = level_steps_small(M) && !ctx->level_tile_override && !ctx->force_ltile;
     if (small_steps) tile = level_small_tile();
     if (k >= 2 && smax * 3 < tile + 3) return fail(ctx, KD_EINVAL, "switch threshold too small");
 
@@ -2241,42 +2239,64 @@ kd_status kd_autotune(kd_ctx* ctx, int k, kd_dtype dtype, int64_t n, int reps, i
         CKS(S.get(&right, (size_t)n * 4));
         CKS(S.get(&dim, (size_t)n));
         cudaEvent_t e0 = take_event(ctx), e1 = take_event(ctx);
-        double best = 1e30;
         int bsm = 1024, blt = level_tile(k);
+        // median time of a build with subtrees of sm and tiles of lt (0: those a
+        // build takes without a fixed tile)
+        auto timed = [&](int sm, int lt, double* med) -> kd_status {
+            ctx->force_smax = sm;
+            ctx->force_ltile = lt;
+            std::vector<float> ms;
+            kd_status st = KD_OK;
+            for (int r = 0; r <= reps && st == KD_OK; ++r) {  // the first run is a warm-up
+                kd_tree t{0, -1, node, left, right, dim, 1};
+                cudaEventRecord(e0, ctx->stream);
+                st = build_batch(ctx, H, &t);
+                cudaEventRecord(e1, ctx->stream);
+                if (st == KD_OK && r > 0) {
+                    cudaEventSynchronize(e1);
+                    float x = 0;
+                    cudaEventElapsedTime(&x, e0, e1);
+                    ms.push_back(x);
+                }
+            }
+            ctx->force_smax = ctx->force_ltile = 0;
+            if (st != KD_OK) return st;
+            std::sort(ms.begin(), ms.end());
+            *med = ms[ms.size() / 2];
+            return KD_OK;
+        };
+        // The fastest pair; where a build's steps are one launch each, whatever
+        // the tile, the fastest subtree with those and its fastest tile.
+        const bool one_launch = level_steps_small(H->M) && !ctx->level_tile_override;
+        double best = 1e30, best_tile = 1e30;
+        kd_status st = KD_OK;
         for (int sm : {1024, 2048, 4096}) {
             if (k > finish_kmax(sm)) continue;
+            double med = 1e30;
+            if (one_launch) {
+                st = timed(sm, 0, &med);
+                if (st != KD_OK) break;
+                if (med >= best) continue;
+                best = med;
+                best_tile = 1e30;
+            }
             for (int lt : {1024, 2048}) {
                 if (!level_tile_supported(k, lt) || sm * 3 < lt + 3) continue;
-                ctx->force_smax = sm;
-                ctx->force_ltile = lt;
-                std::vector<float> ms;
-                kd_status st = KD_OK;
-                for (int r = 0; r <= reps && st == KD_OK; ++r) {  // the first run is a warm-up
-                    kd_tree t{0, -1, node, left, right, dim, 1};
-                    cudaEventRecord(e0, ctx->stream);
-                    st = build_batch(ctx, H, &t);
-                    cudaEventRecord(e1, ctx->stream);
-                    if (st == KD_OK && r > 0) {
-                        cudaEventSynchronize(e1);
-                        float x = 0;
-                        cudaEventElapsedTime(&x, e0, e1);
-                        ms.push_back(x);
-                    }
-                }
-                ctx->force_smax = ctx->force_ltile = 0;
-                if (st != KD_OK) {
-                    ctx->event_pool.push_back(e0);
-                    ctx->event_pool.push_back(e1);
-                    return st;
-                }
-                std::sort(ms.begin(), ms.end());
-                const double med = ms[ms.size() / 2];
-                if (med < best) {
-                    best = med;
+                st = timed(sm, lt, &med);
+                if (st != KD_OK) break;
+                if (med < best_tile) {
+                    best_tile = med;
                     bsm = sm;
                     blt = lt;
                 }
             }
+            if (st != KD_OK) break;
+        }
+        if (!one_launch) best = best_tile;
+        if (st != KD_OK) {
+            ctx->event_pool.push_back(e0);
+            ctx->event_pool.push_back(e1);
+            return st;
         }
         ctx->event_pool.push_back(e0);
         ctx->event_pool.push_back(e1);
