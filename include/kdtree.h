@@ -56,7 +56,9 @@ typedef enum { KD_I32 = 0, KD_I64 = 1, KD_F32 = 2 } kd_dtype;
 typedef struct {
     int device;              /* CUDA device ordinal */
     void *cuda_stream;       /* cudaStream_t to order work on; NULL: the library makes its own */
-    size_t mem_budget_bytes; /* cap on the library's device workspace; 0: no cap */
+    size_t mem_budget_bytes; /* cap on the library's device workspace, counted in the bytes asked for and
+                                those kept for reuse (from 1 GiB on, blocks of up to 1 MiB may be up to
+                                twice as large, and the driver's pools round up); 0: no cap */
     int level_tile;          /* positions per level-step tile: 1024, or 2048 (k <= 4); 0: builds of at most
                                 2^21 tuples in all take steps of one launch on tiles of 1024, larger ones
                                 the tuned tile, else 2048 for k <= 4 and 1024 above */

@@ -151,15 +151,19 @@ struct Request;
 // a pool of their own: kept between the large blocks they split that pool's
 // free memory, which the driver then mapped anew on each call (2^26 tuples,
 // presorted and built with the handle held: 27.2 ms a step against 20.9).
+// Under a memory budget the kept blocks count and go first; one below
+// ROUND_BUDGET, of which the rounding of the live blocks (some 10 MB at most)
+// could be a good part, takes blocks of the sizes asked for.
 constexpr size_t SMALL_BLOCK = (size_t)1 << 20;
-constexpr int SMALL_CLASSES = 13;  // 256 bytes ... SMALL_BLOCK
 constexpr size_t SMALL_KEPT = (size_t)32 << 20;
+constexpr size_t SMALL_SIZES = 64;
+constexpr size_t ROUND_BUDGET = (size_t)1 << 30;
 constexpr size_t PINNED_BYTES = (size_t)256 << 10;
 
-int small_class(size_t bytes) {
-    int c = 0;
-    while (((size_t)256 << c) < bytes) ++c;
-    return c;
+size_t small_round(size_t bytes) {
+    size_t b = 256;
+    while (b < bytes) b *= 2;
+    return b;
 }
 
 }  // namespace
@@ -183,7 +187,7 @@ struct kd_ctx {
     cudaMemPool_t pool = nullptr;
     cudaMemPool_t small_pool = nullptr;  // blocks of at most SMALL_BLOCK bytes
     size_t budget = 0;
-    size_t in_use = 0;
+    size_t in_use = 0;  // bytes asked for and not freed
     int debug = 0;
     int smax_override = 0;
     int level_tile_override = 0;
@@ -206,10 +210,13 @@ struct kd_ctx {
     bool inject_level_timeout = false;  // bit 16: the same for the next build's first level step
     std::string last_error;
     std::recursive_mutex mu;
-    std::unordered_map<void*, size_t> sizes;
-    // freed blocks of at most SMALL_BLOCK bytes, by power of two, for the next
-    // allocations on this stream (at most SMALL_KEPT bytes in all)
-    std::vector<void*> small_free[SMALL_CLASSES];
+    struct Block {
+        size_t asked, size;
+    };
+    std::unordered_map<void*, Block> blocks;
+    // freed blocks of at most SMALL_BLOCK bytes, by size, for the next
+    // allocations on this stream (at most SMALL_KEPT bytes and SMALL_SIZES sizes)
+    std::vector<std::pair<size_t, std::vector<void*>>> small_free;
     size_t small_kept = 0;
     std::atomic<int64_t> launches{0};
     // kernel timing (debug bit 2)
@@ -275,12 +282,18 @@ kd_status fail(kd_ctx* ctx, kd_status code, const std::string& msg) {
         if (_s != KD_OK) return _s;                                                                \
     } while (0)
 
+// The kept small blocks of one size (nullptr: none so far).
+std::vector<void*>* small_list(kd_ctx* ctx, size_t size) {
+    for (auto& v : ctx->small_free)
+        if (v.first == size) return &v.second;
+    return nullptr;
+}
+
 // The kept small blocks back to the pool.
 void small_release(kd_ctx* ctx) {
-    for (auto& v : ctx->small_free) {
-        for (void* p : v) cudaFreeAsync(p, ctx->stream);
-        v.clear();
-    }
+    for (auto& v : ctx->small_free)
+        for (void* p : v.second) cudaFreeAsync(p, ctx->stream);
+    ctx->small_free.clear();
     ctx->small_kept = 0;
 }
 
@@ -288,28 +301,30 @@ kd_status dev_alloc(kd_ctx* ctx, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return KD_OK;
     bytes = (bytes + 255) & ~(size_t)255;
+    const bool small = bytes <= SMALL_BLOCK;
+    const size_t size = small && (!ctx->budget || ctx->budget >= ROUND_BUDGET) ? small_round(bytes) : bytes;
     if (ctx->budget && ctx->in_use + bytes > ctx->budget)
         return fail(ctx, KD_ENOMEM, "device memory budget exceeded (" + std::to_string(ctx->in_use + bytes) +
                                         " > " + std::to_string(ctx->budget) + " bytes)");
-    const bool small = bytes <= SMALL_BLOCK;
-    const int c = small ? small_class(bytes) : 0;
-    if (small && !ctx->small_free[c].empty()) {
-        *p = ctx->small_free[c].back();
-        ctx->small_free[c].pop_back();
-        ctx->small_kept -= (size_t)256 << c;
+    std::vector<void*>* const kept = small ? small_list(ctx, size) : nullptr;
+    if (kept && !kept->empty()) {
+        *p = kept->back();
+        kept->pop_back();
+        ctx->small_kept -= size;
     } else {
+        if (ctx->budget && ctx->in_use + ctx->small_kept + bytes > ctx->budget) small_release(ctx);
         cudaMemPool_t pool = small ? ctx->small_pool : ctx->pool;
-        cudaError_t e = cudaMallocFromPoolAsync(p, small ? (size_t)256 << c : bytes, pool, ctx->stream);
+        cudaError_t e = cudaMallocFromPoolAsync(p, size, pool, ctx->stream);
         if (e == cudaErrorMemoryAllocation && ctx->small_kept) {  // once more without the kept blocks
             cudaGetLastError();
             small_release(ctx);
             cudaStreamSynchronize(ctx->stream);
             cudaMemPoolTrimTo(ctx->small_pool, 0);
-            e = cudaMallocFromPoolAsync(p, small ? (size_t)256 << c : bytes, pool, ctx->stream);
+            e = cudaMallocFromPoolAsync(p, size, pool, ctx->stream);
         }
         if (e == cudaErrorMemoryAllocation && small) {  // from what the large blocks' pool holds
             cudaGetLastError();
-            e = cudaMallocFromPoolAsync(p, (size_t)256 << c, ctx->pool, ctx->stream);
+            e = cudaMallocFromPoolAsync(p, size, ctx->pool, ctx->stream);
         }
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -318,24 +333,30 @@ kd_status dev_alloc(kd_ctx* ctx, void** p, size_t bytes) {
         }
     }
     ctx->in_use += bytes;
-    ctx->sizes[*p] = bytes;
+    ctx->blocks[*p] = {bytes, size};
     return KD_OK;
 }
 
 void dev_free(kd_ctx* ctx, void* p) {
     if (!p) return;
-    auto it = ctx->sizes.find(p);
-    if (it != ctx->sizes.end()) {
-        const size_t bytes = it->second;
-        ctx->in_use -= bytes;
-        ctx->sizes.erase(it);
-        if (bytes <= SMALL_BLOCK) {
-            const int c = small_class(bytes);
-            if (ctx->small_kept + ((size_t)256 << c) <= SMALL_KEPT) {
-                ctx->small_free[c].push_back(p);  // its users so far precede the next user on the stream
-                ctx->small_kept += (size_t)256 << c;
-                return;
+    auto it = ctx->blocks.find(p);
+    if (it != ctx->blocks.end()) {
+        const size_t size = it->second.size;
+        ctx->in_use -= it->second.asked;
+        ctx->blocks.erase(it);
+        if (size <= SMALL_BLOCK) {
+            std::vector<void*>* kept = small_list(ctx, size);
+            if (ctx->small_kept + size > SMALL_KEPT || (!kept && ctx->small_free.size() == SMALL_SIZES)) {
+                small_release(ctx);
+                kept = nullptr;
             }
+            if (!kept) {
+                ctx->small_free.push_back({size, {}});
+                kept = &ctx->small_free.back().second;
+            }
+            kept->push_back(p);  // its users so far precede the next user on the stream
+            ctx->small_kept += size;
+            return;
         }
     }
     cudaFreeAsync(p, ctx->stream);
