@@ -1405,7 +1405,6 @@ __global__ void __launch_bounds__(FIN_THREADS, fin_min_blocks(SMAX, K))
         // (a segment of at most 32 tuples is done in six levels; ranks that
         // contradict each other, from inconsistent inputs, would leave a lane
         // active for ever: its node stays unset and is reported below)
-#pragma unroll 1
         for (int l = 0; l < 6 && __any_sync(0xffffffffu, active); ++l, p = p + 1 == K ? 0 : p + 1) {
             uint32_t lp = 0;
 #pragma unroll
