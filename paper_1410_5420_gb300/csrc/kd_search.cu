@@ -1044,8 +1044,10 @@ struct CallScratch {
     kd_ctx* ctx;
     std::vector<void*> ptrs;
     explicit CallScratch(kd_ctx* c) : ctx(c) {}
-    ~CallScratch() {
+    ~CallScratch() { clear(); }
+    void clear() {
         for (void* p : ptrs) kd::ctx_free(ctx, p);
+        ptrs.clear();
     }
     kd_status get(void** p, size_t bytes) {
         kd_status s = kd::ctx_alloc(ctx, p, bytes);
@@ -1457,14 +1459,15 @@ kd_status kd_region(kd_ctx* ctx, kd_index ix, const void* lo, const void* hi, in
     if (st == KD_OK) st = S.get((void**)&d_err, sizeof(int));
     if (st != KD_OK) return st;
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
-    const uint32_t* order = region_order(ctx, ix, S, dlo, nq, s);
+    CallScratch O(ctx);  // what the walks only go faster with
+    const uint32_t* order = region_order(ctx, ix, O, dlo, nq, s);
     // where the indices of many boxes are wanted, the first of every box are
     // kept (if they fit), then the list of the boxes that have more and its
     // length.  (Of few boxes, some have more, and the second walk takes as
     // long for them as for all.)
     int32_t* kept = nullptr;
     if (idx_out && nq >= KEEP_MIN_BOXES && nq <= UINT32_MAX &&
-        S.get((void**)&kept, ((size_t)nq * (REGION_KEEP + 1) + 1) * 4) != KD_OK)
+        O.get((void**)&kept, ((size_t)nq * (REGION_KEEP + 1) + 1) * 4) != KD_OK)
         sfail(ctx, KD_OK, "");
     uint32_t* list = kept ? (uint32_t*)kept + (size_t)nq * REGION_KEEP : nullptr;
     if (list) cudaMemsetAsync(list + nq, 0, 4, s);
@@ -1482,6 +1485,14 @@ kd_status kd_region(kd_ctx* ctx, kd_index ix, const void* lo, const void* hi, in
         int32_t* dout = idx_out;
         if (!on_device) {
             st = S.get((void**)&dout, (size_t)total * 4);
+            if (st == KD_ENOMEM && (order || kept)) {  // the indices before what speeds their search up
+                O.clear();
+                order = nullptr;
+                kept = nullptr;
+                list = nullptr;
+                st = S.get((void**)&dout, (size_t)total * 4);
+                if (st == KD_OK) sfail(ctx, KD_OK, "");
+            }
             if (st != KD_OK) return st;
         }
         if (list) {
