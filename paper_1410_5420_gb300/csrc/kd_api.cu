@@ -81,7 +81,6 @@ cudaError_t launch_sel_level(int key64, void* const* id, void* const* key, int c
 cudaError_t launch_sel_order(int key64, void* const* id, void* const* key, int cur, int k, int32_t m, int lam,
                              uint32_t** plane, uint32_t** perm, int* err, cudaStream_t s);
 bool level_tile_supported(int k, int tile);
-int level_status_stride(int k);
 cudaError_t launch_level_pass(int k, int tile, const AllBufs& bufs, int q, const LevelJob* jobs, int njobs, int ntiles,
                               const CloudDev* clouds, uint32_t* medr, const uint32_t* perm0, uint32_t* status,
                               int* err, cudaStream_t s, uint32_t spin_limit, int withhold);

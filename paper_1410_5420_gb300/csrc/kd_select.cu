@@ -34,7 +34,7 @@
 namespace kd {
 
 constexpr int SEL_THREADS = 256;
-constexpr int SEL_TILE = 2048;   // largest tile of the level kernels (positions)
+constexpr int SEL_TILE = 2048;   // tile of the level kernels (positions)
 constexpr int SEL_IPT = SEL_TILE / SEL_THREADS;
 constexpr uint32_t KNONE = 0xffffffffu;
 constexpr int SEL_RUN = 32;  // longest run of equal sort words ordered by compares
@@ -660,8 +660,8 @@ static cudaError_t sel_level(const SelBufs<KW>& B, int cur, int k, int32_t m, in
 }
 
 // One level of the selection build over every segment of level L, in tiles
-// of `tile` positions (a tile must touch at most LEVEL_NSMAX segments: with
-// segments of at least 1024 tuples, 2048).
+// of `tile` = SEL_TILE positions (a tile must touch at most LEVEL_NSMAX
+// segments, so these hold at least 1024 tuples).
 // phase 0: reset the segments' state; 3: the shared leading bytes of every
 // segment (*unresolved, as an int32, receives the smallest first byte to
 // select; it must hold the byte count before); 1: selection rounds
@@ -671,7 +671,7 @@ cudaError_t launch_sel_level(int key64, void* const* id, void* const* key, int c
                              void* segs, uint32_t* ghist, int32_t* gany, uint32_t* unresolved, int32_t* node,
                              int64_t in_off, int* err, cudaStream_t s, int round_begin, int round_end, int phase) {
     if (m <= 0) return cudaSuccess;
-    if (tile != SEL_TILE && tile != SEL_TILE / 2) return cudaErrorInvalidValue;
+    if (tile != SEL_TILE) return cudaErrorInvalidValue;
     if (key64)
         return sel_level<uint64_t>(sel_bufs<uint64_t>(id, key, k), cur, k, m, L, tile, segs, ghist, gany, unresolved,
                                    node, in_off, err, s, round_begin, round_end, phase);
