@@ -59,6 +59,7 @@ struct kd_index_s {
     int64_t box_off[5] = {};  // level l: first word in boxes ...
     int32_t nbox[5] = {};     // ... and number of boxes
     int top = 0;
+    bool dense = false;  // integers that fill a good part of their range (index_dense)
 };
 
 namespace {
@@ -1118,6 +1119,19 @@ void index_fill(kd_ctx* ctx, kd_index_s* ix, const void* coords, int64_t n, int*
     }
 }
 
+// Whether the m tuples of a plane fill at least a quarter of the integer points
+// of their range, from the top level's boxes (b: one group, on the host).
+template <typename T>
+bool index_dense(const kd_index_s* ix, const T* b) {
+    double points = 1.0;
+    for (int d = 0; d < 2; ++d) {
+        const T lo = *std::min_element(b + d * BOX_W, b + d * BOX_W + ix->nbox[ix->top]);
+        const T hi = *std::max_element(b + (2 + d) * BOX_W, b + (2 + d) * BOX_W + ix->nbox[ix->top]);
+        points *= (double)hi - (double)lo + 1.0;
+    }
+    return points <= 4.0 * (double)ix->m;
+}
+
 template <typename T, int K>
 void knn_as(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err, bool exact,
             cudaStream_t s) {
@@ -1171,10 +1185,24 @@ void cells_as(kd_index_s* ix, int levels, const void* lo, int64_t nq, uint32_t* 
         default: NAME<T, MAXK>(__VA_ARGS__); break;               \
     }
 
+// Searches of few neighbours that one thread each answers faster than one warp
+// each: over one dimension, whose split planes are its distances, or over a
+// plane whose points fill it, where the boxes touch and tie.  One nearest and
+// two nearest of each of 2^20 tuples, by warps and by threads: k = 1 int32 0.92
+// and 0.66, 0.93 and 0.74 ms (four nearest 0.97 and 0.96, of half-filled
+// integers 0.87 and 0.75, of float32 1.09 and 1.19; 4096 tuples 0.05 and 0.09),
+// a half-filled lattice of k = 2 1.84 and 1.38, 2.04 and 1.58 (four nearest 2.40
+// and 2.00; eight 0.36 and 0.49 at 2^17), spread int32 of k = 2 0.68 and 1.49.
+constexpr int64_t WALK_MIN_QUERIES = 1 << 16;
+bool knn_by_walk(const kd_index_s* ix, int64_t nq, int kn) {
+    if (!ix->boxes) return true;
+    return nq >= WALK_MIN_QUERIES && (ix->k == 1 || ix->dense) && kn <= (ix->dtype == KD_F32 ? 2 : 4);
+}
+
 template <typename T>
 void knn_of(kd_index_s* ix, const void* queries, int64_t nq, int kn, int32_t* di, double* dd, int* err, bool exact,
             cudaStream_t s) {
-    if (ix->m > 0 && !ix->boxes)  // (a thread per query, so a grid that no cap of grid_of cuts)
+    if (ix->m > 0 && knn_by_walk(ix, nq, kn))  // (a thread per query, so a grid that no cap of grid_of cuts)
         k_knn_walk<T><<<(unsigned)((nq + SEARCH_THREADS - 1) / SEARCH_THREADS), SEARCH_THREADS, 0, s>>>(
             (const T*)ix->pts, ix->m, ix->node_tuple, (int32_t)ix->m, ix->k, (const T*)queries, nq, kn, di, dd, err);
     else
@@ -1308,11 +1336,19 @@ kd_status kd_index_create(kd_ctx* ctx, const kd_cloud* cloud, const kd_tree* tre
     if (ix->dtype == KD_I32) index_fill<int32_t>(ctx, ix.get(), coords, cloud->n, d_err, s);
     else if (ix->dtype == KD_I64) index_fill<int64_t>(ctx, ix.get(), coords, cloud->n, d_err, s);
     else index_fill<float>(ctx, ix.get(), coords, cloud->n, d_err, s);
+    const bool plane = ix->boxes && ix->k == 2 && ix->dtype != KD_F32;
+    int64_t range[4 * BOX_W];
+    if (plane)
+        cudaMemcpyAsync(range, (const char*)ix->boxes + ix->box_off[ix->top] * ts, 4 * BOX_W * ts,
+                        cudaMemcpyDeviceToHost, s);
     st = read_err(ctx, d_err, s);
     if (st != KD_OK) {
         kd_index_destroy(ctx, ix.release());
         return st;
     }
+    if (plane)
+        ix->dense = ix->dtype == KD_I32 ? index_dense(ix.get(), reinterpret_cast<const int32_t*>(range))
+                                        : index_dense(ix.get(), range);
     *out = ix.release();
     return KD_OK;
 }
@@ -1421,7 +1457,8 @@ kd_status kd_reverse_knn(kd_ctx* ctx, kd_index ix, int kn, int on_device, int64_
     cudaMemsetAsync(inv, 0xff, (size_t)n * 4, s);
     cudaMemsetAsync(cnt, 0, (size_t)m * 8, s);
     launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, false, s);
-    if (ix->boxes) launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, true, s);  // (finds none to do, mostly)
+    if (!knn_by_walk(ix, m, kn))
+        launch_knn(ctx, ix, nullptr, m, kn, nn, nullptr, d_err, true, s);  // (finds none to do, mostly)
     k_inv_map<<<grid_of(m, 256), 256, 0, s>>>(ix->node_tuple, m, n, inv, d_err);
     k_rev_count<<<grid_of(total, 256), 256, 0, s>>>(nn, total, inv, n, cnt, d_err);
     launch_offsets(ctx, cnt, m, cursor, offs, s);  // (the cursors' words hold the chunk sums meanwhile)
