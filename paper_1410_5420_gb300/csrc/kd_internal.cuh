@@ -87,7 +87,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // may start while the previous kernel on its stream is still running; it
 // calls pdl_wait() before its first global-memory access, which returns once
 // that kernel has completed and its writes are visible (at once when the
-// kernel was launched without the attribute).  pdl_trigger() lets the
+// kernel was launched without the attribute).  (k_level_small reads tables
+// before it, from its second launch on; it says why it may.)  pdl_trigger() lets the
 // dependent grid launch as soon as every block of this grid has issued it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

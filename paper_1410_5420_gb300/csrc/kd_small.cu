@@ -34,6 +34,9 @@ constexpr int SMALL_MANY = 150000;
 constexpr int64_t SMALL_RUNS = 1100000;
 // Chunks of 2048 tuples up to 16384, 4096 up to 65536, 8192 above: a block's
 // sort takes longer with its chunk, the merge with the number of chunks.
+// Presorts of k = 3: 16384 float32 in chunks of 2048 52 us, of 4096 60; 30000
+// int64 74 and 63; 40000 int64 in chunks of 4096 74, of 8192 87; 100000 float32
+// 130 and 112.
 __host__ __device__ constexpr int small_chunk(int n) { return n <= 16384 ? 2048 : (n <= 65536 ? 4096 : 8192); }
 
 // Key of a coordinate (floats are checked for NaN before).
