@@ -43,7 +43,7 @@ __device__ __forceinline__ int cloud_of(const P* start, int lo, int hi, Q p) {
 // hist layout: row (d * D + b) for coordinate d, key byte b; then rows
 // (k * D + b) for the cloud-id plane of a batch.  Dynamic smem: the block's
 // histogram rows followed by a 256-point staging tile of coordinates.
-template <typename T, typename KW>
+template <typename T, typename KW, bool BATCH>
 __global__ void __launch_bounds__(256) k_transform(const T* __restrict__ coords, int64_t n, int k,
                                                    KW* __restrict__ keys, int64_t stride, KW* __restrict__ tail,
                                                    const int64_t* __restrict__ cloud_start, int ncloud,
@@ -55,27 +55,28 @@ __global__ void __launch_bounds__(256) k_transform(const T* __restrict__ coords,
     const int nrows = k * D + cloud_digits;
     uint32_t* sh = smem;
     T* sc = reinterpret_cast<T*>(smem + nrows * RADIX);
-    __shared__ int s_cloud[2];  // the 256 points' clouds lie between these
+    __shared__ int s_cloud[2];  // a batch: the 256 points' clouds lie between these
     const int tid = threadIdx.x;
     for (int i = tid; i < nrows * RADIX; i += 256) sh[i] = 0;
     int nan = 0;
     // A batch: the block's tiles are consecutive, so that each tile's clouds are
     // found from the last one's (38.9 million tuples in 4096 clouds: 599 -> 384
     // us).  One cloud: the blocks' tiles alternate, so that the blocks read and
-    // write side by side (2^26 tuples: 486 us, consecutive 553).
+    // write side by side (2^26 tuples: 482 us, consecutive 553, and 553 where the
+    // kernel chooses between the two at run time).
     const int64_t tiles = (n + 255) / 256;
-    int64_t base = (int64_t)blockIdx.x * 256, past = n, stride_pts = (int64_t)gridDim.x * 256;
-    if (ncloud > 1) {
+    int64_t base = (int64_t)blockIdx.x * 256, past = n;
+    const int64_t stride_pts = BATCH ? 256 : (int64_t)gridDim.x * 256;
+    if constexpr (BATCH) {
         base = tiles * blockIdx.x / gridDim.x * 256;
         past = min(tiles * (blockIdx.x + 1) / gridDim.x * 256, n);
-        stride_pts = 256;
         if (tid == 0) s_cloud[1] = cloud_of(cloud_start, 0, ncloud, base);
     }
     __syncthreads();
     for (; base < past; base += stride_pts) {
         const int cnt = (int)(n - base < 256 ? n - base : 256);
         for (int i = tid; i < cnt * k; i += 256) sc[i] = coords[base * k + i];
-        if (ncloud > 1 && tid == 0) {
+        if (BATCH && tid == 0) {
             int lo = s_cloud[1], hi = lo + 1;
             s_cloud[0] = lo;
             for (int step = 1; hi < ncloud && cloud_start[hi] <= base + cnt - 1; step *= 2) {
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(256) k_transform(const T* __restrict__ coords,
                 for (int b = 0; b < D; ++b)
                     atomicAdd(&sh[(d * D + b) * RADIX + (uint32_t)((key >> (8 * b)) & 255u)], 1u);
             }
-            if (ncloud > 1) {
+            if constexpr (BATCH) {
                 const int c = cloud_of(cloud_start, s_cloud[0], s_cloud[1] + 1, p);
                 cloud_plane[p] = (uint32_t)c;
                 for (int b = 0; b < cloud_digits; ++b)
@@ -1816,15 +1817,17 @@ cudaError_t launch_transform(int dtype, const void* coords, int64_t n, int k, vo
     const size_t smem = (size_t)(k * D + cloud_digits) * RADIX * 4 + 256 * k * tsz;
     if (smem > TRANSFORM_SMEM_MAX) return cudaErrorInvalidValue;
     const int grid = grid_for(n, 256, 152 * 8);
-    if (dtype == 0)
-        k_transform<int32_t, uint32_t><<<grid, 256, smem, s>>>((const int32_t*)coords, n, k, (uint32_t*)keys, stride,
-                                                              (uint32_t*)tail, cloud_start, ncloud, cloud_plane, cloud_digits, hist, err);
-    else if (dtype == 1)
-        k_transform<int64_t, uint64_t><<<grid, 256, smem, s>>>((const int64_t*)coords, n, k, (uint64_t*)keys, stride,
-                                                              (uint64_t*)tail, cloud_start, ncloud, cloud_plane, cloud_digits, hist, err);
-    else
-        k_transform<float, uint32_t><<<grid, 256, smem, s>>>((const float*)coords, n, k, (uint32_t*)keys, stride,
-                                                            (uint32_t*)tail, cloud_start, ncloud, cloud_plane, cloud_digits, hist, err);
+#define KD_TRANSFORM(T, KW, BATCH)                                                                                  \
+    k_transform<T, KW, BATCH><<<grid, 256, smem, s>>>((const T*)coords, n, k, (KW*)keys, stride, (KW*)tail,          \
+                                                      cloud_start, ncloud, cloud_plane, cloud_digits, hist, err)
+    const bool batch = ncloud > 1;
+    if (dtype == 0 && batch) KD_TRANSFORM(int32_t, uint32_t, true);
+    else if (dtype == 0) KD_TRANSFORM(int32_t, uint32_t, false);
+    else if (dtype == 1 && batch) KD_TRANSFORM(int64_t, uint64_t, true);
+    else if (dtype == 1) KD_TRANSFORM(int64_t, uint64_t, false);
+    else if (batch) KD_TRANSFORM(float, uint32_t, true);
+    else KD_TRANSFORM(float, uint32_t, false);
+#undef KD_TRANSFORM
     return cudaGetLastError();
 }
 
@@ -1951,9 +1954,12 @@ cudaError_t init_presort_kernels() {
     auto set = [&](const void* f, size_t bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    set((const void*)k_transform<int32_t, uint32_t>, TRANSFORM_SMEM_MAX);
-    set((const void*)k_transform<int64_t, uint64_t>, TRANSFORM_SMEM_MAX);
-    set((const void*)k_transform<float, uint32_t>, TRANSFORM_SMEM_MAX);
+    set((const void*)k_transform<int32_t, uint32_t, false>, TRANSFORM_SMEM_MAX);
+    set((const void*)k_transform<int32_t, uint32_t, true>, TRANSFORM_SMEM_MAX);
+    set((const void*)k_transform<int64_t, uint64_t, false>, TRANSFORM_SMEM_MAX);
+    set((const void*)k_transform<int64_t, uint64_t, true>, TRANSFORM_SMEM_MAX);
+    set((const void*)k_transform<float, uint32_t, false>, TRANSFORM_SMEM_MAX);
+    set((const void*)k_transform<float, uint32_t, true>, TRANSFORM_SMEM_MAX);
     set((const void*)k_run_tiles<uint32_t, 0>, run_tile_smem(0, MAXK - 1));
     set((const void*)k_run_tiles<uint32_t, 1>, run_tile_smem(0, 1));
     set((const void*)k_run_tiles<uint32_t, 2>, run_tile_smem(0, 2));
