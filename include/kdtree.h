@@ -124,7 +124,8 @@ kd_status kd_create(kd_ctx **out, const kd_config *cfg);
  * KD_EDEVICE, KD_ETIMEOUT.  Synchronises the stream three times: to read
  * the key-byte histograms (constant digits are skipped), the run lengths of
  * array 0 after its sort by x_0 (k >= 2: long or costly runs take the
- * whole-key sort), and m.  Clouds of at most 196608 tuples: once, to read m.
+ * whole-key sort), and m.  Clouds of at most 196608 tuples: once, to read m
+ * (those of few values per coordinate: then as the larger ones).
  */
 kd_status kd_presort(kd_ctx *ctx, const kd_cloud *cloud, kd_handle *out);
 
